@@ -263,20 +263,18 @@ mt_status mt_batch_prepare(const float *d_arena, const mt_grid *h_grids, uint32_
 
 /* Launch configurations (bits of cfg; 0 is the default). Every
  * configuration gives the same results; they differ only in speed:
- *   MT_CFG_SMALL_TILES  16x16x8 tiles of 256 threads instead of 16x16x16 tiles
- *                       of 512 threads (batches only: small fields leave
- *                       most of a large tile empty)
- *   MT_CFG_FOUR_ROUNDS  4 level buckets per tile instead of 8: the in-tile
- *                       edges are merged, and their vertices repaired, in 4
- *                       rounds by level instead of 8 (Algorithm 1 merges the
+ *   MT_CFG_SMALL_TILES  16x16x8 tiles instead of 16x16x16 tiles, 256 threads
+ *                       each (batches only: small fields leave most of a
+ *                       large tile empty)
+ *   MT_CFG_FOUR_ROUNDS  accepted, chooses nothing: the tile kernel merges the
+ *                       in-tile edges in one round (Algorithm 1 merges the
  *                       edges in any order)
  *   MT_CFG_REPAIR_256   the repair kernel (Algorithm 5) in CTAs of 256
  *                       threads instead of 512
- *   MT_CFG_LARGE_TILES  32x16x16 tiles of 1024 threads, two CTAs per SM,
- *                       instead of 16x16x16 tiles of 512 threads, four per SM
- *                       (single fields only: fewer edges between tiles
- *                       against fewer warps per SM to issue while a tile
- *                       waits at a round barrier)
+ *   MT_CFG_LARGE_TILES  32x16x16 tiles of 512 threads instead of 16x16x16
+ *                       tiles of 256 (single fields only: fewer edges
+ *                       between tiles against fewer warps per SM to issue
+ *                       while a tile waits at a barrier)
  * A batch takes the configurations 0 .. MT_CFG_COUNT - 1; a single field the
  * even ones of 0 .. 15 (MT_CFG_SINGLE_MASK). */
 #define MT_CFG_SMALL_TILES 1u

@@ -81,10 +81,10 @@ __all__ = [
 MT_OK = 0
 MT_SUPERLEVEL = 1  # flag of the _ex calls: the tree of -f (superlevel sets, the split tree)
 # launch configurations (bits; every one gives the same results)
-MT_CFG_SMALL_TILES = 1  # 16x16x8 tiles of 256 threads (batches only)
-MT_CFG_FOUR_ROUNDS = 2  # 4 level buckets (merge/repair rounds) per tile instead of 8
+MT_CFG_SMALL_TILES = 1  # 16x16x8 tiles (batches only)
+MT_CFG_FOUR_ROUNDS = 2  # accepted, chooses nothing (the tile kernel has no rounds)
 MT_CFG_REPAIR_256 = 4   # repair CTAs of 256 threads instead of 512
-MT_CFG_LARGE_TILES = 8  # 32x16x16 tiles of 1024 threads (single fields only)
+MT_CFG_LARGE_TILES = 8  # 32x16x16 tiles (single fields only)
 MT_CFG_COUNT = 8        # batch configurations 0 .. 7
 MT_CFG_SINGLE_MASK = MT_CFG_FOUR_ROUNDS | MT_CFG_REPAIR_256 | MT_CFG_LARGE_TILES
 STATUS_NAMES = {0: "MT_OK", -1: "MT_ERR_INVALID", -2: "MT_ERR_TOO_LARGE", -3: "MT_ERR_NONFINITE",

@@ -30,63 +30,76 @@ namespace mt {
 // 32-bit keys whose unsigned order is the float order (-0 and +0 share one
 // key), so a vertex comparison is an integer comparison of (key, id).
 //
-// Seed. T[l] = (l, lln(l)), lln(l) the first vertex of l's closed in-tile
-// neighbourhood (a normalised triplet of the graph of steepest-descent
-// edges); pointer jumping then moves every inner vertex straight to the
-// minimum its descent reaches. An edge whose ends reach the same minimum
-// needs no merge.
+// Which edges. Let S be the upper end of an edge (S, a). If another lower
+// neighbour c of S lies on a common grid square with a, and the square's
+// fourth corner q is below S too, then a - q - c joins a and c below S: once
+// one of the edges (S, a), (S, c) is merged the other adds nothing, at any
+// level. (The edges of that path have levels below S; by induction over the
+// levels they may have been left out for the same reason, and their ends are
+// still joined at their own levels.) So among the lower neighbours of S only
+// the components of "joined through a square below S" matter. One lower
+// neighbour seeds S (Algorithm 1 starts at T[S] = (S, lower neighbour): a
+// valid triplet of the graph of descent edges), every other component gives
+// one edge. On a lognormal field 0.23 edges per vertex are left of the 1.55
+// whose ends descend to different minima, for about 0.11 minima; all of them
+// are merged straight away, in no order, by short climbs (4 links each).
 //
-// Level buckets and shortcuts. The remaining edges are merged in NB rounds
-// by the level of their upper end S (NB buckets of about equal size, cut from
-// a histogram of the tile's keys); within a round the order is free, as
-// Algorithm 1 allows. SC[m] is a shortcut for minimum m: the vertex m's climb
-// reaches through the links whose saddle lies in buckets before the current
-// one, i.e. the deepest vertex of m's component below the round. Those links
-// do not change during a round (a merge at level S only displaces links above
-// S), so a shortcut is computed on first use in a round and stored with the
-// round number in its top bits. An edge (S, a, c) starts its climbs at SC[a]
-// and SC[c] (both joined to a, c below S), and when they coincide the ends are
-// already connected below S and the edge is settled by two shared-memory
-// loads, as about nine edges in ten are on these fields. The others are
-// collected and merged together once the bucket's scan is done, so that the
-// lanes of a warp run their merges side by side instead of one after another.
-// They are collected in a shared-memory hash keyed by the pair of shortcuts
-// that keeps, per pair, only the edge with the earliest upper end: once that
-// one is merged, the two components are joined below the level of every
-// other edge of the pair, which Merge would then find connected and skip. On
-// these fields about two collected edges in five repeat a pair.
+// The lower-than relations are computed bit-sliced. A thread owns a column of
+// TZ vertices along z and slides a window of keys up it: nine comparisons
+// per vertex (with the neighbours at +x, +y, +z and six of the twelve square
+// corners) give nine words of one bit per vertex. The other nine relations
+// are the complements of the neighbour columns' bits, exchanged through
+// shared memory, and the components are then flooded for all vertices of the
+// column at once, one LOP3 per word and square.
 //
-// Repair. Right after round b no later merge can change a component below
-// the levels of bucket b, so every inner vertex l of bucket b gets its final
-// tile triplet (l, deepest vertex below l) by a short climb from its
-// minimum's shortcut (Algorithms 4 and 5). Branch minima are repaired at the
-// end.
+// Repair. After the merges the branch minima are repaired (Algorithm 5), then
+// every inner vertex l climbs from its descent minimum to its final tile
+// triplet (l, deepest vertex below l), 1.6 links on average, which goes
+// straight to global memory.
+//
+// What it costs. The kernel is bound by instruction issue (75 % of the issue
+// slots, HBM 7 % busy): 12.5 warp instructions per vertex. On the 1024^3
+// lognormal field it takes 14.5 ms: loads 1.2, relations 0.7, components 1.0,
+// edge list 0.7, descent 1.1, merges 3.5, minima 0.6, inner vertices 3.8,
+// faces 1.8. The earlier design, which kept every edge whose ends descend to
+// different minima and settled most of them by comparing cached climbs in 8
+// rounds over level buckets, took 31.5 ms (29 warp instructions per vertex).
+// The climbs and merges are loops whose lanes stay together by votes: with
+// ordinary divergent loops the same algorithm took 24.0 ms, since a warp
+// whose lanes left a loop one by one ran what follows it once per group.
 //
 // What leaves the kernel is, for every vertex, its triplet in the subgraph
 // induced by its tile: a valid normalised triplet tree of the full grid minus
 // the edges between tiles, which k_cross merges next.
 constexpr int log2i(int x) { return x <= 1 ? 0 : 1 + log2i(x / 2); }
 
-template <int LX, int LY, int LZ, int NT = 512>
+template <int LX, int LY, int LZ>
 struct Tile {
     static constexpr int TX = 1 << LX, TY = 1 << LY, TZ = 1 << LZ;
     static constexpr int TV = TX * TY * TZ;
-    static_assert(TV <= 65536, "local ids are 16-bit");
+    static constexpr int NT = TX * TY;  // a thread per column
+    static_assert(TZ <= 16, "a column's bits fit half a word");
+    static_assert(LX + LY + LZ + 3 <= 16, "an edge entry packs a local id and a direction into 16 bits");
     static_assert(TX % 4 == 0, "rows are loaded as float4");
-    static constexpr int kBins = NT;     // key histogram, one bin per thread
-    static constexpr int kQueue = 2048 * TV / 8192 > NT ? 2048 * TV / 8192 : NT;  // 32-bit words of the edge hash
-    static constexpr int kHashLog = log2i(kQueue / 3);                            // slots: 32-bit pair + 64-bit level
-    static constexpr int kHash = 1 << kHashLog;
-    static_assert(kHash * 12 <= kQueue * 4, "hash fits its buffer");
-    // shared memory: keys + triplets (4 B each), shortcuts + bucket-sorted
-    // vertex list (2 B each), edge hash (aliased by the key histogram)
-    static constexpr size_t kSmem = (size_t)TV * (4 + 4 + 2 + 2) + (size_t)kQueue * 4;
-    static_assert(kQueue >= kBins, "the histogram lives in the hash buffer");
+    static constexpr int kList = NT * 8 / kTileListShrink;  // edges listed (the others are merged in place)
+    // shared memory: a link word (8 B) per x-adjacent pair of vertices, of
+    // which at most one is a minimum; keys (4 B) and seeds (2 B) per vertex;
+    // then 16 B per thread that hold in turn the exchanged words, the edge
+    // list and the list of face edges
+    static constexpr size_t kSmem = (size_t)TV * (4 + 4 + 2) + (size_t)NT * 16;
+    static constexpr int kCTAs = (int)(227 * 1024 / (kSmem + 1024)) < 1536 / NT ? (int)(227 * 1024 / (kSmem + 1024)) : 1536 / NT;
+    // face record of a tile (u32 words): per group of 32 edges of the faces
+    // +x, +y, +z the number of kept ones (a byte each), then the tops in this
+    // tile of the kept edges' ends on the + faces and on the - faces, then the
+    // levels S of the + faces' edges; 16 entries per group
+    static constexpr int G = (TY * TZ + TX * TZ + TX * TY) / 32;
+    static constexpr int kFaceHead = (G + 15) / 16 * 4, kFaceSide = 16 * G;
+    static constexpr int kFaceWords = kFaceHead + 3 * kFaceSide;
+    static_assert(TY * TZ <= NT && TX * TZ <= NT, "one edge of a face per thread");
+    static constexpr int FX = TY * TZ, FY = TX * TZ, FZ = TX * TY, FH = FX + FY + FZ;  // edges of the + faces
+    static_assert(2 * FH * 8 <= TV * 4, "the faces' levels fit the key array");
+    static_assert(2 * kFaceSide * 4 <= NT * 16, "the face edge list fits its buffer");
 };
-
-__device__ __forceinline__ uint32_t sm_pack(uint32_t s, uint32_t v) { return (s << 16) | v; }
-__device__ __forceinline__ uint32_t sm_s(uint32_t w) { return w >> 16; }
-__device__ __forceinline__ uint32_t sm_v(uint32_t w) { return w & 0xFFFFu; }
 
 // Order-preserving 32-bit key of a float (+0 and -0 map to the same key).
 __device__ __forceinline__ uint32_t order_key(float x)
@@ -100,91 +113,80 @@ __device__ __forceinline__ bool kbefore(uint32_t ka, uint32_t a, uint32_t kb, ui
     return ka < kb || (ka == kb && a < b);
 }
 
-// Climb (Algorithm 3 / 4) in the tile's tree from x through links whose
-// saddle is at or below (kS, S); a root stops it. Chains lead to ever earlier
-// vertices, so a walk longer than the tile means a corrupted tree (ok=false).
-// The next vertex's triplet is read together with the saddle's key, before
-// the test that decides whether it is needed (indices are masked to the
-// tile, so a read that turns out unneeded stays in bounds).
-template <int TV>
-__device__ __forceinline__ uint32_t sm_climb(const uint32_t *T, const uint32_t *K, uint32_t x, uint32_t S,
-                                             uint32_t kS, uint32_t &w, bool &ok)
+// The key of no vertex: above every finite key. Vertices outside the grid
+// have it, and so has the link word of a root.
+constexpr uint32_t kNoKey = 0xFFFFFFFFu;
+
+// A minimum's link in the tile's tree as one 64-bit word: the saddle's key,
+// its local id (16 bits), the target's local id (16 bits). Links compare as
+// integers by level: a walk to level (kS, S) follows word w iff
+// w <= level_word(kS, S), and a root's word (kNoKey) stops every walk.
+__device__ __forceinline__ uint64_t level_word(uint32_t kS, uint32_t S)
 {
-    const volatile uint32_t *vT = T;
-    uint32_t wx = vT[x];
-    for (uint32_t h = 0; h < (uint32_t)TV; h++) {
-        const uint32_t s = sm_s(wx), nx = sm_v(wx);
-        const uint32_t ks = K[s & (TV - 1)];
-        const uint32_t wn = vT[nx & (TV - 1)];
-        if (wx == sm_pack(x, x) || (s != S && !kbefore(ks, s, kS, S))) {
-            w = wx;
-            return x;
-        }
-        x = nx;
-        wx = wn;
+    return (uint64_t)kS << 32 | S << 16 | 0xFFFFu;
+}
+__device__ __forceinline__ uint32_t link_s(uint64_t w) { return (uint32_t)w >> 16; }
+__device__ __forceinline__ uint32_t link_v(uint64_t w) { return (uint32_t)w & 0xFFFFu; }
+
+// Merge (Algorithm 3) on the tile's tree, lock-free with 64-bit CAS on the
+// link words L (of vertex x at L[x / 2]). One try: u and v have climbed to
+// their deepest vertices below the level `lim` and differ; the later one (its
+// word wv) is linked under the earlier, and the link it held is re-inserted
+// by going on from there (a displaced root carries none; after a failed CAS
+// both climb again). Returns true when the edge is done.
+__device__ __forceinline__ bool sm_link(uint64_t *L, const uint32_t *K, uint64_t &lim, uint32_t &u, uint32_t &v,
+                                        uint64_t wu, uint64_t wv)
+{
+    const bool sw = kbefore(K[v], v, K[u], u);
+    const uint32_t lo = sw ? v : u;
+    v = sw ? u : v, u = lo;
+    wv = sw ? wu : wv;
+    const uint64_t want = (lim & ~(uint64_t)0xFFFFu) | u;
+    if (atomicCAS(reinterpret_cast<unsigned long long *>(L + (v >> 1)), (unsigned long long)wv,
+                  (unsigned long long)want) == wv) {
+        if ((uint32_t)(wv >> 32) == kNoKey) return true;
+        lim = wv | 0xFFFFu;
+        v = link_v(wv);
     }
-    ok = false;
-    w = wx;
+    return u == v;
+}
+
+// The minimum that vertex x descends to along the seeds D.
+template <int TV>
+__device__ __forceinline__ uint32_t sm_descend(const uint16_t *D, uint32_t x)
+{
+    const volatile uint16_t *vD = D;
+    for (uint32_t h = 0; h < (uint32_t)TV; h++) {
+        const uint32_t y = vD[x];
+        if (y == x) break;
+        x = y;
+    }
     return x;
 }
 
-// Both climbs of a merge side by side, so that their reads overlap.
+// A whole merge of the edge (S, w), out of line for the rare edges that find
+// the list full.
 template <int TV>
-__device__ __forceinline__ void sm_climb2(const uint32_t *T, const uint32_t *K, uint32_t &u, uint32_t &v,
-                                          uint32_t S, uint32_t kS, uint32_t &wu, uint32_t &wv, bool &ok)
+__device__ __noinline__ bool sm_merge_rare(uint64_t *L, const uint32_t *K, const uint16_t *D, uint32_t S, uint32_t w)
 {
-    const volatile uint32_t *vT = T;
-    wu = vT[u], wv = vT[v];
-    bool du = false, dv = false;
-    for (uint32_t h = 0; h < 2u * TV; h++) {
-        const uint32_t su = sm_s(wu), nu = sm_v(wu), sv = sm_s(wv), nv = sm_v(wv);
-        const uint32_t ku = K[su & (TV - 1)], kv = K[sv & (TV - 1)];
-        const uint32_t wnu = vT[nu & (TV - 1)], wnv = vT[nv & (TV - 1)];
-        du = du || wu == sm_pack(u, u) || (su != S && !kbefore(ku, su, kS, S));
-        dv = dv || wv == sm_pack(v, v) || (sv != S && !kbefore(kv, sv, kS, S));
-        if (du && dv) return;
-        if (!du) u = nu, wu = wnu;
-        if (!dv) v = nv, wv = wnv;
-    }
-    ok = false;
-}
-
-// Merge (Algorithm 3) on the tile's shared-memory tree, lock-free with 32-bit
-// CAS (Algorithm 2): climb a and c to their deepest vertices below S; if they
-// differ, link the later one under the earlier at S and re-insert the link
-// it held before (a displaced root carries none); on a failed CAS climb again.
-template <int TV>
-__device__ __forceinline__ void sm_merge(uint32_t *T, const uint32_t *K, uint32_t S, uint32_t kS, uint32_t a,
-                                         uint32_t c, bool &ok)
-{
-    uint32_t u = a, v = c;
+    uint32_t u = sm_descend<TV>(D, S), v = sm_descend<TV>(D, w);
+    const volatile uint64_t *vL = L;
+    uint64_t lim = level_word(K[S], S);
     for (uint32_t it = 0; it < kMergeStepLimit; it++) {
-        uint32_t Tu, Tv;
-        sm_climb2<TV>(T, K, u, v, S, kS, Tu, Tv, ok);
-        if (!ok || u == v) return;
-        if (kbefore(K[v], v, K[u], u)) {
-            const uint32_t x = u;
-            u = v;
-            v = x;
-            const uint32_t y = Tu;
-            Tu = Tv;
-            Tv = y;
-        }
-        if (atomicCAS(T + v, Tv, sm_pack(S, u)) == Tv) {
-            if (Tv == sm_pack(v, v)) return;
-            S = sm_s(Tv);
-            kS = K[S];
-            v = sm_v(Tv);
-        }
+        const uint64_t wu = vL[u >> 1], wv = vL[v >> 1];
+        const bool mu = wu <= lim, mv = wv <= lim;
+        if (mu) u = link_v(wu);
+        if (mv) v = link_v(wv);
+        if (u == v || (!mu && !mv && sm_link(L, K, lim, u, v, wu, wv))) return true;
     }
-    ok = false;
+    return false;
 }
 
 // WIDE: the triplets leave the tile as 128-bit words of two 64-bit ids
 // (W[2u] = s, W[2u + 1] = v) for grids of 2^32 vertices and more; the work
-// inside the tile, on 16-bit local ids, is the same, and no face buffer is
+// inside the tile, on 16-bit local ids, is the same, and no face record is
 // written (the wide path merges the edges between tiles from their ends).
-template <int LX, int LY, int LZ, int NT, int NB, bool FULL, bool WIDE = false>
+template <int LX, int LY, int LZ, bool WIDE = false>
 __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, uint32_t *status)
 {
     using Id = typename std::conditional<WIDE, uint64_t, uint32_t>::type;
@@ -192,418 +194,410 @@ __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, ui
     const float sg = fd.sg;
     uint64_t *__restrict__ W = fd.W;
     const uint32_t nx = fd.nx, ny = fd.ny, nz = fd.nz, ntx = fd.ntx, nty = fd.nty;
-    const bool vec = (nx % 4 == 0) && ((uintptr_t)f % 16 == 0) && ((uintptr_t)W % 16 == 0);
-    using TS = Tile<LX, LY, LZ, NT>;
-    constexpr int TX = TS::TX, TY = TS::TY, TZ = TS::TZ, TV = TS::TV, BINS = TS::kBins, HS = TS::kHash, HLOG = TS::kHashLog;
-    constexpr uint32_t IDB = LX + LY + LZ;  // bits of a local id
-    constexpr uint32_t IDM = (1u << IDB) - 1u;
-    static_assert(NT >= BINS, "one histogram bin per thread");
-    static_assert(IDB + 3 <= 16 && NB <= 8, "a shortcut packs a local id and a round number into 16 bits");
-    extern __shared__ __align__(16) uint32_t smem[];
-    uint32_t *K = smem;                                           // order keys
-    uint32_t *T = smem + TV;                                      // triplets (s << 16) | v
-    uint16_t *SC = reinterpret_cast<uint16_t *>(smem + 2 * TV);   // shortcuts (round << IDB) | vertex
-    uint16_t *vlist = SC + TV;                                    // vertices sorted by bucket
-    // edges to merge in the current round, one per pair of shortcuts:
-    // hkey = (lo << IDB) | hi, hlev = (key << 32) | S of the earliest upper end
-    unsigned long long *hlev = reinterpret_cast<unsigned long long *>(vlist + TV);
-    uint32_t *hkey = reinterpret_cast<uint32_t *>(hlev + HS);
-    uint32_t *hist = reinterpret_cast<uint32_t *>(hlev);          // key histogram (before the rounds)
-    __shared__ uint8_t s_bmap[BINS];                              // histogram bin -> bucket
-    __shared__ uint32_t s_nvalid, s_warp[NT / 32], s_wmin[NT / 32], s_wmax[NT / 32];
-    __shared__ uint32_t s_boff[NB + 2], s_bcur[NB + 1], s_thr[NB];
+    using TS = Tile<LX, LY, LZ>;
+    constexpr uint32_t TX = TS::TX, TY = TS::TY, TZ = TS::TZ, TV = TS::TV, NT = TS::NT, LV = LX + LY + LZ;
+    extern __shared__ __align__(16) uint64_t tile_smem[];
+    uint64_t *L = tile_smem;                                  // link words of the minima
+    uint32_t *K = reinterpret_cast<uint32_t *>(L + TV / 2);   // order keys
+    uint16_t *D = reinterpret_cast<uint16_t *>(K + TV);       // seeds, then descent minima
+    uint32_t *X = reinterpret_cast<uint32_t *>(D + TV);       // 16 B per thread, see Tile
+    uint16_t *list = reinterpret_cast<uint16_t *>(X);
+    volatile uint64_t *vL = L;
+    volatile uint16_t *vD = D;
+    __shared__ uint32_t s_nlist, s_nface;
 
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t lane = threadIdx.x & 31;
     const uint32_t tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
     const uint32_t x0 = tx * TX, y0 = ty * TY, z0 = tz * TZ;
-    // a FULL tile lies inside the grid: its extents are the tile's
-    const uint32_t wx = FULL ? (uint32_t)TX : min((uint32_t)TX, nx - x0),
-                   wy = FULL ? (uint32_t)TY : min((uint32_t)TY, ny - y0),
-                   wz = FULL ? (uint32_t)TZ : min((uint32_t)TZ, nz - z0);
+    const uint32_t wx = min(TX, nx - x0), wy = min(TY, ny - y0), wz = min(TZ, nz - z0);
     const Id nxy = (Id)nx * ny;  // n < 2^32 unless WIDE, so every id fits an Id
     const Id base = (Id)z0 * nxy + (Id)y0 * nx + x0;
     auto lxo = [](uint32_t l) { return l & (TX - 1); };
     auto lyo = [](uint32_t l) { return (l >> LX) & (TY - 1); };
     auto lzo = [](uint32_t l) { return l >> (LX + LY); };
-    auto valid = [&](uint32_t l) { return FULL || (lxo(l) < wx && lyo(l) < wy && lzo(l) < wz); };
     auto gid = [&](uint32_t l) -> Id { return base + (Id)lzo(l) * nxy + (Id)lyo(l) * nx + lxo(l); };
-    // (the barrier after the loads orders these writes before their uses)
-    if (threadIdx.x == 0) s_nvalid = wx * wy * wz;
-    if (threadIdx.x <= NB) s_bcur[threadIdx.x] = 0;
-    for (uint32_t i = threadIdx.x; i < (uint32_t)BINS; i += NT) hist[i] = 0;
 
-    // 1. load the tile's values (rows of TX floats) as order keys
+    // 1. load the tile's values (rows of TX floats) as order keys; vertices
+    //    outside the grid get kNoKey
     bool bad = false;
-    uint32_t kmin = 0xFFFFFFFFu, kmax = 0;
-    if (vec) {
-        for (uint32_t q = threadIdx.x; q < TV / 4; q += NT) {
-            const uint32_t l = 4 * q;
-            if (valid(l)) {
+    if (nx % 4 == 0 && (uintptr_t)f % 16 == 0) {
+#pragma unroll
+        for (uint32_t i = 0; i < TV / 4 / NT; i++) {
+            const uint32_t l = 4 * (i * NT + threadIdx.x);
+            uint4 k = make_uint4(kNoKey, kNoKey, kNoKey, kNoKey);
+            if (lxo(l) < wx && lyo(l) < wy && lzo(l) < wz) {
                 float4 v = __ldg(reinterpret_cast<const float4 *>(f + gid(l)));
                 v.x *= sg, v.y *= sg, v.z *= sg, v.w *= sg;
                 bad |= !isfinite(v.x) | !isfinite(v.y) | !isfinite(v.z) | !isfinite(v.w);
-                const uint4 k = make_uint4(order_key(v.x), order_key(v.y), order_key(v.z), order_key(v.w));
-                kmin = min(kmin, min(min(k.x, k.y), min(k.z, k.w)));
-                kmax = max(kmax, max(max(k.x, k.y), max(k.z, k.w)));
-                *reinterpret_cast<uint4 *>(K + l) = k;
+                k = make_uint4(order_key(v.x), order_key(v.y), order_key(v.z), order_key(v.w));
             }
+            *reinterpret_cast<uint4 *>(K + l) = k;
         }
     } else {
-        for (uint32_t l = threadIdx.x; l < TV; l += NT) {
-            if (valid(l)) {
+#pragma unroll 8
+        for (uint32_t i = 0; i < TV / NT; i++) {
+            const uint32_t l = i * NT + threadIdx.x;
+            uint32_t k = kNoKey;
+            if (lxo(l) < wx && lyo(l) < wy && lzo(l) < wz) {
                 const float v = sg * __ldg(f + gid(l));
                 bad |= !isfinite(v);
-                const uint32_t k = order_key(v);
-                kmin = min(kmin, k);
-                kmax = max(kmax, k);
-                K[l] = k;
+                k = order_key(v);
             }
+            K[l] = k;
         }
     }
+    if (threadIdx.x == 0) s_nlist = 0, s_nface = 0;
     if (bad) raise_status(status, ST_NONFINITE);
-    for (int o = 16; o > 0; o >>= 1) {
-        kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-        kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-    }
-    if (lane == 0) s_wmin[warp] = kmin, s_wmax[warp] = kmax;
-    __syncthreads();
-    kmin = lane < NT / 32 ? s_wmin[lane] : 0xFFFFFFFFu;
-    kmax = lane < NT / 32 ? s_wmax[lane] : 0u;
-    for (int o = 16; o > 0; o >>= 1) {
-        kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-        kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-    }
-
-    // Spare bits of a triplet (ids take IDB of each 16-bit half) carry a
-    // mask of neighbour directions d (-x, -y, -z, +x, +y, +z): from the seed
-    // to step 4 the lower neighbours of the vertex, from step 4 on (inner
-    // vertices only) its cross mask: the lower neighbours that descend to
-    // another minimum. Only those edges can join two components; the scan of
-    // the vertex's level bucket reads them from here. The bucket repair of
-    // the vertex rewrites its triplet and so clears the bits; minima never
-    // carry any (a minimum has no lower neighbour).
-    auto tid_s = [](uint32_t w) { return (w >> 16) & IDM; };
-    auto tid_v = [](uint32_t w) { return w & IDM; };
-    auto xmask = [](uint32_t w) { return ((w >> IDB) & 7u) | (((w >> (16 + IDB)) & 7u) << 3); };
-    auto with_mask = [](uint32_t w, uint32_t m) { return w | ((m & 7u) << IDB) | ((m >> 3) << (16 + IDB)); };
-    constexpr uint32_t SPARE = ~(IDM | (IDM << 16));
-    auto nbr = [](uint32_t l, uint32_t d) -> uint32_t {
-        const uint32_t a = d < 3 ? d : d - 3;
-        const uint32_t step = 1u << (a == 0 ? 0 : a == 1 ? LX : LX + LY);
-        return d < 3 ? l - step : l + step;
-    };
-
-    // 2. seed: T[l] = (l, first vertex of the closed in-tile neighbourhood)
-    //    with l's lower neighbours in the spare bits; key histogram for the
-    //    level buckets
-    const uint32_t kmin_t = kmin, kmax_t = kmax;
-    const float bscale = (float)BINS / ((float)(kmax_t - kmin_t) + 1.0f);
-    auto bin_of = [&](uint32_t k) { return min((uint32_t)BINS - 1, (uint32_t)((float)(k - kmin_t) * bscale)); };
-    for (uint32_t l = threadIdx.x; l < TV; l += NT) {
-        if (!valid(l)) continue;
-        const uint32_t lx = lxo(l), ly = lyo(l), lz = lzo(l);
-        const uint32_t kl = K[l];
-        uint32_t b = l, kb = kl;
-        atomicAdd(&hist[bin_of(kb)], 1u);
-        // candidates in ascending local index order: an earlier id wins ties,
-        // so an earlier candidate replaces b only if strictly lower; a
-        // neighbour is lower than l if its key is lower, or equal and its id
-        // earlier (the -x, -y, -z neighbours)
-        const uint32_t kmz = lz > 0 ? K[l - TX * TY] : 0xFFFFFFFFu, kmy = ly > 0 ? K[l - TX] : 0xFFFFFFFFu,
-                       kmx = lx > 0 ? K[l - 1] : 0xFFFFFFFFu;
-        const uint32_t kpx = lx + 1 < wx ? K[l + 1] : 0u, kpy = ly + 1 < wy ? K[l + TX] : 0u,
-                       kpz = lz + 1 < wz ? K[l + TX * TY] : 0u;
-        if (lz > 0 && kmz <= kb) b = l - TX * TY, kb = kmz;
-        if (ly > 0 && kmy <= kb && (kmy < kb || l - TX < b)) b = l - TX, kb = kmy;
-        if (lx > 0 && kmx <= kb && (kmx < kb || l - 1 < b)) b = l - 1, kb = kmx;
-        if (lx + 1 < wx && kpx < kb) b = l + 1, kb = kpx;
-        if (ly + 1 < wy && kpy < kb) b = l + TX, kb = kpy;
-        if (lz + 1 < wz && kpz < kb) b = l + TX * TY, kb = kpz;
-        const uint32_t lm = (uint32_t)(lx > 0 && kmx <= kl) | (uint32_t)(ly > 0 && kmy <= kl) << 1 |
-                            (uint32_t)(lz > 0 && kmz <= kl) << 2 | (uint32_t)(lx + 1 < wx && kpx < kl) << 3 |
-                            (uint32_t)(ly + 1 < wy && kpy < kl) << 4 | (uint32_t)(lz + 1 < wz && kpz < kl) << 5;
-        T[l] = with_mask(sm_pack(l, b), lm);
-    }
     __syncthreads();
 
-    // 3. pointer jumping along the descent links (concurrent jumps only
-    //    shorten chains, so racing readers stay correct); shortcuts start at
-    //    the minima themselves. Bin -> bucket map from the histogram's
-    //    prefix sums (monotone in the key).
+    // 2. lower-than words of the thread's column: bit z of p<d> says that the
+    //    neighbour at d is before vertex (x, y, z). In p.. the neighbour has
+    //    the later id, so it is before only with a strictly lower key; in
+    //    q.. (one plane down) it has the earlier id. Reads past the tile's
+    //    faces give some other word of shared memory; those bits are masked
+    //    below.
+    const uint32_t col = threadIdx.x, cx = lxo(col), cy = lyo(col);
+    uint32_t px = 0, py = 0, pz = 0, pxy = 0, pmxy = 0, pxz = 0, pyz = 0, qxz = 0, qyz = 0;
     {
-        volatile uint32_t *vT = T;
-        for (uint32_t l = threadIdx.x; l < TV; l += NT) {
-            if (!valid(l)) continue;
-            const uint32_t w = vT[l];
-            if (tid_v(w) == l) {
-                SC[l] = (uint16_t)l;
-                continue;
+        uint32_t kc = K[col], kx = K[col + 1], ky = K[col + TX], kxd = 0, kyd = 0;
+#pragma unroll
+        for (uint32_t z = 0; z < TZ; z++) {
+            const uint32_t l = col + z * NT;
+            const uint32_t kcu = z + 1 < TZ ? K[l + NT] : kNoKey, kxu = z + 1 < TZ ? K[l + NT + 1] : kNoKey,
+                           kyu = z + 1 < TZ ? K[l + NT + TX] : kNoKey;
+            px |= (uint32_t)(kx < kc) << z;
+            py |= (uint32_t)(ky < kc) << z;
+            pz |= (uint32_t)(kcu < kc) << z;
+            pxy |= (uint32_t)(K[l + TX + 1] < kc) << z;
+            pmxy |= (uint32_t)(K[l + TX - 1] < kc) << z;
+            pxz |= (uint32_t)(kxu < kc) << z;
+            pyz |= (uint32_t)(kyu < kc) << z;
+            if (z > 0) {
+                qxz |= (uint32_t)(kxd <= kc) << z;
+                qyz |= (uint32_t)(kyd <= kc) << z;
             }
-            uint32_t x = tid_v(w);
-            for (uint32_t h = 0; h < (uint32_t)TV; h++) {
-                const uint32_t wx_ = vT[x];
-                if (tid_v(wx_) == x) break;
-                x = tid_v(wx_);
-            }
-            if (x != tid_v(w)) vT[l] = sm_pack(l, x) | (w & SPARE);
+            kxd = kx, kyd = ky;
+            kc = kcu, kx = kxu, ky = kyu;
         }
-        const uint32_t c = threadIdx.x < (uint32_t)BINS ? hist[threadIdx.x] : 0u;
-        uint32_t incl = c;
+    }
+    X[col] = px | pxz << 16;
+    X[NT + col] = qxz | pxy << 16;
+    X[2 * NT + col] = py | pyz << 16;
+    X[3 * NT + col] = qyz | pmxy << 16;
+    __syncthreads();
+
+    // 3. the lower neighbours of every vertex, their components, the seed
+    //    and the edges left to merge
+    const bool inx = cx < wx && cy < wy;
+    const uint32_t zm = inx ? (1u << wz) - 1u : 0u;
+    uint32_t minima;       // bit z: vertex z of the column is a minimum of the tile
+    uint32_t ex, ey, ez;   // edges to merge: bits z (towards -) and 16 + z (towards +)
+    {
+        const uint32_t cm = (col - 1) & (NT - 1);
+        const uint32_t a = X[cm], b = X[NT + cm];                          // column (x - 1, y)
+        const uint32_t c = X[2 * NT + ((col - TX) & (NT - 1))], d = X[3 * NT + ((col - TX) & (NT - 1))];  // (x, y - 1)
+        const uint32_t e = X[NT + ((col - TX - 1) & (NT - 1))];            // (x - 1, y - 1)
+        const uint32_t g = X[3 * NT + ((col - TX + 1) & (NT - 1))];        // (x + 1, y - 1)
+        // lower neighbours (a relation to a neighbour with an earlier id is
+        // the complement of that neighbour's relation to this vertex)
+        const uint32_t lx0 = cx > 0 ? ~a & zm : 0u, lx1 = cx + 1 < wx ? px & zm : 0u;
+        const uint32_t ly0 = cy > 0 ? ~c & zm : 0u, ly1 = cy + 1 < wy ? py & zm : 0u;
+        const uint32_t lz0 = (~pz << 1) & zm, lz1 = pz & zm;
+        minima = zm & ~(lx0 | lx1 | ly0 | ly1 | lz0 | lz1);
+        // squares: both neighbours and the corner between them are lower
+        const uint32_t x0y0 = lx0 & ly0 & ~(e >> 16), x1y0 = lx1 & ly0 & ~(g >> 16);
+        const uint32_t x0y1 = lx0 & ly1 & pmxy, x1y1 = lx1 & ly1 & pxy;
+        const uint32_t x0z0 = lx0 & lz0 & (~(a >> 16) << 1), x1z0 = lx1 & lz0 & qxz;
+        const uint32_t x0z1 = lx0 & lz1 & (~(b & 0xFFFFu) >> 1), x1z1 = lx1 & lz1 & pxz;
+        const uint32_t y0z0 = ly0 & lz0 & (~(c >> 16) << 1), y1z0 = ly1 & lz0 & qyz;
+        const uint32_t y0z1 = ly0 & lz1 & (~(d & 0xFFFFu) >> 1), y1z1 = ly1 & lz1 & pyz;
+        // the seed: the first lower neighbour
+        const uint32_t sx0 = lx0, sx1 = lx1 & ~lx0, m2 = lx0 | lx1;
+        const uint32_t sy0 = ly0 & ~m2, m3 = m2 | ly0, sy1 = ly1 & ~m3, m4 = m3 | ly1;
+        const uint32_t sz0 = lz0 & ~m4, sz1 = lz1 & ~(m4 | lz0);
+        // flood its component (three passes reach all but a few; a
+        // component cut in two only costs an edge that adds nothing)
+        uint32_t rx0 = sx0, rx1 = sx1, ry0 = sy0, ry1 = sy1, rz0 = sz0, rz1 = sz1;
+#pragma unroll
+        for (int it = 0; it < 3; it++) {
+            ry0 |= (rx0 & x0y0) | (rx1 & x1y0) | (rz0 & y0z0) | (rz1 & y0z1);
+            ry1 |= (rx0 & x0y1) | (rx1 & x1y1) | (rz0 & y1z0) | (rz1 & y1z1);
+            rz0 |= (rx0 & x0z0) | (rx1 & x1z0) | (ry0 & y0z0) | (ry1 & y1z0);
+            rz1 |= (rx0 & x0z1) | (rx1 & x1z1) | (ry0 & y0z1) | (ry1 & y1z1);
+            rx0 |= (ry0 & x0y0) | (ry1 & x0y1) | (rz0 & x0z0) | (rz1 & x0z1);
+            rx1 |= (ry0 & x1y0) | (ry1 & x1y1) | (rz0 & x1z0) | (rz1 & x1z1);
+        }
+        // of the other components, the first neighbour (a neighbour joined
+        // to one earlier in the order x0 x1 y0 y1 z0 z1 is left out)
+        ex = (lx0 & ~rx0) | (lx1 & ~rx1) << 16;
+        ey = (ly0 & ~(ry0 | x0y0 | x1y0)) | (ly1 & ~(ry1 | x0y1 | x1y1)) << 16;
+        ez = (lz0 & ~(rz0 | x0z0 | x1z0 | y0z0 | y1z0)) | (lz1 & ~(rz1 | x0z1 | x1z1 | y0z1 | y1z1)) << 16;
+#pragma unroll
+        for (uint32_t z = 0; z < TZ; z++) {
+            const uint32_t l = col + z * NT;
+            uint32_t v = l, bit = 1u << z;
+            if (sx0 & bit) v = l - 1;
+            if (sx1 & bit) v = l + 1;
+            if (sy0 & bit) v = l - TX;
+            if (sy1 & bit) v = l + TX;
+            if (sz0 & bit) v = l - NT;
+            if (sz1 & bit) v = l + NT;
+            D[l] = (uint16_t)v;
+        }
+        for (uint32_t m = minima; m; m &= m - 1) {
+            const uint32_t l = col + (__ffs(m) - 1) * NT;
+            L[l >> 1] = (uint64_t)kNoKey << 32 | 0xFFFF0000u | l;
+        }
+    }
+    __syncthreads();
+
+    // 4. list the edges; pointer jumping along the seeds (concurrent jumps
+    //    only shorten chains, so racing readers stay correct)
+    bool ok = true;
+    {
+        const uint32_t cnt = __popc(ex) + __popc(ey) + __popc(ez);
+        uint32_t incl = cnt;
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= (uint32_t)o) incl += y;
         }
-        if (lane == 31) s_warp[warp] = incl;
-        __syncthreads();
-        uint32_t before_w = 0;
-        for (uint32_t w = 0; w < warp; w++) before_w += s_warp[w];
-        if (threadIdx.x < (uint32_t)BINS)
-            s_bmap[threadIdx.x] =
-                (uint8_t)min((uint32_t)NB - 1, (uint32_t)(((uint64_t)(before_w + incl - c) * NB) / s_nvalid));
-    }
-    __syncthreads();
-    volatile uint32_t *vT = T;
-    auto bucket_of = [&](uint32_t k) { return (uint32_t)s_bmap[bin_of(k)]; };
-    // The bucket of a key grows with the key, so "in bucket b or later" is
-    // k >= s_thr[b], the smallest key of bucket b or after (kmax + 1 if none):
-    // one compare in the shortcut climbs instead of the bin lookup. Read
-    // only after the barriers that end step 4.
-    if (threadIdx.x < (uint32_t)NB) {
-        uint32_t lo = kmin_t, hi = kmax_t + 1u;
-        while (lo < hi) {
-            const uint32_t mid = lo + (hi - lo) / 2;
-            if (bucket_of(mid) >= threadIdx.x) hi = mid;
-            else lo = mid + 1;
-        }
-        s_thr[threadIdx.x] = lo;
-    }
-    // The cross masks of step 4 (from there on, until the bucket repair
-    // rewrites the triplet) are kept in the same bits.
-
-    // 4. cross masks, then a counting sort of the vertices by segment:
-    //    inner vertices by level bucket (segments 0 .. NB-1), minima last
-    //    (segment NB); the histogram is consumed, so the edge hash is cleared
-    for (uint32_t i = threadIdx.x; i < (uint32_t)HS; i += NT) hkey[i] = 0xFFFFFFFFu, hlev[i] = ~0ull;
-    for (uint32_t l = threadIdx.x; l < TV; l += NT) {
-        if (!valid(l)) continue;
-        const uint32_t w0 = vT[l];
-        const uint32_t dl = tid_v(w0);
-        if (dl == l) {  // a minimum
-            atomicAdd(&s_bcur[NB], 1u);
-            continue;
-        }
-        const uint32_t lm = xmask(w0);  // lower neighbours, from the seed
-        uint32_t m = 0;
+        uint32_t pos = 0;
+        if (lane == 31) pos = atomicAdd(&s_nlist, incl);
+        pos = __shfl_sync(0xffffffffu, pos, 31) + incl - cnt;
 #pragma unroll
-        for (uint32_t d = 0; d < 6; d++) {
-            if (!((lm >> d) & 1u)) continue;
-            const uint32_t w = nbr(l, d);
-            if (tid_v(vT[w]) != dl) m |= 1u << d;  // w's minimum is another
+        for (uint32_t axis = 0; axis < 3; axis++) {
+            for (uint32_t m = axis == 0 ? ex : axis == 1 ? ey : ez; m; m &= m - 1) {
+                const uint32_t i = __ffs(m) - 1, up = i >> 4, S = col + (i & 15) * NT;
+                if (pos < (uint32_t)TS::kList) {
+                    list[pos] = (uint16_t)(S | (2 * axis + up) << LV);
+                } else {  // list full: merge in place
+                    const uint32_t step = axis == 0 ? 1u : axis == 1 ? TX : NT;
+                    ok &= sm_merge_rare<TV>(L, K, D, S, up ? S + step : S - step);
+                }
+                pos++;
+            }
         }
-        atomicAdd(&s_bcur[bucket_of(K[l])], 1u);
-        vT[l] = with_mask(sm_pack(l, dl), m);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t run = 0;
-        for (int b = 0; b <= NB; b++) {
-            s_boff[b] = run;
-            run += s_bcur[b];
-            s_bcur[b] = s_boff[b];
-        }
-        s_boff[NB + 1] = run;
-    }
-    __syncthreads();
-    for (uint32_t l = threadIdx.x; l < TV; l += NT) {
-        if (!valid(l)) continue;
-        const uint32_t b = tid_v(vT[l]) == l ? (uint32_t)NB : bucket_of(K[l]);
-        vlist[atomicAdd(&s_bcur[b], 1u)] = (uint16_t)l;  // order within a segment is free
+#pragma unroll 4
+    for (uint32_t z = 0; z < TZ; z++) {
+        const uint32_t l = col + z * NT;
+        uint32_t x = vD[l];
+        x = vD[x];
+        x = vD[x];
+        uint32_t y = vD[x];
+        for (uint32_t h = 0; h < TV && __any_sync(0xffffffffu, x != y); h++) x = y, y = vD[x];
+        vD[l] = (uint16_t)x;
     }
     __syncthreads();
 
-    // 5. rounds over the level buckets
-    bool ok = true;
-    volatile uint16_t *vSC = SC;
-    volatile uint32_t *vHK = hkey;
-    volatile unsigned long long *vHL = hlev;
-    // Round b's bucket repair (5c) runs in the same phase as round b+1's
-    // scan (5a), with no barrier between them. The scan of round b stores in
-    // every vertex of bucket b the round-b shortcut of its minimum, where its
-    // repair starts, so the repair needs no shortcut cache; its climbs follow
-    // links at or below the vertex's own level, which round b+1 never
-    // changes (its merges, in the hash-crowded case run during the scan,
-    // displace only links above bucket b). The scan reads the triplet of a
-    // lower neighbour that the repair may be rewriting: before, (w, minimum)
-    // or (w, shortcut); after, (w, representative) -- every one a vertex of
-    // w's component below the round, with the same shortcut.
-    for (int b = 0; b <= NB; b++) {
-        // 5c. final tile triplets of the inner vertices of bucket b - 1 (this
-        //     also clears their cross masks)
-        if (b > 0) {
-            for (uint32_t i = s_boff[b - 1] + threadIdx.x; i < s_boff[b]; i += NT) {
-                const uint32_t l = vlist[i];
-                uint32_t wr;
-                const uint32_t r = sm_climb<TV>(T, K, tid_v(vT[l]), l, K[l], wr, ok);
-                T[l] = sm_pack(l, r);
-            }
-        }
-        if (b == NB) {
-            // 6. repair the branch minima (Algorithm 5), beside the last
-            //    bucket repair: both only follow links of minima, and a
-            //    minimum's repair moves its target along its own chain below
-            //    its own saddle, which leaves every climb's result unchanged
-            for (uint32_t i = s_boff[NB] + threadIdx.x; i < s_boff[NB + 1]; i += NT) {
-                const uint32_t l = vlist[i];
-                const uint32_t w = vT[l];
-                const uint32_t s = sm_s(w);
-                if (s == l) continue;  // inner vertex or root
-                uint32_t wr;
-                const uint32_t r = sm_climb<TV>(T, K, sm_v(w), s, K[s], wr, ok);
-                if (r != sm_v(w)) T[l] = sm_pack(s, r);
-            }
-            break;
-        }
-        // shortcut of minimum m for round b: climb through the links whose
-        // saddle lies in an earlier bucket, from where round (SC >> IDB) left it
-        auto shortcut = [&](uint32_t m) -> uint32_t {
-            const uint32_t sc = vSC[m];
-            uint32_t x = sc & IDM;
-            if ((sc >> IDB) == (uint32_t)b) return x;
-            for (uint32_t h = 0; h < (uint32_t)TV; h++) {
-                const uint32_t w = vT[x];
-                if (w == sm_pack(x, x) || K[sm_s(w)] >= s_thr[b]) break;
-                x = sm_v(w);
-            }
-            vSC[m] = (uint16_t)(((uint32_t)b << IDB) | x);
-            return x;
-        };
-        // 5a. scan the cross edges whose upper end S lies in bucket b; collect
-        //     those whose ends are not yet known to be connected below S,
-        //     one per pair of shortcuts (the earliest S); store every
-        //     vertex's shortcut for its repair
-        for (uint32_t i = s_boff[b] + threadIdx.x; i < s_boff[b + 1]; i += NT) {
-            const uint32_t S = vlist[i];
-            const uint32_t TSw = vT[S];
-            uint32_t m = xmask(TSw);
-            const uint32_t aS = shortcut(tid_v(TSw));
-            vT[S] = sm_pack(S, aS);
-            if (m == 0) continue;
-            const uint32_t kS = K[S];
-            do {
-                const uint32_t d = __ffs(m) - 1;
-                m &= m - 1;
-                const uint32_t w = nbr(S, d);
-                const uint32_t Tw = vT[w];
-                // a vertex of w's component below the round: an inner
-                // vertex's target, else w itself
-                const uint32_t dw = (tid_s(Tw) == w && tid_v(Tw) != w) ? tid_v(Tw) : w;
-                const uint32_t aw = shortcut(dw);
-                if (aw == aS) continue;  // already connected below S
-                const uint32_t pr = aS < aw ? (aS << IDB) | aw : (aw << IDB) | aS;
-                const unsigned long long lev = ((unsigned long long)kS << 32) | S;
-                uint32_t h = (pr * 0x9E3779B1u) >> (32 - HLOG);
-                bool placed = false;
-                for (uint32_t p = 0; p < kTileHashProbes; p++) {
-                    uint32_t k0 = vHK[h];
-                    if (k0 == 0xFFFFFFFFu) k0 = atomicCAS(hkey + h, 0xFFFFFFFFu, pr);
-                    if (k0 == 0xFFFFFFFFu || k0 == pr) {  // the pair's slot: keep the earliest level
-                        if (vHL[h] > lev) atomicMin(hlev + h, lev);
-                        placed = true;
-                        break;
-                    }
-                    h = (h + 1) & (HS - 1);
+    // 5. merge the listed edges, from the minima their ends descend to. A
+    //    warp takes its share of the list in order; a lane that is done with
+    //    an edge takes the share's next one, so that the lanes do not wait for
+    //    the longest re-insertion of each round. The loop is uniform over the
+    //    warp (votes, no divergent branches): two links of both climbs, then
+    //    one try to link where both have stopped.
+    {
+        const uint32_t nlist = min(s_nlist, (uint32_t)TS::kList);
+        const uint32_t share = (nlist + NT / 32 - 1) / (NT / 32);
+        uint32_t next = (threadIdx.x >> 5) * share;
+        const uint32_t end = min(next + share, nlist), below = (1u << lane) - 1u;
+        uint32_t u = 0, v = 0, it = 0;
+        uint64_t lim = 0;
+        bool have = false;
+        for (;;) {
+            const uint32_t need = __ballot_sync(0xffffffffu, !have);
+            if (need) {
+                const uint32_t i = next + __popc(need & below);
+                if (!have && i < end) {
+                    const uint32_t e = list[i];
+                    const uint32_t S = e & (TV - 1), d = e >> LV;
+                    const uint32_t step = d < 2 ? 1u : d < 4 ? (uint32_t)TX : NT;
+                    u = vD[S];
+                    v = vD[(d & 1) ? S + step : S - step];
+                    lim = level_word(K[S], S);
+                    have = u != v;
                 }
-                if (!placed) sm_merge<TV>(T, K, S, kS, aS, aw, ok);  // hash crowded: merge in place
-            } while (m);
+                __syncwarp();
+                next += __popc(need);
+                if (next >= end && !__any_sync(0xffffffffu, have)) break;
+            }
+            uint64_t wu = 0, wv = 0;
+            bool mu = false, mv = false;
+#pragma unroll
+            for (int hop = 0; hop < 2; hop++) {
+                if (have) {
+                    wu = vL[u >> 1], wv = vL[v >> 1];
+                    mu = wu <= lim, mv = wv <= lim;
+                    u = mu ? link_v(wu) : u;
+                    v = mv ? link_v(wv) : v;
+                }
+                __syncwarp();
+            }
+            have = have && u != v;
+            if (have && !mu && !mv) have = !sm_link(L, K, lim, u, v, wu, wv);
+            __syncwarp();
+            if (++it > kMergeStepLimit) {
+                ok = false;
+                break;
+            }
+        }
+    }
+    __syncthreads();
+
+    // 6. repair the branch minima (Algorithm 5); concurrent repairs move
+    //    targets along their own chains below their own saddles, which
+    //    leaves the end of every walk unchanged
+    for (uint32_t m = minima; m; m &= m - 1) {
+        const uint32_t l = col + (__ffs(m) - 1) * NT;
+        const uint64_t w = vL[l >> 1];
+        if ((uint32_t)(w >> 32) == kNoKey) continue;  // a root
+        const uint64_t lim = w | 0xFFFFu;
+        uint32_t x = link_v(w);
+        for (uint32_t h = 0; h < TV; h++) {
+            const uint64_t wx_ = vL[x >> 1];
+            if (wx_ > lim) break;
+            x = link_v(wx_);
+        }
+        if (x != link_v(w)) vL[l >> 1] = (w & ~(uint64_t)0xFFFFu) | x;
+    }
+    __syncthreads();
+
+    // 7. final tile triplets: inner vertices climb from their minimum
+    for (uint32_t z = 0; z < wz; z++) {
+        const uint32_t l = col + z * NT;
+        const bool is_min = (minima >> z) & 1u;
+        uint32_t x = inx ? vD[l] : vD[0];
+        uint64_t w = vL[x >> 1];
+        const uint64_t lim = is_min || !inx ? 0 : level_word(K[l], l);
+        bool go = w <= lim;
+        for (uint32_t h = 0; h < TV && __any_sync(0xffffffffu, go); h++) {
+            if (go) {
+                x = link_v(w);
+                w = vL[x >> 1];
+                go = w <= lim;
+            }
+            __syncwarp();
+        }
+        // a minimum's own link (a root's word leads to itself)
+        const uint32_t s = is_min && (uint32_t)(w >> 32) != kNoKey ? link_s(w) : l;
+        x = is_min ? link_v(w) : x;
+        if (inx) {
+            const Id gs = gid(s), gv = gid(x);
+            if constexpr (WIDE) reinterpret_cast<ulonglong2 *>(W)[gid(l)] = make_ulonglong2(gs, gv);
+            else W[gid(l)] = tri_pack(gs, gv);
+        }
+    }
+
+    // 8. for k_cross: the edges into the neighbouring tiles that can matter,
+    //    with the tile-local top of their end in this tile, i.e. the deepest
+    //    vertex of its tile component below the edge's level S. By the same
+    //    argument as above an edge (a, b) between tiles adds nothing if a
+    //    parallel edge (c, q) of the face beside it has a lower level: both
+    //    its ends are before S, so with a - c and q - b inside the tiles they
+    //    join a and b below S. What is left are the local minima of the
+    //    level over each face (about 44 of 256 edges on a lognormal field),
+    //    no two of them neighbours, so at most 16 of a group of 32 (one or
+    //    two rows of a face). Both tiles of a face find the same edges in the
+    //    same order. The kept edges of all faces are listed before their
+    //    climbs, so that the climbs run with all lanes busy.
+    if constexpr (!WIDE) {
+        uint64_t *lev = reinterpret_cast<uint64_t *>(K);  // (key, id) of the levels, face after face
+        uint32_t *rec = fd.faces + (size_t)tile * TS::kFaceWords;
+        const uint32_t e = threadIdx.x;
+        auto face_size = [](uint32_t fc) -> uint32_t { return fc % 3 == 0 ? TS::FX : fc % 3 == 1 ? TS::FY : TS::FZ; };
+        auto face_off = [](uint32_t fc) -> uint32_t {
+            return (fc / 3) * TS::FH + (fc % 3 == 0 ? 0 : fc % 3 == 1 ? TS::FX : TS::FX + TS::FY);
+        };
+        uint64_t mine[6];
+#pragma unroll
+        for (uint32_t fc = 0; fc < 6; fc++) {  // faces +x, +y, +z, -x, -y, -z
+            const uint32_t dir = fc % 3, side = fc / 3, lg1 = dir == 0 ? LY : LX;
+            const uint32_t c1 = e & ((1u << lg1) - 1), c2 = e >> lg1;  // in-face coordinates
+            const bool in = e < face_size(fc) && c1 < (dir == 0 ? wy : wx) &&
+                            c2 < (dir == 2 ? wy : wz);
+            const bool has = side == 0 ? (dir == 0 ? x0 + TX < nx : dir == 1 ? y0 + TY < ny : z0 + TZ < nz)
+                                       : (dir == 0 ? x0 : dir == 1 ? y0 : z0) > 0;
+            mine[fc] = ~0ull;
+            if (has && in) {
+                const uint32_t last = dir == 0 ? TX - 1 : dir == 1 ? (TY - 1) * TX : (TZ - 1) * NT;
+                const uint32_t l = (dir == 0 ? c1 * TX + c2 * NT : dir == 1 ? c1 + c2 * NT : e) + (side ? 0u : last);
+                const uint32_t step = dir == 0 ? 1u : dir == 1 ? nx : (uint32_t)nxy;
+                const uint32_t ga = (uint32_t)gid(l), gb = side ? ga - step : ga + step;
+                const uint64_t ka = (uint64_t)K[l] << 32 | ga,
+                               kb = (uint64_t)order_key(sg * __ldg(f + gb)) << 32 | gb;
+                mine[fc] = ka > kb ? ka : kb;
+            }
         }
         __syncthreads();
-        // 5b. run the collected merges side by side and clear the hash
-        for (uint32_t i = threadIdx.x; i < (uint32_t)HS; i += NT) {
-            const uint32_t pr = hkey[i];
-            if (pr == 0xFFFFFFFFu) continue;
-            const unsigned long long lev = hlev[i];
-            hkey[i] = 0xFFFFFFFFu, hlev[i] = ~0ull;
-            sm_merge<TV>(T, K, (uint32_t)lev, (uint32_t)(lev >> 32), pr >> IDB, pr & IDM, ok);
+#pragma unroll
+        for (uint32_t fc = 0; fc < 6; fc++)
+            if (e < face_size(fc)) lev[face_off(fc) + e] = mine[fc];
+        __syncthreads();
+        uint32_t bal[6], tot = 0;
+#pragma unroll
+        for (uint32_t fc = 0; fc < 6; fc++) {
+            // edges outside the face have level ~0: they are not kept (no
+            // level is) and put no other out
+            const uint32_t dir = fc % 3, lg1 = dir == 0 ? LY : LX;
+            const uint32_t m1 = 1u << lg1, m2 = dir == 2 ? TY : TZ, c1 = e & (m1 - 1), c2 = e >> lg1;
+            const uint64_t *p = lev + face_off(fc) + e;
+            const uint64_t v = mine[fc];
+            const bool keep = v != ~0ull && !((c1 > 0 && p[-1] < v) || (c1 + 1 < m1 && p[1] < v) ||
+                                              (c2 > 0 && *(p - m1) < v) || (c2 + 1 < m2 && p[m1] < v));
+            bal[fc] = __ballot_sync(0xffffffffu, keep);
+            tot += __popc(bal[fc]);
+        }
+        uint32_t pos = 0;
+        if (lane == 0) pos = atomicAdd(&s_nface, tot);
+        pos = __shfl_sync(0xffffffffu, pos, 0);
+        const uint32_t grp = threadIdx.x >> 5, below = (1u << lane) - 1u;
+#pragma unroll
+        for (uint32_t fc = 0; fc < 6; fc++) {
+            const uint32_t side = fc / 3, goff = face_off(fc % 3) / 32;
+            if (grp < face_size(fc) / 32) {
+                if (side == 0 && lane == 0) reinterpret_cast<uint8_t *>(rec)[goff + grp] = (uint8_t)__popc(bal[fc]);
+                if ((bal[fc] >> lane) & 1u) {
+                    const uint32_t r = __popc(bal[fc] & below);
+                    // entry: place in the record's tops, edge number
+                    X[pos + r] = (side * TS::kFaceSide + 16 * (goff + grp) + r) << 16 | (face_off(fc) + e);
+                }
+            }
+            pos += __popc(bal[fc]);
         }
         __syncthreads();
+        const uint32_t nface = s_nface;
+        for (uint32_t i = threadIdx.x; i < nface; i += NT) {
+            const uint32_t en = X[i], out = en >> 16, fe = en & 0xFFFFu;
+            const uint64_t v = lev[fe];
+            const uint32_t kS = (uint32_t)(v >> 32), gS = (uint32_t)v;
+            const uint32_t side = fe >= TS::FH, r = fe - side * TS::FH;
+            const uint32_t dir = r < TS::FX ? 0u : r < TS::FX + TS::FY ? 1u : 2u, lg1 = dir == 0 ? LY : LX;
+            const uint32_t ee = r - face_off(dir), c1 = ee & ((1u << lg1) - 1), c2 = ee >> lg1;
+            const uint32_t last = side ? 0u : dir == 0 ? TX - 1 : dir == 1 ? (TY - 1) * TX : (TZ - 1) * NT;
+            uint32_t x = D[(dir == 0 ? c1 * TX + c2 * NT : dir == 1 ? c1 + c2 * NT : ee) + last];
+            for (uint32_t h = 0; h < TV; h++) {
+                const uint64_t w = vL[x >> 1];
+                const uint32_t ks = (uint32_t)(w >> 32);
+                if (ks > kS || (ks == kS && (uint32_t)gid(link_s(w)) > gS)) break;  // link above the level
+                x = link_v(w);
+            }
+            rec[TS::kFaceHead + out] = (uint32_t)gid(x);
+            if (!side) rec[TS::kFaceHead + 2 * TS::kFaceSide + out] = gS;
+        }
     }
     if (!ok) raise_status(status, ST_TIMEOUT);
-    __syncthreads();
-
-    // 6b. for k_cross: the tile-local top of every face vertex at the level
-    //     of its edge into the neighbouring tile, i.e. the deepest vertex of
-    //     its tile component below that level. Levels compare (key, global
-    //     id), since the other end lies outside the tile. Face buffer of a
-    //     tile: +x, +y, +z, then -x, -y, -z faces, each indexed by the two
-    //     in-face coordinates on the full tile extent.
-    if (!WIDE && fd.faces) {
-        constexpr uint32_t FX = TY * TZ, FY = TX * TZ, FZ = TX * TY, FH = FX + FY + FZ;
-        uint32_t *out = fd.faces + (size_t)tile * (2 * FH);
-        const uint32_t has_n = (uint32_t)(x0 + TX < nx) | (uint32_t)(y0 + TY < ny) << 1 |
-                               (uint32_t)(z0 + TZ < nz) << 2 | (uint32_t)(x0 > 0) << 3 | (uint32_t)(y0 > 0) << 4 |
-                               (uint32_t)(z0 > 0) << 5;
-        for (uint32_t e = threadIdx.x; e < 2 * FH; e += NT) {
-            const uint32_t side = e / FH, r = e - side * FH;  // side 0: + faces, 1: - faces
-            uint32_t dir, lx, ly, lz;
-            if (r < FX) dir = 0, ly = r % TY, lz = r / TY, lx = side ? 0 : TX - 1;
-            else if (r < FX + FY) dir = 1, lx = (r - FX) % TX, lz = (r - FX) / TX, ly = side ? 0 : TY - 1;
-            else dir = 2, lx = (r - FX - FY) % TX, ly = (r - FX - FY) / TX, lz = side ? 0 : TZ - 1;
-            if (!((has_n >> (dir + 3 * side)) & 1u) || lx >= wx || ly >= wy || lz >= wz) continue;
-            const uint32_t l = lx + TX * (ly + TY * lz);
-            const uint32_t ga = gid(l);
-            const uint32_t step = dir == 0 ? 1u : dir == 1 ? nx : nxy;
-            const uint32_t gb = side ? ga - step : ga + step;
-            const uint32_t kb = order_key(sg * __ldg(f + gb)), ka = K[l];
-            uint32_t kS = ka, gS = ga;  // level: the later end of the edge
-            if (kbefore(ka, ga, kb, gb)) kS = kb, gS = gb;
-            uint32_t x = l;
-            for (uint32_t h = 0; h < (uint32_t)TV; h++) {
-                const uint32_t w = vT[x];
-                if (w == sm_pack(x, x)) break;
-                const uint32_t sv = sm_s(w);
-                if (kbefore(kS, gS, K[sv], gid(sv))) break;  // link above the level
-                x = sm_v(w);
-            }
-            out[e] = gid(x);
-        }
-    }
-
-    // 7. write the tile's triplets with global ids (coalesced rows)
-    if constexpr (WIDE) {
-        for (uint32_t l = threadIdx.x; l < TV; l += NT) {
-            if (!valid(l)) continue;
-            const uint32_t w = T[l];
-            reinterpret_cast<ulonglong2 *>(W)[gid(l)] = make_ulonglong2(gid(sm_s(w)), gid(sm_v(w)));
-        }
-    } else if (vec) {
-        for (uint32_t q = threadIdx.x; q < TV / 2; q += NT) {
-            const uint32_t l = 2 * q;
-            if (!valid(l)) continue;
-            const uint32_t T0 = T[l], T1 = T[l + 1];
-            *reinterpret_cast<ulonglong2 *>(W + gid(l)) = make_ulonglong2(
-                tri_pack(gid(sm_s(T0)), gid(sm_v(T0))), tri_pack(gid(sm_s(T1)), gid(sm_v(T1))));
-        }
-    } else {
-        for (uint32_t l = threadIdx.x; l < TV; l += NT) {
-            if (!valid(l)) continue;
-            const uint32_t w = T[l];
-            W[gid(l)] = tri_pack(gid(sm_s(w)), gid(sm_v(w)));
-        }
-    }
 }
 
 // One CTA per tile (queue == null), or a persistent grid that takes tiles
-// from a device-side counter until none is left (the batched build). FULL is
-// set when every tile lies inside the grid (grid sides multiples of the tile
-// sides), which drops all partial-tile bounds checks.
-template <int LX, int LY, int LZ, int NT, int NB, class Loc, bool FULL, bool WIDE = false>
-__global__ void __launch_bounds__(NT, NT >= 1024 ? 2 : NT == 512 ? 4 : 1536 / NT) k_tile(Loc loc, uint32_t ntiles, uint32_t *queue,
-                                                                      uint32_t *status)
+// from a device-side counter until none is left (the batched build).
+template <int LX, int LY, int LZ, class Loc, bool WIDE = false>
+__global__ void __launch_bounds__(Tile<LX, LY, LZ>::NT, Tile<LX, LY, LZ>::kCTAs)
+    k_tile(Loc loc, uint32_t ntiles, uint32_t *queue, uint32_t *status)
 {
     if (queue == nullptr) {
         uint32_t local;
         const FieldDesc fd = loc.tile(blockIdx.x, local);
-        tile_body<LX, LY, LZ, NT, NB, FULL, WIDE>(fd, local, status);
+        tile_body<LX, LY, LZ, WIDE>(fd, local, status);
         return;
     }
     __shared__ uint32_t s_next;
@@ -615,7 +609,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 2 : NT == 512 ? 4 : 1536 / NT
         if (t >= ntiles) break;
         uint32_t local;
         const FieldDesc fd = loc.tile(t, local);
-        tile_body<LX, LY, LZ, NT, NB, FULL>(fd, local, status);
+        tile_body<LX, LY, LZ, WIDE>(fd, local, status);
         __syncthreads();
     }
 }
@@ -625,127 +619,48 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 2 : NT == 512 ? 4 : 1536 / NT
 // The rest of the edge loop of Algorithm 1: the edges between neighbouring
 // tiles, merged with 64-bit CAS on the global triplets (Algorithms 2, 3).
 // CTA t takes the edges from tile t to its +x, +y, +z neighbour tiles. k_tile
-// left, for both ends of every such edge (a, b) at level S, the tile-local
-// top of the end at S (the deepest vertex of its tile component below S). Two
-// edges whose ends have the same pair of tops join the same two tile
-// components, and the later of the two is already represented once the
-// earlier is merged, so the CTA keeps, per pair of tops, only the edge with
-// the earliest level (a shared-memory hash with 64-bit atomicMin on
-// (key, id) of S) and merges that one, starting its climbs at the tops.
-//
-// Pairs from different faces never coincide (their second tops lie in
-// different neighbour tiles), so the three faces go through one small hash
-// in turn: fill it with the face's edges, then each edge that still holds
-// its slot's minimum (S identifies an edge within a face) lists itself and
-// clears the slot. The merges then run from the list, one per thread, all
-// lanes busy; the small footprint lets 8 CTAs share an SM.
-constexpr uint32_t kCrossHash = 1024;
-
+// left the edges that can matter (the local minima of the level over each
+// face), in the same order in the records of both tiles: the level S, and for
+// each end its tile-local top at S (the deepest vertex of its tile component
+// below S), where the merge's climbs start. The kernel is bound by the latency
+// of those climbs: 6.3 ms for the 132 edges per tile of the 1024^3 lognormal
+// field (6.4 ms when the CTA read all 768 edges of its faces and found those
+// to merge in a hash of the pairs of tops).
 template <int LX, int LY, int LZ, class Loc>
-__global__ void __launch_bounds__(256, 8) k_cross(Loc loc, uint32_t *status)
+__global__ void __launch_bounds__(128) k_cross(Loc loc, uint32_t *status)
 {
     if (block_skips(status)) return;
     using TS = Tile<LX, LY, LZ>;
-    constexpr uint32_t TX = TS::TX, TY = TS::TY, TZ = TS::TZ;
-    constexpr uint32_t FX = TY * TZ, FY = TX * TZ, FZ = TX * TY, FH = FX + FY + FZ;
-    constexpr uint32_t FMAX = FX > FY ? (FX > FZ ? FX : FZ) : (FY > FZ ? FY : FZ);
-    constexpr uint32_t PER = (FMAX + 255) / 256;  // edges of one face per thread
-    static_assert(FMAX <= kCrossHash / 3 * 2, "hash load factor");
-    static_assert(FH <= 65536, "16-bit face edge indices");
-    constexpr unsigned long long EMPTY = ~0ull;
-    __shared__ unsigned long long hkey[kCrossHash], hval[kCrossHash];
-    __shared__ uint32_t todo_s[FH];  // the saddle S of each edge to merge
-    __shared__ uint16_t todo_e[FH];  // and its face edge index
-    __shared__ uint32_t s_ntodo;
+    constexpr uint32_t G = TS::G, GX = TS::FX / 32, GY = TS::FY / 32;
+    __shared__ uint32_t off[65];  // first edge of each group
     uint32_t tile;
     const FieldDesc fd = loc.tile(blockIdx.x, tile);
-    uint64_t *W = fd.W;
     const Field f{fd.f, fd.sg};
-    const uint32_t nx = fd.nx, ny = fd.ny, nz = fd.nz, ntx = fd.ntx, nty = fd.nty;
-    const uint32_t tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
-    const uint32_t x0 = tx * TX, y0 = ty * TY, z0 = tz * TZ;
-    const uint32_t wx = min(TX, nx - x0), wy = min(TY, ny - y0), wz = min(TZ, nz - z0);
-    const uint32_t nxy = nx * ny;
-    const uint32_t base = z0 * nxy + y0 * nx + x0;
-    const uint32_t *fa = fd.faces + (size_t)tile * (2 * FH);
-    const uint32_t *fbx = fd.faces + (size_t)(tile + 1) * (2 * FH) + FH;
-    const uint32_t *fby = fd.faces + (size_t)(tile + ntx) * (2 * FH) + FH + FX;
-    const uint32_t *fbz = fd.faces + (size_t)(tile + ntx * nty) * (2 * FH) + FH + FX + FY;
-    const bool hx = x0 + TX < nx, hy = y0 + TY < ny, hz = z0 + TZ < nz;
-    // edge e of the +x, +y, +z faces: its ends (a in this tile, b in the
-    // neighbour) and their tops; false where the edge does not exist
-    auto edge = [&](uint32_t e, uint32_t &a, uint32_t &b, uint32_t &ta, uint32_t &tb) -> bool {
-        if (e < FX) {
-            const uint32_t ly = e % TY, lz = e / TY;
-            if (!hx || ly >= wy || lz >= wz) return false;
-            a = base + lz * nxy + ly * nx + (TX - 1);
-            b = a + 1;
-            tb = fbx[e];
-        } else if (e < FX + FY) {
-            const uint32_t k = e - FX, lx = k % TX, lz = k / TX;
-            if (!hy || lx >= wx || lz >= wz) return false;
-            a = base + lz * nxy + (TY - 1) * nx + lx;
-            b = a + nx;
-            tb = fby[k];
-        } else {
-            const uint32_t k = e - FX - FY, lx = k % TX, ly = k / TX;
-            if (!hz || lx >= wx || ly >= wy) return false;
-            a = base + (TZ - 1) * nxy + ly * nx + lx;
-            b = a + nxy;
-            tb = fbz[k];
+    const uint32_t *rec = fd.faces + (size_t)tile * TS::kFaceWords;
+    if (threadIdx.x < 32) {
+        static_assert(G <= 64, "two groups per lane");
+        const uint8_t *cnt = reinterpret_cast<const uint8_t *>(rec);
+        const uint32_t g = 2 * threadIdx.x, c0 = g < G ? cnt[g] : 0u, c1 = g + 1 < G ? cnt[g + 1] : 0u;
+        uint32_t incl = c0 + c1;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (threadIdx.x >= (uint32_t)o) incl += y;
         }
-        ta = fa[e];
-        return true;
-    };
-    for (uint32_t i = threadIdx.x; i < kCrossHash; i += blockDim.x) hkey[i] = EMPTY, hval[i] = EMPTY;
-    if (threadIdx.x == 0) s_ntodo = 0;
-    __syncthreads();
-    for (uint32_t face = 0; face < 3; face++) {
-        const uint32_t e0 = face == 0 ? 0 : face == 1 ? FX : FX + FY;
-        const uint32_t e1 = face == 0 ? FX : face == 1 ? FX + FY : FH;
-        uint32_t slot[PER];
-        unsigned long long mine[PER];
-#pragma unroll
-        for (uint32_t q = 0; q < PER; q++) {
-            const uint32_t e = e0 + q * 256 + threadIdx.x;
-            mine[q] = EMPTY;
-            uint32_t a, b, ta, tb;
-            if (e >= e1 || !edge(e, a, b, ta, tb)) continue;
-            const float va = f[a], vb = f[b];
-            const uint32_t S = before(vb, b, va, a) ? a : b;
-            const float vS = S == a ? va : vb;
-            const unsigned long long key = ((unsigned long long)ta << 32) | tb;
-            const uint32_t bits = vS == 0.0f ? 0u : __float_as_uint(vS);
-            const uint32_t kS = (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
-            mine[q] = ((unsigned long long)kS << 32) | S;
-            uint32_t h = (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> 54) & (kCrossHash - 1);
-            for (uint32_t p = 0; p < kCrossHash; p++) {
-                const unsigned long long k0 = atomicCAS(&hkey[h], EMPTY, key);
-                if (k0 == EMPTY || k0 == key) {
-                    atomicMin(&hval[h], mine[q]);
-                    break;
-                }
-                h = (h + 1) & (kCrossHash - 1);
-            }
-            slot[q] = h;
-        }
-        __syncthreads();
-        // the winner of each slot lists its edge and clears the slot
-#pragma unroll
-        for (uint32_t q = 0; q < PER; q++) {
-            if (mine[q] == EMPTY || hval[slot[q]] != mine[q]) continue;
-            const uint32_t j = atomicAdd(&s_ntodo, 1u);
-            todo_s[j] = (uint32_t)mine[q];
-            todo_e[j] = (uint16_t)(e0 + q * 256 + threadIdx.x);
-            hkey[slot[q]] = EMPTY, hval[slot[q]] = EMPTY;
-        }
-        __syncthreads();
+        off[g] = incl - c0 - c1, off[g + 1] = incl - c1;
+        if (threadIdx.x == 31) off[64] = incl;
     }
+    __syncthreads();
     bool ok = true;
-    for (uint32_t j = threadIdx.x; j < s_ntodo; j += blockDim.x) {
-        uint32_t a, b, ta, tb;
-        edge(todo_e[j], a, b, ta, tb);
-        ok &= merge(W, f, todo_s[j], ta, tb);
+    for (uint32_t i = threadIdx.x; i < off[64]; i += blockDim.x) {
+        uint32_t g = 0;  // the last group whose first edge is at or before i
+#pragma unroll
+        for (uint32_t w = 32; w > 0; w >>= 1)
+            if (off[g + w] <= i) g += w;
+        const uint32_t p = 16 * g + i - off[g];
+        const uint32_t nb = g < GX ? 1u : g < GX + GY ? fd.ntx : fd.ntx * fd.nty;  // the neighbour tile
+        const uint32_t ta = rec[TS::kFaceHead + p], S = rec[TS::kFaceHead + 2 * TS::kFaceSide + p];
+        const uint32_t tb = rec[(size_t)nb * TS::kFaceWords + TS::kFaceHead + TS::kFaceSide + p];
+        ok &= merge(fd.W, f, S, ta, tb);
     }
     if (!ok) raise_status(status, ST_TIMEOUT);
 }
@@ -1089,21 +1004,17 @@ __global__ void __launch_bounds__(NT, 3) k_repair(Loc loc, uint32_t *status, con
 
 // ------------------------------------------------------------ host side
 
-// Tile shapes. Variant 0: 16 x 16 x 16, 4096 vertices, about 53 KiB of
-// shared memory, four CTAs of 512 threads per SM (32 x 16 x 16 tiles in two
-// CTAs of 1024 threads run the tile kernel 6 % slower on the 1024^3 field:
-// with four CTAs per SM, one CTA's round barrier leaves three others to
-// issue). Variant 1: 16 x 16 x 8, 2048 vertices, about 26 KiB, six CTAs of
-// 256 threads per SM, for batches of small fields that would leave most of a
-// large tile empty. 8 level buckets in both. Variant 2: 32 x 16 x 16 bricks
-// of 8192 vertices, the unit of the repair pass of a single field (its
+// Tile shapes. Variant 0: 16 x 16 x 16, 4096 vertices, 44 KB of shared memory,
+// five CTAs of 256 threads per SM. Variant 1: 16 x 16 x 8, for batches of small
+// fields that would leave most of a large tile empty. Variant 2: 32 x 16 x 16
+// bricks of 8192 vertices, the unit of the repair pass of a single field (its
 // shared-memory copies of target chains serve twice as many vertices as in
 // a 16^3 brick) and of the wide-id tile kernel.
-constexpr int kBuckets = 8;
 template <int V> struct Variant;
-template <> struct Variant<0> { static constexpr int LX = 4, LY = 4, LZ = 4, NT = 512; };
-template <> struct Variant<1> { static constexpr int LX = 4, LY = 4, LZ = 3, NT = 256; };
-template <> struct Variant<2> { static constexpr int LX = 5, LY = 4, LZ = 4, NT = 1024; };
+template <> struct Variant<0> { static constexpr int LX = 4, LY = 4, LZ = 4; };
+template <> struct Variant<1> { static constexpr int LX = 4, LY = 4, LZ = 3; };
+template <> struct Variant<2> { static constexpr int LX = 5, LY = 4, LZ = 4; };
+template <int V> using TileOf = Tile<Variant<V>::LX, Variant<V>::LY, Variant<V>::LZ>;
 
 void tile_shape(int variant, uint32_t &tx, uint32_t &ty, uint32_t &tz)
 {
@@ -1116,11 +1027,14 @@ void tile_shape(int variant, uint32_t &tx, uint32_t &ty, uint32_t &tz)
     }
 }
 
+// Workspace words per tile: one per end of every edge of its six faces, more
+// than the face record takes.
 uint32_t face_words(int variant)
 {
-    uint32_t tx, ty, tz;
-    tile_shape(variant, tx, ty, tz);
-    return 2 * (ty * tz + tx * tz + tx * ty);
+    static_assert(TileOf<0>::kFaceWords <= 2 * TileOf<0>::FH && TileOf<1>::kFaceWords <= 2 * TileOf<1>::FH &&
+                      TileOf<2>::kFaceWords <= 2 * TileOf<2>::FH,
+                  "the face records fit the workspace");
+    return 2 * (variant == 1 ? TileOf<1>::FH : variant == 2 ? TileOf<2>::FH : TileOf<0>::FH);
 }
 
 uint64_t tile_count(int variant, uint32_t nx, uint32_t ny, uint32_t nz)
@@ -1130,21 +1044,26 @@ uint64_t tile_count(int variant, uint32_t nx, uint32_t ny, uint32_t nz)
     return (uint64_t)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty) * ((nz + tz - 1) / tz);
 }
 
-template <int V, int NB, class Loc, bool FULL>
-static cudaError_t tile_attrs()
+template <int V, class Loc, bool WIDE = false>
+static cudaError_t launch_tile(const Loc &loc, uint32_t ntiles, uint32_t *queue, int persistent_grid,
+                               uint32_t *status, cudaStream_t st)
 {
     using VV = Variant<V>;
-    using TS = Tile<VV::LX, VV::LY, VV::LZ, VV::NT>;
+    using TS = TileOf<V>;
+    auto kern = k_tile<VV::LX, VV::LY, VV::LZ, Loc, WIDE>;
     static AttrFlags flags;  // per instantiation
     int dev;
-    if (!flags.pending(dev)) return cudaSuccess;
-    auto ktile = k_tile<VV::LX, VV::LY, VV::LZ, VV::NT, NB, Loc, FULL>;
-    cudaError_t e = cudaFuncSetAttribute(ktile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TS::kSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(ktile, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    flags.done(dev);
-    return cudaSuccess;
+    if (flags.pending(dev)) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TS::kSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     cudaSharedmemCarveoutMaxShared);
+        if (e != cudaSuccess) return e;
+        flags.done(dev);
+    }
+    kern<<<queue ? (unsigned)persistent_grid : ntiles, TS::NT, TS::kSmem, st>>>(loc, ntiles, queue, status);
+    count_launch();
+    return cudaGetLastError();
 }
 
 template <int V, int NT, class Loc, bool LAB>
@@ -1162,34 +1081,6 @@ static cudaError_t repair_attrs()
     return e;
 }
 
-// The tile kernel with NB level buckets (merge rounds); FULL only for a
-// single field whose sides are multiples of the tile's.
-template <int V, int NB, class Loc>
-static cudaError_t launch_tile(const Loc &loc, uint32_t ntiles, uint32_t *queue, int persistent_grid, bool full,
-                               uint32_t *status, cudaStream_t st)
-{
-    using VV = Variant<V>;
-    using TS = Tile<VV::LX, VV::LY, VV::LZ, VV::NT>;
-    const unsigned grid = queue ? (unsigned)persistent_grid : ntiles;
-    cudaError_t e;
-    if constexpr (std::is_same<Loc, OneField>::value) {  // batches never take the FULL form
-        if (full) {
-            if ((e = tile_attrs<V, NB, Loc, true>()) != cudaSuccess) return e;
-            k_tile<VV::LX, VV::LY, VV::LZ, VV::NT, NB, Loc, true><<<grid, VV::NT, TS::kSmem, st>>>(loc, ntiles,
-                                                                                               queue, status);
-            count_launch();
-            return cudaGetLastError();
-        }
-    }
-    {
-        if ((e = tile_attrs<V, NB, Loc, false>()) != cudaSuccess) return e;
-        k_tile<VV::LX, VV::LY, VV::LZ, VV::NT, NB, Loc, false><<<grid, VV::NT, TS::kSmem, st>>>(loc, ntiles, queue,
-                                                                                            status);
-    }
-    count_launch();
-    return cudaGetLastError();
-}
-
 template <int V, int NT, class Loc, bool LAB = false>
 static cudaError_t launch_repair(const Loc &loc, uint32_t ntiles, uint32_t *status, cudaStream_t st,
                                  const LabelArgs &la = LabelArgs{})
@@ -1205,25 +1096,22 @@ static cudaError_t launch_repair(const Loc &loc, uint32_t ntiles, uint32_t *stat
 }
 
 // Build steps with tile variant V and the knobs of cfg (MT_CFG_* bits of
-// include/mt.h): the number of level buckets of the tile kernel (its merge
-// and repair rounds) and the CTA size of the repair kernel. Every
-// configuration gives the same triplets.
+// include/mt.h): the CTA size of the repair kernel (MT_CFG_FOUR_ROUNDS chooses
+// nothing: the tile kernel has no rounds). Every configuration gives the same
+// triplets.
 template <int V, class Loc>
-static cudaError_t run_build(const Loc &loc, uint32_t ntiles, uint32_t *queue, int persistent_grid, bool full,
-                             uint32_t *status, cudaStream_t st, uint32_t cfg, const LabelArgs *la = nullptr)
+static cudaError_t run_build(const Loc &loc, uint32_t ntiles, uint32_t *queue, int persistent_grid, uint32_t *status,
+                             cudaStream_t st, uint32_t cfg, const LabelArgs *la = nullptr)
 {
     using VV = Variant<V>;
     cudaError_t e;
     {
         PhaseScope ps(kTile, st);
-        e = (cfg & MT_CFG_FOUR_ROUNDS)
-                ? launch_tile<V, 4>(loc, ntiles, queue, persistent_grid, full, status, st)
-                : launch_tile<V, kBuckets>(loc, ntiles, queue, persistent_grid, full, status, st);
-        if (e != cudaSuccess) return e;
+        if ((e = launch_tile<V>(loc, ntiles, queue, persistent_grid, status, st)) != cudaSuccess) return e;
     }
     {
         PhaseScope ps(kMerge, st);
-        k_cross<VV::LX, VV::LY, VV::LZ, Loc><<<ntiles, 256, 0, st>>>(loc, status);
+        k_cross<VV::LX, VV::LY, VV::LZ, Loc><<<ntiles, 128, 0, st>>>(loc, status);
         count_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -1264,8 +1152,7 @@ static cudaError_t build_one(const float *f, uint64_t *W, uint32_t nx, uint32_t 
     loc.d.nty = (ny + (1u << VV::LY) - 1) >> VV::LY;
     const uint32_t ntz = (nz + (1u << VV::LZ) - 1) >> VV::LZ;
     const uint64_t ntiles = (uint64_t)loc.d.ntx * loc.d.nty * ntz;
-    const bool full = nx % (1u << VV::LX) == 0 && ny % (1u << VV::LY) == 0 && nz % (1u << VV::LZ) == 0;
-    return run_build<V>(loc, (uint32_t)ntiles, nullptr, 0, full, ws.status, st, cfg, la);
+    return run_build<V>(loc, (uint32_t)ntiles, nullptr, 0, ws.status, st, cfg, la);
 }
 
 cudaError_t launch_build(const float *f, uint64_t *W, uint32_t nx, uint32_t ny, uint32_t nz, Workspace &ws,
@@ -1282,7 +1169,6 @@ cudaError_t launch_tile_wide(const float *f, uint64_t *W2, uint32_t nx, uint32_t
                              uint32_t *status, cudaStream_t st)
 {
     using VV = Variant<2>;
-    using TS = Tile<VV::LX, VV::LY, VV::LZ, VV::NT>;
     OneField loc;
     loc.d = FieldDesc{};
     loc.d.f = f;
@@ -1296,23 +1182,7 @@ cudaError_t launch_tile_wide(const float *f, uint64_t *W2, uint32_t nx, uint32_t
     const uint64_t ntz = (nz + (1u << VV::LZ) - 1) >> VV::LZ;
     const uint64_t ntiles = (uint64_t)loc.d.ntx * loc.d.nty * ntz;
     if (ntiles >= 0x80000000ull) return cudaErrorInvalidValue;
-    const bool full = nx % (1u << VV::LX) == 0 && ny % (1u << VV::LY) == 0 && nz % (1u << VV::LZ) == 0;
-    static AttrFlags attr[2];
-    auto kfull = k_tile<VV::LX, VV::LY, VV::LZ, VV::NT, kBuckets, OneField, true, true>;
-    auto kpart = k_tile<VV::LX, VV::LY, VV::LZ, VV::NT, kBuckets, OneField, false, true>;
-    auto kern = full ? kfull : kpart;
-    int dev;
-    if (attr[full].pending(dev)) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TS::kSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        attr[full].done(dev);
-    }
-    kern<<<(unsigned)ntiles, VV::NT, TS::kSmem, st>>>(loc, (uint32_t)ntiles, nullptr, status);
-    count_launch();
-    return cudaGetLastError();
+    return launch_tile<2, OneField, true>(loc, (uint32_t)ntiles, nullptr, 0, status, st);
 }
 
 cudaError_t launch_batch_build(const FieldDesc *d_descs, uint32_t nfields, uint32_t ntiles, uint32_t cfg,
@@ -1323,10 +1193,10 @@ cudaError_t launch_batch_build(const FieldDesc *d_descs, uint32_t nfields, uint3
     if (e != cudaSuccess) return e;
     // persistent grid: as many CTAs as fit on the GPU at once
     const bool small = cfg & MT_CFG_SMALL_TILES;
-    const int per_sm = small ? 1536 / Variant<1>::NT : 2048 / Variant<0>::NT;
+    const int per_sm = small ? TileOf<1>::kCTAs : TileOf<0>::kCTAs;
     const int grid = device_sms() * per_sm;
-    if (small) return run_build<1>(loc, ntiles, queue, grid, false, status, st, cfg);
-    return run_build<0>(loc, ntiles, queue, grid, false, status, st, cfg);
+    if (small) return run_build<1>(loc, ntiles, queue, grid, status, st, cfg);
+    return run_build<0>(loc, ntiles, queue, grid, status, st, cfg);
 }
 
 }  // namespace mt

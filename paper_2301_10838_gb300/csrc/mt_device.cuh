@@ -23,11 +23,11 @@ enum : uint32_t {
 // MT_STRESS_TABLES shrinks the tables so that the tests reach every such
 // path; its results are the same.
 #ifdef MT_STRESS_TABLES
-constexpr uint32_t kTileHashProbes = 1;   // k_tile: probes before merging in place
+constexpr int kTileListShrink = 64;       // k_tile: edge list 64x smaller
 constexpr uint32_t kRepairShrink = 64;    // k_repair: hash, copies and minima list 64x smaller
 constexpr uint32_t kLabelHashLog = 6;     // k_labels: 64 chain starts per brick
 #else
-constexpr uint32_t kTileHashProbes = 16;
+constexpr int kTileListShrink = 1;
 constexpr uint32_t kRepairShrink = 1;
 constexpr uint32_t kLabelHashLog = 12;    // 4096 chain starts per brick
 #endif
