@@ -269,8 +269,8 @@ mt_status mt_batch_prepare(const float *d_arena, const mt_grid *h_grids, uint32_
  *   MT_CFG_FOUR_ROUNDS  accepted, chooses nothing: the tile kernel merges the
  *                       in-tile edges in one round (Algorithm 1 merges the
  *                       edges in any order)
- *   MT_CFG_REPAIR_256   the repair kernel (Algorithm 5) in CTAs of 256
- *                       threads instead of 512
+ *   MT_CFG_REPAIR_256   accepted, chooses nothing: the repair kernel
+ *                       (Algorithm 5) runs a thread per column of a tile
  *   MT_CFG_LARGE_TILES  32x16x16 tiles of 512 threads instead of 16x16x16
  *                       tiles of 256 (single fields only: fewer edges
  *                       between tiles against fewer warps per SM to issue

@@ -83,7 +83,7 @@ MT_SUPERLEVEL = 1  # flag of the _ex calls: the tree of -f (superlevel sets, the
 # launch configurations (bits; every one gives the same results)
 MT_CFG_SMALL_TILES = 1  # 16x16x8 tiles (batches only)
 MT_CFG_FOUR_ROUNDS = 2  # accepted, chooses nothing (the tile kernel has no rounds)
-MT_CFG_REPAIR_256 = 4   # repair CTAs of 256 threads instead of 512
+MT_CFG_REPAIR_256 = 4   # accepted, chooses nothing (the repair kernel has a thread per column)
 MT_CFG_LARGE_TILES = 8  # 32x16x16 tiles (single fields only)
 MT_CFG_COUNT = 8        # batch configurations 0 .. 7
 MT_CFG_SINGLE_MASK = MT_CFG_FOUR_ROUNDS | MT_CFG_REPAIR_256 | MT_CFG_LARGE_TILES

@@ -95,6 +95,11 @@ struct Tile {
     static constexpr int G = (TY * TZ + TX * TZ + TX * TY) / 32;
     static constexpr int kFaceHead = (G + 15) / 16 * 4, kFaceSide = 16 * G;
     static constexpr int kFaceWords = kFaceHead + 3 * kFaceSide;
+    // after the face record, for the repair pass: the minima of every column
+    // (16 bits each), the tile's highest key; the wide path has only these
+    static constexpr int kNoteWords = NT / 2 + 4;
+    template <bool WIDE> static constexpr int kNote = WIDE ? 0 : kFaceWords;
+    template <bool WIDE> static constexpr int kTileWords = kNote<WIDE> + kNoteWords;
     static_assert(TY * TZ <= NT && TX * TZ <= NT, "one edge of a face per thread");
     static constexpr int FX = TY * TZ, FY = TX * TZ, FZ = TX * TY, FH = FX + FY + FZ;  // edges of the + faces
     static_assert(2 * FH * 8 <= TV * 4, "the faces' levels fit the key array");
@@ -182,6 +187,35 @@ __device__ __noinline__ bool sm_merge_rare(uint64_t *L, const uint32_t *K, const
     return false;
 }
 
+// A triplet in global memory: one 64-bit word of two 32-bit ids, or (WIDE) two
+// 64-bit words whose ids carry the merges' tags in their upper 30 bits.
+template <bool WIDE>
+struct Tri {
+    using Id = typename std::conditional<WIDE, uint64_t, uint32_t>::type;
+    static constexpr uint64_t kMask = (1ull << 34) - 1;
+    // saddle id of the word of a tile's inner vertex between the tile kernel
+    // and the repair pass; the word's other id is then the local id of
+    // the tile minimum the vertex descends to (no merge reads such words:
+    // every target of a link is a minimum of its tile)
+    static constexpr Id kInner = WIDE ? (Id)kMask : (Id)0xFFFFFFFFu;
+    static __device__ __forceinline__ void load(const uint64_t *W, Id u, Id &s, Id &v)
+    {
+        if constexpr (WIDE) {
+            const ulonglong2 w = reinterpret_cast<const ulonglong2 *>(W)[u];
+            s = w.x & kMask, v = w.y & kMask;
+        } else {
+            const uint64_t w = W[u];
+            s = tri_s(w), v = tri_v(w);
+        }
+    }
+    static __device__ __forceinline__ void store(uint64_t *W, Id u, Id s, Id v)
+    {
+        if constexpr (WIDE)
+            asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(W + 2 * u), "l"(s), "l"(v) : "memory");
+        else st_tri(W + u, tri_pack(s, v));
+    }
+};
+
 // WIDE: the triplets leave the tile as 128-bit words of two 64-bit ids
 // (W[2u] = s, W[2u + 1] = v) for grids of 2^32 vertices and more; the work
 // inside the tile, on 16-bit local ids, is the same, and no face record is
@@ -189,7 +223,8 @@ __device__ __noinline__ bool sm_merge_rare(uint64_t *L, const uint32_t *K, const
 template <int LX, int LY, int LZ, bool WIDE = false>
 __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, uint32_t *status)
 {
-    using Id = typename std::conditional<WIDE, uint64_t, uint32_t>::type;
+    using TR = Tri<WIDE>;
+    using Id = typename TR::Id;
     const float *__restrict__ f = fd.f;
     const float sg = fd.sg;
     uint64_t *__restrict__ W = fd.W;
@@ -204,7 +239,7 @@ __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, ui
     uint16_t *list = reinterpret_cast<uint16_t *>(X);
     volatile uint64_t *vL = L;
     volatile uint16_t *vD = D;
-    __shared__ uint32_t s_nlist, s_nface;
+    __shared__ uint32_t s_nlist, s_nface, s_kmax;
 
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
@@ -216,6 +251,11 @@ __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, ui
     auto lyo = [](uint32_t l) { return (l >> LX) & (TY - 1); };
     auto lzo = [](uint32_t l) { return l >> (LX + LY); };
     auto gid = [&](uint32_t l) -> Id { return base + (Id)lzo(l) * nxy + (Id)lyo(l) * nx + lxo(l); };
+
+    auto put = [&](Id u, Id sd, Id tg) {
+        if constexpr (WIDE) reinterpret_cast<ulonglong2 *>(W)[u] = make_ulonglong2(sd, tg);
+        else W[u] = tri_pack(sd, tg);
+    };
 
     // 1. load the tile's values (rows of TX floats) as order keys; vertices
     //    outside the grid get kNoKey
@@ -246,7 +286,7 @@ __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, ui
             K[l] = k;
         }
     }
-    if (threadIdx.x == 0) s_nlist = 0, s_nface = 0;
+    if (threadIdx.x == 0) s_nlist = 0, s_nface = 0, s_kmax = 0;
     if (bad) raise_status(status, ST_NONFINITE);
     __syncthreads();
 
@@ -257,7 +297,7 @@ __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, ui
     //    faces give some other word of shared memory; those bits are masked
     //    below.
     const uint32_t col = threadIdx.x, cx = lxo(col), cy = lyo(col);
-    uint32_t px = 0, py = 0, pz = 0, pxy = 0, pmxy = 0, pxz = 0, pyz = 0, qxz = 0, qyz = 0;
+    uint32_t px = 0, py = 0, pz = 0, pxy = 0, pmxy = 0, pxz = 0, pyz = 0, qxz = 0, qyz = 0, kmax = 0;
     {
         uint32_t kc = K[col], kx = K[col + 1], ky = K[col + TX], kxd = 0, kyd = 0;
 #pragma unroll
@@ -265,6 +305,7 @@ __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, ui
             const uint32_t l = col + z * NT;
             const uint32_t kcu = z + 1 < TZ ? K[l + NT] : kNoKey, kxu = z + 1 < TZ ? K[l + NT + 1] : kNoKey,
                            kyu = z + 1 < TZ ? K[l + NT + TX] : kNoKey;
+            kmax = max(kmax, kc + 1);  // kNoKey, outside the grid, gives 0
             px |= (uint32_t)(kx < kc) << z;
             py |= (uint32_t)(ky < kc) << z;
             pz |= (uint32_t)(kcu < kc) << z;
@@ -280,6 +321,8 @@ __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, ui
             kc = kcu, kx = kxu, ky = kyu;
         }
     }
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) atomicMax(&s_kmax, kmax);
     X[col] = px | pxz << 16;
     X[NT + col] = qxz | pxy << 16;
     X[2 * NT + col] = py | pyz << 16;
@@ -450,42 +493,31 @@ __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, ui
     for (uint32_t m = minima; m; m &= m - 1) {
         const uint32_t l = col + (__ffs(m) - 1) * NT;
         const uint64_t w = vL[l >> 1];
-        if ((uint32_t)(w >> 32) == kNoKey) continue;  // a root
-        const uint64_t lim = w | 0xFFFFu;
-        uint32_t x = link_v(w);
-        for (uint32_t h = 0; h < TV; h++) {
-            const uint64_t wx_ = vL[x >> 1];
-            if (wx_ > lim) break;
-            x = link_v(wx_);
-        }
-        if (x != link_v(w)) vL[l >> 1] = (w & ~(uint64_t)0xFFFFu) | x;
-    }
-    __syncthreads();
-
-    // 7. final tile triplets: inner vertices climb from their minimum
-    for (uint32_t z = 0; z < wz; z++) {
-        const uint32_t l = col + z * NT;
-        const bool is_min = (minima >> z) & 1u;
-        uint32_t x = inx ? vD[l] : vD[0];
-        uint64_t w = vL[x >> 1];
-        const uint64_t lim = is_min || !inx ? 0 : level_word(K[l], l);
-        bool go = w <= lim;
-        for (uint32_t h = 0; h < TV && __any_sync(0xffffffffu, go); h++) {
-            if (go) {
-                x = link_v(w);
-                w = vL[x >> 1];
-                go = w <= lim;
+        uint32_t s = l, x = l;  // a root's triplet
+        if ((uint32_t)(w >> 32) != kNoKey) {
+            const uint64_t lim = w | 0xFFFFu;
+            s = link_s(w), x = link_v(w);
+            for (uint32_t h = 0; h < TV; h++) {
+                const uint64_t wx_ = vL[x >> 1];
+                if (wx_ > lim) break;
+                x = link_v(wx_);
             }
-            __syncwarp();
+            if (x != link_v(w)) vL[l >> 1] = (w & ~(uint64_t)0xFFFFu) | x;
         }
-        // a minimum's own link (a root's word leads to itself)
-        const uint32_t s = is_min && (uint32_t)(w >> 32) != kNoKey ? link_s(w) : l;
-        x = is_min ? link_v(w) : x;
-        if (inx) {
-            const Id gs = gid(s), gv = gid(x);
-            if constexpr (WIDE) reinterpret_cast<ulonglong2 *>(W)[gid(l)] = make_ulonglong2(gs, gv);
-            else W[gid(l)] = tri_pack(gs, gv);
-        }
+        put(gid(l), gid(s), gid(x));
+    }
+
+    // 7. for k_repair: the words of the inner vertices say which tile minimum
+    //    they descend to (they get their triplets once all merges are done);
+    //    the tile's minima and highest key
+    uint32_t *rec = fd.faces + (size_t)tile * TS::template kTileWords<WIDE>;
+    reinterpret_cast<uint16_t *>(rec + TS::template kNote<WIDE>)[col] = (uint16_t)minima;
+    if (threadIdx.x == 0) rec[TS::template kNote<WIDE> + NT / 2] = s_kmax - 1;
+    if (inx) {
+        const Id u0 = gid(col);
+#pragma unroll
+        for (uint32_t z = 0; z < TZ; z++)
+            if (z < wz && !((minima >> z) & 1u)) put(u0 + z * nxy, TR::kInner, (Id)vD[col + z * NT]);
     }
 
     // 8. for k_cross: the edges into the neighbouring tiles that can matter,
@@ -502,7 +534,6 @@ __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, ui
     //    climbs, so that the climbs run with all lanes busy.
     if constexpr (!WIDE) {
         uint64_t *lev = reinterpret_cast<uint64_t *>(K);  // (key, id) of the levels, face after face
-        uint32_t *rec = fd.faces + (size_t)tile * TS::kFaceWords;
         const uint32_t e = threadIdx.x;
         auto face_size = [](uint32_t fc) -> uint32_t { return fc % 3 == 0 ? TS::FX : fc % 3 == 1 ? TS::FY : TS::FZ; };
         auto face_off = [](uint32_t fc) -> uint32_t {
@@ -636,7 +667,8 @@ __global__ void __launch_bounds__(128) k_cross(Loc loc, uint32_t *status)
     uint32_t tile;
     const FieldDesc fd = loc.tile(blockIdx.x, tile);
     const Field f{fd.f, fd.sg};
-    const uint32_t *rec = fd.faces + (size_t)tile * TS::kFaceWords;
+    constexpr uint32_t kWords = TS::template kTileWords<false>;
+    const uint32_t *rec = fd.faces + (size_t)tile * kWords;
     if (threadIdx.x < 32) {
         static_assert(G <= 64, "two groups per lane");
         const uint8_t *cnt = reinterpret_cast<const uint8_t *>(rec);
@@ -659,7 +691,7 @@ __global__ void __launch_bounds__(128) k_cross(Loc loc, uint32_t *status)
         const uint32_t p = 16 * g + i - off[g];
         const uint32_t nb = g < GX ? 1u : g < GX + GY ? fd.ntx : fd.ntx * fd.nty;  // the neighbour tile
         const uint32_t ta = rec[TS::kFaceHead + p], S = rec[TS::kFaceHead + 2 * TS::kFaceSide + p];
-        const uint32_t tb = rec[(size_t)nb * TS::kFaceWords + TS::kFaceHead + TS::kFaceSide + p];
+        const uint32_t tb = rec[(size_t)nb * kWords + TS::kFaceHead + TS::kFaceSide + p];
         ok &= merge(fd.W, f, S, ta, tb);
     }
     if (!ok) raise_status(status, ST_TIMEOUT);
@@ -673,48 +705,75 @@ __global__ void __launch_bounds__(128) k_cross(Loc loc, uint32_t *status)
 // order is not yet part of the sublevel set at s. Concurrent repairs only
 // replace a target by one further along the same chain below the same level,
 // so a stale copy of an entry is still a valid (longer) way to the same
-// answer: every chase here uses ordinary cached loads.
+// answer: every read of a triplet here is an ordinary cached load.
 //
-// One CTA per tile, in four steps:
-//  1. scan the tile: collect its branch minima (s != u) in a list, and enter
-//     the target v of every inner vertex (s == u != v) in a shared-memory
-//     hash of targets (about 360 distinct targets serve the 7,400 inner
-//     vertices of a tile on the 1024^3 lognormal field);
-//  2. give each hashed target a slot for a copy of its chain;
-//  3. repair the branch minima, and copy the first kHops links of the chain
-//     of every hashed target into its slot, with the order keys of their
-//     saddles (one loop over both kinds of work, all lanes busy). A link
-//     whose saddle is not above the one before is folded into it (whoever
-//     passed the earlier saddle passes this one too), so the saddles of a
-//     copy increase strictly;
-//  4. repair every inner vertex: a binary search in its target's copy finds
-//     the last link at or below it, and only when the whole copy lies below
-//     it does the walk go on along the global chain.
-// Steps 1 and 4 load four rows per thread before using any, so that the
-// loads of a thread overlap. A branch minimum that finds the list full is
-// marked in a bitmap in step 1 and repaired in step 3 (kept out of the
-// unrolled row loop); a target without a slot (hash or copies full) is
-// chased along the global chain in step 4.
+// One CTA per tile of the tile kernel, a thread per column. The chains that
+// the tile's vertices climb are copied to shared memory once, as a small
+// forest of link words that is closed up to the tile's highest value:
+//  1. number the tile's minima densely (the tile kernel left a bit per
+//     vertex, the tile's highest key, and in the word of every inner vertex
+//     the local id of the minimum it descends to);
+//  2. a node per minimum: its link's saddle (key, and local id if the saddle
+//     lies in the tile) and the node of its target. A target outside the tile
+//     is entered in a small hash, and its own link follows in the next round,
+//     until the links lie above the tile's highest value. On a lognormal
+//     field a tile has about 450 minima and 46 such foreign nodes, in 4 rounds;
+//  3. repair the branch minima by climbing the forest (past its edge, the
+//     global chain);
+//  4. repair every inner vertex: from its minimum's node follow the links at
+//     or below it (2.4 on average), voting so that the warp stays together.
+// Tables that are full (more than kMin minima, a crowded hash) leave a link
+// without a node; whoever needs it goes on along the global chain.
+//
+// What it costs, on the 1024^3 lognormal field: 9.7 ms, 10.8 ms with labels
+// (11.7 and 14.2 ms with copies of each target's first 8 links found through
+// a hash per vertex, from triplets that the tile kernel had repaired itself
+// at 3.8 ms more): numbering 1.0, links 3.2 (chains of dependent reads),
+// targets and labels 0.7 to 1.2, inner vertices 4.9 to 5.4 (16 to 24 bytes
+// each way per vertex, 130 thread instructions). Issue slots are 60 % busy.
+// Climbing the forest before its targets are repaired costs 1.4 ms more.
 //
 // With LAB the pass also labels the components of G_t (the labels of
 // k_labels) where it already stands. The representative of u at level t is
 // the end of the walk from u along links with f(s) <= t (Algorithm 4 with a
 // value test). Any valid triplet forest gives the same end, repaired or not:
 // a walk stops at the first link above t, and every link it passes joins two
-// vertices of one component of G_t, the second deeper. So a branch minimum
-// continues the walk from its repaired target when its saddle is at or below
-// t (step 3), every copied chain gives its target's label by a search of the
-// copy for t, shared by all inner vertices of the target (step 3), and step 4
-// writes every vertex's label: 0xFFFFFFFF above t, the copy's label, or a
-// global walk for a target without a copy. Concurrent repairs move entries
-// along their own chains below their own saddles, which keeps every walk's
-// end.
+// vertices of one component of G_t, the second deeper. So a node at the edge
+// of the forest takes its label from a global walk, every other node by
+// climbing the forest to t or to such a node, and a vertex in G_t has the
+// label of its representative's node: t >= f(u), so the walk at t passes the
+// representative at u. Concurrent repairs move entries along their own
+// chains below their own saddles, which keeps every walk's end.
+
+// The end of the walk from x along links at or below level (fS, S)
+// (Algorithm 4 along the global chain), the next triplet read beside the
+// saddle's value. ok = false if the walk ran out of steps. Out of line, like
+// label_walk: few vertices need it, and inlined copies slow the common path.
+template <bool WIDE>
+__device__ __noinline__ typename Tri<WIDE>::Id repair_walk(const uint64_t *W, const float *f, float sg,
+                                                          typename Tri<WIDE>::Id x, typename Tri<WIDE>::Id S,
+                                                          float fS, bool *ok)
+{
+    using Id = typename Tri<WIDE>::Id;
+    Id s, v;
+    Tri<WIDE>::load(W, x, s, v);
+    for (uint32_t h = 0; h <= kChaseLimit; h++) {
+        if (s == x && v == x) return x;
+        const float fs = sg * __ldg(f + s);
+        Id ns, nv;
+        Tri<WIDE>::load(W, v, ns, nv);
+        if (s != S && !(fs < fS || (fs == fS && s < S))) return x;
+        x = v, s = ns, v = nv;
+    }
+    *ok = false;
+    return x;
+}
+
 // The label at t of the component reached from x: the end r of the walk
 // along links with f(s) <= t (Algorithm 4 with a value test), or 0xFFFFFFFF
 // when eps > 0 and r heads a branch of persistence below eps (its component
 // lies in a filled pit). Bit 32 of the result is set if the walk ran out of
-// steps. Out of line: the callers take it for a minority of vertices, and
-// inlined copies in their unrolled loops slow the common path.
+// steps.
 __device__ __noinline__ uint64_t label_walk(const uint64_t *W, const Field f, uint32_t x, float t, float eps)
 {
     for (uint32_t h = 0;; h++) {
@@ -731,272 +790,375 @@ __device__ __noinline__ uint64_t label_walk(const uint64_t *W, const Field f, ui
     return x;
 }
 
-// Representative(x, u) for an inner vertex whose target's copy does not reach
-// its level (Algorithm 4 along the global chain); bit 32 set if the walk ran
-// out of steps. Out of line for the same reason as label_walk.
-__device__ __noinline__ uint64_t repair_walk(const uint64_t *W, const Field f, uint32_t x, uint32_t u, float fu)
-{
-    uint32_t steps = 0;
-    const uint32_t r = representative_cached(W, f, x, u, fu, steps);
-    return steps > kChaseLimit ? (1ull << 32) | r : r;
-}
-
-template <int LX, int LY, int LZ>
+template <int LX, int LY, int LZ, bool LAB, bool WIDE>
 struct RepairShape {
-    static constexpr uint32_t TV = 1u << (LX + LY + LZ);
-    static constexpr uint32_t kHops = 8;          // links copied per target
-    static constexpr uint32_t kCap = TV / 16 / kRepairShrink;   // copies
-    static constexpr uint32_t kHash = TV / 8 / kRepairShrink;   // hash slots for targets
-    static constexpr uint32_t kList = TV / 4 / kRepairShrink;   // branch minima listed
-    static constexpr size_t kSmem = (size_t)kCap * kHops * 12 + (size_t)kHash * 4 + (size_t)kHash * 2 +
-                                    (size_t)kList * 2 + (size_t)kCap * 2 + (size_t)TV / 8;
-    static constexpr size_t kSmemLab = kSmem + (size_t)kCap * 4;  // + each copy's label
+    static constexpr uint32_t TV = 1u << (LX + LY + LZ), NT = 1u << (LX + LY);
+    static constexpr uint32_t kMin = TV / 4 / kRepairShrink;    // minima with a node
+    static constexpr uint32_t kHash = TV / 16 / kRepairShrink;  // hash slots (nodes) of foreign minima
+    static constexpr uint32_t kNodes = kMin + kHash;
+    // shared memory: link word and global id (with LAB also the label) of
+    // every node (and of the one that stands for none), hash keys, the node of
+    // each minimum by x-adjacent pair, the foreign nodes in the order they
+    // were entered
+    static constexpr size_t kSmem = (size_t)(kNodes + 4) * 8 + (size_t)kNodes * (LAB || WIDE ? 8 : 4) +
+                                    (size_t)kHash * (WIDE ? 8 : 4) + (size_t)TV / 2 * 2 + (size_t)kHash * 2;
+    static constexpr int kFit = (int)(227 * 1024 / (kSmem + 1024));
+    static constexpr int kCTAs = kFit < (int)(1536 / NT) ? kFit : (int)(1536 / NT);
 };
 
-template <int LX, int LY, int LZ, int NT, class Loc, bool LAB>
-__global__ void __launch_bounds__(NT, 3) k_repair(Loc loc, uint32_t *status, const LabelArgs la)
+template <int LX, int LY, int LZ, class Loc, bool LAB, bool WIDE = false>
+__global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, WIDE>::kCTAs)
+    k_repair(Loc loc, uint32_t *status, const LabelArgs la)
 {
     if (block_skips(status)) return;
-    using RS = RepairShape<LX, LY, LZ>;
-    constexpr uint32_t TX = 1u << LX, TY = 1u << LY, TV = RS::TV, H = RS::kHops, CAP = RS::kCap,
-                       HS = RS::kHash, LIST = RS::kList;
-    constexpr uint32_t NB = 4;  // rows loaded together
-    static_assert(TV % (NT * NB) == 0, "whole batches of rows");
-    static_assert((H & (H - 1)) == 0 && (HS & (HS - 1)) == 0, "powers of two");
-    static_assert((HS + LIST + CAP) % 2 == 0, "the bitmap after the 16-bit arrays is 4-byte aligned");
-    constexpr uint32_t EMPTY = 0xFFFFFFFFu;  // free hash slot (not a vertex id: ids are < n < 2^32 - 1)
-    constexpr uint32_t END = 0xFFFFFFFFu;    // copied saddle after the chain's root: above every (key, id)
-    constexpr uint16_t NOSLOT = 0xFFFFu;
+    static_assert(!(LAB && WIDE), "labels have 32-bit ids");
+    using RS = RepairShape<LX, LY, LZ, LAB, WIDE>;
+    using TR = Tri<WIDE>;
+    using Id = typename TR::Id;
+    constexpr uint32_t TX = 1u << LX, TY = 1u << LY, TZ = 1u << LZ, TV = RS::TV, NT = RS::NT, MIN = RS::kMin,
+                       HS = RS::kHash, NN = RS::kNodes;
+    static_assert((HS & (HS - 1)) == 0, "power of two");
+    constexpr uint32_t NONE = 0xFFFFu;             // no node, no local id
+    constexpr Id EMPTY = ~(Id)0;                   // free hash slot (no vertex id)
     constexpr uint32_t kProbes = 16;
-    extern __shared__ __align__(16) uint32_t smem[];
-    uint32_t *es = smem;                       // copied links: saddle, its key, target
-    uint32_t *ek = es + CAP * H;
-    uint32_t *ev = ek + CAP * H;
-    uint32_t *hkey = ev + CAP * H;             // hashed targets
-    uint32_t *slab = hkey + HS;                // LAB: label at t of each copy's target
-    uint16_t *hslot = reinterpret_cast<uint16_t *>(slab + (LAB ? CAP : 0));  // copy slots of the targets
-    uint16_t *list = hslot + HS;               // branch minima (tile-local ids)
-    uint16_t *cslot = list + LIST;             // hash slot of each copy's target
-    uint32_t *ovf = reinterpret_cast<uint32_t *>(cslot + CAP);  // bit per vertex: minima past the list
-    __shared__ uint32_t s_nmin, s_ncopy;
+    // word of a node whose target found no node, and of node NN, which stands
+    // for a minimum without one: stops every climb, and whoever ends there
+    // goes on along the global chain
+    constexpr uint64_t LOST = (uint64_t)kNoKey << 32 | 0xFFFEFFFFu;
+    extern __shared__ __align__(16) uint64_t rep_smem[];
+    uint64_t *word = rep_smem;                     // links: saddle's key, its local id (NONE: outside), next node
+    uint64_t *out = word + NN + 4;                 // LAB: label and global id of each node, else global id
+    Id *ids = reinterpret_cast<Id *>(out);
+    Id *hkey = reinterpret_cast<Id *>(out + (LAB || WIDE ? NN : NN / 2));
+    uint16_t *node = reinterpret_cast<uint16_t *>(hkey + HS);  // of the minimum of each x-adjacent pair
+    uint16_t *order = node + TV / 2;
+    __shared__ uint32_t s_nmin, s_nf;
+    auto id_of = [&](uint32_t x) -> Id {
+        if constexpr (LAB) return (uint32_t)out[x];
+        else return ids[x];
+    };
 
     uint32_t tile;
     const FieldDesc fd = loc.tile(blockIdx.x, tile);
     uint64_t *W = fd.W;
-    const Field f{fd.f, fd.sg};
+    const float *__restrict__ f = fd.f;
+    const float sg = fd.sg;
     const uint32_t nx = fd.nx, ny = fd.ny, nz = fd.nz, ntx = fd.ntx, nty = fd.nty;
     const uint32_t tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
-    const uint32_t x0 = tx * TX, y0 = ty * TY, z0 = tz * (1u << LZ);
-    const uint32_t wx = min(TX, nx - x0), wy = min(TY, ny - y0), wz = min(1u << LZ, nz - z0);
-    const uint32_t nxy = nx * ny;
-    const uint32_t base = z0 * nxy + y0 * nx + x0;
-    const uint32_t lane = threadIdx.x & 31;
-    auto gid_of = [&](uint32_t l) {
-        return base + (l >> (LX + LY)) * nxy + ((l >> LX) & (TY - 1)) * nx + (l & (TX - 1));
+    const uint32_t x0 = tx * TX, y0 = ty * TY, z0 = tz * TZ;
+    const uint32_t wx = min(TX, nx - x0), wy = min(TY, ny - y0), wz = min(TZ, nz - z0);
+    const Id nxy = (Id)nx * ny;
+    const Id base = (Id)z0 * nxy + (Id)y0 * nx + x0;
+    const uint32_t lane = threadIdx.x & 31, col = threadIdx.x, cx = col & (TX - 1), cy = col >> LX;
+    const bool inx = cx < wx && cy < wy;
+    const Id ucol = base + (Id)cy * nx + cx;       // vertex z of the column: ucol + z * nxy
+    bool ok = true;
+    auto val = [&](Id u) { return sg * __ldg(f + u); };
+    // local id of vertex v, NONE outside the tile. Within the tile's span the
+    // quotients are below 16, so a product with the reciprocal is off by at
+    // most one, which the remainder shows.
+    const float rnxy = 1.0f / (float)nxy, rnx = 1.0f / (float)nx;
+    auto local_of = [&](Id v) -> uint32_t {
+        const Id rel = v - base;                   // wraps far beyond the tile for an earlier vertex
+        if ((uint64_t)rel >= (uint64_t)TZ * nxy) return NONE;
+        uint32_t dz = (uint32_t)((float)rel * rnxy);
+        if ((Id)dz * nxy > rel) dz--;
+        Id r = rel - (Id)dz * nxy;
+        if (r >= nxy) dz++, r -= nxy;
+        if ((uint64_t)r >= (uint64_t)TY * nx) return NONE;
+        uint32_t dy = (uint32_t)((float)(uint32_t)r * rnx);
+        if (dy * nx > (uint32_t)r) dy--;
+        uint32_t dx = (uint32_t)r - dy * nx;
+        if (dx >= nx) dy++, dx -= nx;
+        return dx < wx && dy < wy && dz < wz ? dx + TX * (dy + TY * dz) : NONE;
     };
-    auto inside = [&](uint32_t l) {
-        return (l & (TX - 1)) < wx && ((l >> LX) & (TY - 1)) < wy && (l >> (LX + LY)) < wz;
+    auto id_at = [&](uint32_t l) -> Id {
+        return base + (Id)(l >> (LX + LY)) * nxy + (Id)((l >> LX) & (TY - 1)) * nx + (l & (TX - 1));
     };
-    auto hash0 = [](uint32_t v) { return (v * 0x9E3779B1u) >> (32 - log2i(HS)); };
-    // slot of target v in the hash, HS if absent
-    auto find = [&](uint32_t v) -> uint32_t {
-        uint32_t h = hash0(v);
+    // the tile's rows of values and triplets start on their way to L2: the
+    // forest is built with dependent loads, each a trip to HBM otherwise
+    auto prefetch_tri = [&](Id u) { asm volatile("prefetch.global.L2 [%0];" ::"l"(W + (WIDE ? 2 : 1) * (size_t)u)); };
+    if (threadIdx.x < TV / 16) {
+        const uint32_t l = 16 * threadIdx.x, lx = l & (TX - 1), ly = (l >> LX) & (TY - 1), lz = l >> (LX + LY);
+        if (lx < wx && ly < wy && lz < wz) {
+            const Id u = id_at(l);
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(f + u));
+            prefetch_tri(u);
+            if (WIDE && lx + 8 < wx) prefetch_tri(u + 8);
+        }
+    }
+    for (uint32_t i = threadIdx.x; i < HS; i += NT) hkey[i] = EMPTY;
+    if (threadIdx.x == 0) s_nmin = 0, s_nf = 0, word[NN] = LOST;
+    __syncthreads();
+
+    // 1. number the tile's minima (the bits the tile kernel left per column)
+    using TS = Tile<LX, LY, LZ>;
+    const uint32_t *note = fd.faces + (size_t)tile * TS::template kTileWords<WIDE> + TS::template kNote<WIDE>;
+    const uint32_t minima = reinterpret_cast<const uint16_t *>(note)[col], kmax = note[NT / 2];
+    {
+        const uint32_t cnt = __popc(minima);
+        uint32_t incl = cnt;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= (uint32_t)o) incl += y;
+        }
+        uint32_t pos = 0;
+        if (lane == 31) pos = atomicAdd(&s_nmin, incl);
+        pos = __shfl_sync(0xffffffffu, pos, 31) + incl - cnt;
+        for (uint32_t m = minima; m; m &= m - 1, pos++) {
+            const uint32_t z = __ffs(m) - 1;
+            node[(col + z * NT) >> 1] = (uint16_t)(pos < MIN ? pos : NN);
+            if (pos < MIN) {
+                if constexpr (LAB) out[pos] = ucol + z * nxy;
+                else ids[pos] = ucol + z * nxy;
+            }
+        }
+    }
+    __syncthreads();
+    const uint32_t nmin = min(s_nmin, MIN);
+
+    // 2. links of the nodes
+    volatile Id *vhk = hkey;
+    auto node_of = [&](Id v) -> uint32_t {         // the node of minimum v, entered if it is a new foreign one
+        const uint32_t l = local_of(v);
+        if (l != NONE) return node[l >> 1];
+        uint32_t h = ((uint32_t)v * 0x9E3779B1u) >> (32 - log2i(HS));
         for (uint32_t p = 0; p < kProbes; p++) {
-            const uint32_t k = hkey[h];
-            if (k == v) return h;
-            if (k == EMPTY) return HS;
+            Id k = vhk[h];
+            if (k == EMPTY) {
+                if constexpr (WIDE)
+                    k = atomicCAS(reinterpret_cast<unsigned long long *>(hkey + h), (unsigned long long)EMPTY,
+                                  (unsigned long long)v);
+                else k = atomicCAS(hkey + h, EMPTY, v);
+                if (k == EMPTY) {
+                    order[atomicAdd(&s_nf, 1u)] = (uint16_t)h;
+                    if constexpr (LAB) out[MIN + h] = v;
+                    else ids[MIN + h] = v;
+                    return MIN + h;
+                }
+            }
+            if (k == v) return MIN + h;
             h = (h + 1) & (HS - 1);
         }
-        return HS;
+        return NN;
     };
-
-    bool ok = true;
-    constexpr uint32_t OUT = 0xFFFFFFFFu;  // label of a vertex outside G_t (or in a filled pit)
-    const float lt = la.t;
-    // label at t reached from x: x itself when x is known to head its
-    // component (walk false) and eps <= 0, else label_walk
+    const uint32_t kt = order_key(la.t);
+    // the label at t of the component that node x heads or leads out of the forest to
     auto label_from = [&](uint32_t x, bool walk) -> uint32_t {
-        if (!walk && !(la.eps > 0.0f)) return x;
-        const uint64_t r = label_walk(W, f, x, lt, la.eps);
+        if constexpr (!LAB) return 0;
+        if (!walk && !(la.eps > 0.0f)) return (uint32_t)id_of(x);
+        const uint64_t r = label_walk(W, Field{f, sg}, (uint32_t)id_of(x), la.t, la.eps);
         if (r >> 32) ok = false;
         return (uint32_t)r;
     };
-    // label of branch minimum m (saddle value fs) whose link leads to r
-    auto min_label = [&](uint32_t m, float fs, uint32_t r) { return fs <= lt ? label_from(r, true) : label_from(m, false); };
-
-    for (uint32_t i = threadIdx.x; i < HS; i += NT) hkey[i] = EMPTY;
-    for (uint32_t i = threadIdx.x; i < TV / 32; i += NT) ovf[i] = 0;
-    if (threadIdx.x == 0) s_nmin = 0, s_ncopy = 0;
-    __syncthreads();
-
-    // 1. scan
-    volatile uint32_t *vhk = hkey;
-    for (uint32_t l0 = 0; l0 < TV; l0 += NT * NB) {
-        uint64_t Tb[NB];
-#pragma unroll
-        for (uint32_t k = 0; k < NB; k++) {
-            const uint32_t l = l0 + k * NT + threadIdx.x;
-            const uint32_t u = gid_of(l);
-            Tb[k] = inside(l) ? W[u] : tri_pack(u, u);
+    auto set_label = [&](uint32_t x, uint32_t label) { reinterpret_cast<uint32_t *>(out)[2 * x + 1] = label; };
+    auto enter = [&](uint32_t x, Id u, Id s, Id v, float fs) {
+        uint32_t ks = kNoKey, sl = NONE, next = NONE;
+        if (!(s == u && v == u)) {
+            ks = order_key(fs);
+            sl = local_of(s);
+            if (ks <= kmax) next = node_of(v);
         }
-#pragma unroll
-        for (uint32_t k = 0; k < NB; k++) {
-            const uint32_t l = l0 + k * NT + threadIdx.x;
-            const uint32_t u = gid_of(l);
-            const uint32_t s = tri_s(Tb[k]), v = tri_v(Tb[k]);
-            const bool is_min = s != u;
-            if (!is_min && v != u) {  // inner vertex: hash its target
-                uint32_t h = hash0(v);
-                for (uint32_t p = 0; p < kProbes; p++) {
-                    uint32_t kk = vhk[h];
-                    if (kk == EMPTY) kk = atomicCAS(hkey + h, EMPTY, v);
-                    if (kk == EMPTY || kk == v) break;
-                    h = (h + 1) & (HS - 1);
-                }
-            }
-            const uint32_t bal = __ballot_sync(0xffffffffu, is_min);
-            if (bal) {
-                uint32_t pos = 0;
-                if (lane == 0) pos = atomicAdd(&s_nmin, __popc(bal));
-                pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(bal & ((1u << lane) - 1u));
-                if (is_min && pos < LIST) {
-                    list[pos] = (uint16_t)l;
-                } else if (is_min) {  // list full: mark it for step 3
-                    atomicOr(&ovf[l >> 5], 1u << (l & 31));
-                }
-            }
-        }
-    }
-    __syncthreads();
-
-    // 2. copy slots for the hashed targets
-    for (uint32_t i = threadIdx.x; i < HS; i += NT) {
-        if (hkey[i] == EMPTY) continue;
-        const uint32_t c = atomicAdd(&s_ncopy, 1u);
-        hslot[i] = c < CAP ? (uint16_t)c : NOSLOT;
-        if (c < CAP) cslot[c] = (uint16_t)i;
-    }
-    __syncthreads();
-
-    // 3. branch minima (items below nmin) and copies of target chains (one
-    //    item per copy: copy c serves the target in hash slot cslot[c])
-    // Repair of the branch minimum with local id l (and with LAB its label,
-    // which step 4 overwrites with 0xFFFFFFFF above t)
-    auto repair_min = [&](uint32_t l) {
-        const uint32_t u = gid_of(l);
-        const uint64_t T = W[u];
-        const uint32_t s = tri_s(T), t = tri_v(T);
-        uint32_t steps = 0;
-        const float fs = f[s];
-        const uint32_t r = representative_cached(W, f, t, s, fs, steps);
-        if (steps > kChaseLimit) ok = false;
-        else if (r != t) st_tri(W + u, tri_pack(s, r));
-        if (LAB) la.labels[u] = min_label(u, fs, r);
+        word[x] = next == NN ? LOST : (uint64_t)ks << 32 | sl << 16 | next;
+        if (LAB && next >= NN) set_label(x, label_from(x, ks <= kt));
     };
-    // items: the listed minima, the copies, then (when the list overflowed)
-    // the words of the bitmap of the minima past it; the two kinds of minima
-    // share one call of repair_min, so that its code appears once
-    const uint32_t nmin = min(s_nmin, LIST), ncopy = min(s_ncopy, CAP);
-    const uint32_t nover = s_nmin > LIST ? TV / 32 : 0;
-    for (uint32_t i = threadIdx.x; i < nmin + ncopy + nover; i += NT) {
-        if (i < nmin || i >= nmin + ncopy) {
-            const bool listed = i < nmin;
-            const uint32_t w = i - nmin - ncopy;
-            for (uint32_t m = listed ? 1u : ovf[w]; m; m &= m - 1)
-                repair_min(listed ? (uint32_t)list[i] : w * 32 + __ffs(m) - 1);
-            continue;
+    // the tile's minima, two per thread with their loads side by side
+    for (uint32_t i = threadIdx.x; i < nmin; i += 2 * NT) {
+        Id u[2], s[2], v[2];
+        float fs[2];
+#pragma unroll
+        for (uint32_t k = 0; k < 2; k++) {
+            u[k] = id_of(min(i + k * NT, nmin - 1));
+            TR::load(W, u[k], s[k], v[k]);
         }
-        const uint32_t c = i - nmin;  // copy c, of the target in hash slot cslot[c]
-        const uint32_t x0v = hkey[cslot[c]];
-        const uint32_t b = c * H;
-        uint32_t x = x0v, j = 0;
-        bool ended = false;
-        uint64_t T = W[x];
-        for (uint32_t step = 0; step < 4 * H && j < H; step++) {
-            const uint32_t s = tri_s(T), v = tri_v(T);
-            if (s == x && v == x) {  // a root: the chain ends
-                ended = true;
-                break;
-            }
-            const float fs = f[s];
-            const uint64_t Tn = W[v];  // loaded together with the saddle's value
-            const uint32_t ks = order_key(fs);
-            if (j > 0 && !kbefore(ek[b + j - 1], es[b + j - 1], ks, s)) {
-                ev[b + j - 1] = v;  // not above the previous saddle: fold
+#pragma unroll
+        for (uint32_t k = 0; k < 2; k++) {
+            fs[k] = val(s[k]);
+            prefetch_tri(v[k]);                    // read in the next round if it is a new foreign node
+        }
+#pragma unroll
+        for (uint32_t k = 0; k < 2; k++)
+            if (i + k * NT < nmin) enter(i + k * NT, u[k], s[k], v[k], fs[k]);
+    }
+    for (uint32_t done = 0;;) {
+        __syncthreads();
+        const uint32_t nf = s_nf;
+        __syncthreads();
+        if (done >= nf) break;
+        for (uint32_t i = done + threadIdx.x; i < nf; i += NT) {
+            const uint32_t x = MIN + order[i];
+            const Id u = id_of(x);
+            Id s, v;
+            TR::load(W, u, s, v);
+            prefetch_tri(v);
+            enter(x, u, s, v, val(s));
+        }
+        done = nf;
+    }
+
+    // Climbs in the forest: from node x (its word w) follow the links at or
+    // below a level, a comparison of the words as in the tile kernel. Where the
+    // link's saddle or the level's lies outside the tile, its local id is NONE
+    // and the comparison is by key alone; on equal keys the ids decide, read
+    // from W.
+    auto link_next = [](uint64_t w) { return (uint32_t)w & 0xFFFFu; };
+    auto saddle_before = [&](uint32_t x, Id S) -> bool {
+        Id s, v;
+        TR::load(W, id_of(x), s, v);
+        return s <= S;
+    };
+
+    // 3. repair the nodes' targets, in the forest (which shortens the climbs
+    //    that follow) and, for the tile's minima, in W. A node whose link has
+    //    a node lies at or below the tile's highest key, and so do the links it
+    //    follows; a minimum with a higher saddle goes along the global chain.
+    const uint32_t nf = s_nf, nall = nmin + nf;
+    volatile uint64_t *vword = word;
+    for (uint32_t i0 = 0; i0 < nall; i0 += NT) {
+        const uint32_t i = i0 + threadIdx.x;
+        const uint32_t n = i < nmin ? i : i < nall ? MIN + order[i - nmin] : NN;
+        const uint64_t w = vword[n];
+        const uint32_t ks = (uint32_t)(w >> 32), sl = (uint32_t)w >> 16, x0 = link_next(w);
+        const bool link = x0 != NONE;
+        const uint64_t lim = sl != NONE ? w | 0xFFFFu : ((uint64_t)ks << 32) - 1;
+        uint32_t x = link ? x0 : NN;
+        uint64_t wx_ = vword[x];
+        for (uint32_t h = 0; h < 2 * NN; h++) {
+            const bool go = wx_ <= lim && link;
+            if (!__any_sync(0xffffffffu, go)) {
+                bool tie = link && (uint32_t)(wx_ >> 32) == ks && (sl == NONE || (uint32_t)wx_ >= 0xFFFF0000u);
+                if (!__any_sync(0xffffffffu, tie)) break;
+                if (tie) {
+                    Id s, v;
+                    TR::load(W, id_of(n), s, v);
+                    tie = saddle_before(x, s);
+                }
+                if (!__any_sync(0xffffffffu, tie)) break;
+                x = tie ? link_next(wx_) : x;
             } else {
-                es[b + j] = s, ek[b + j] = ks, ev[b + j] = v;
-                j++;
+                x = go ? link_next(wx_) : x;
             }
-            x = v;
-            T = Tn;
+            wx_ = vword[x];
         }
-        // pad: after a root with END (above every level); when the copy
-        // stops short of the root, with the last link again, leading to x
-        // where a vertex above it goes on along the global chain
-        const uint32_t ps = ended ? END : es[b + j - 1], pk = ended ? END : ek[b + j - 1];
-        for (; j < H; j++) es[b + j] = ps, ek[b + j] = pk, ev[b + j] = x;
-        if (LAB) {
-            // links of the copy at or below t (saddle values; END is above
-            // every finite key); past the whole copy the walk goes on globally
-            const uint32_t kt = order_key(lt);
-            uint32_t lo = 0;
-            while (lo < H && ek[b + lo] <= kt) lo++;
-            slab[c] = label_from(lo ? ev[b + lo - 1] : x0v, lo == H);
+        const bool left = link && (uint32_t)wx_ == (uint32_t)LOST;  // further along the global chain
+        if (link && !left && x != x0) vword[n] = (w & ~(uint64_t)0xFFFFu) | x;
+        if (i >= nmin || (ks == kNoKey && w != LOST)) continue;     // foreign, or the root
+        const Id u = id_of(n);
+        Id s, v = 0;
+        if (!link || left || sl == NONE) TR::load(W, u, s, v);
+        else s = id_at(sl);
+        if (!link || left) TR::store(W, u, s, repair_walk<WIDE>(W, f, sg, left ? id_of(x) : v, s, val(s), &ok));
+        else if (x != x0 || WIDE) TR::store(W, u, s, id_of(x));
+    }
+    // with LAB the labels of the nodes (those without a next node have theirs)
+    if constexpr (LAB) {
+        __syncthreads();
+        const uint64_t limt = (uint64_t)kt << 32 | 0xFFFFFFFFu;
+        for (uint32_t i0 = 0; i0 < nall; i0 += NT) {
+            const uint32_t i = i0 + threadIdx.x;
+            const uint32_t n = i < nmin ? i : i < nall ? MIN + order[i - nmin] : NN;
+            uint32_t x = n;
+            uint64_t w = word[n];
+            const bool link = link_next(w) != NONE;
+            for (uint32_t h = 0; h < NN; h++) {
+                const bool go = w <= limt && link_next(w) != NONE;
+                if (!__any_sync(0xffffffffu, go)) break;
+                x = go ? link_next(w) : x;
+                w = word[x];
+            }
+            if (link)
+                set_label(n, link_next(w) == NONE ? reinterpret_cast<volatile uint32_t *>(out)[2 * x + 1]
+                                                  : label_from(x, false));
+        }
+    }
+    // minima without a node
+    if (s_nmin > MIN) {
+        for (uint32_t m = minima; m; m &= m - 1) {
+            const uint32_t z = __ffs(m) - 1;
+            if (node[(col + z * NT) >> 1] != NN) continue;
+            const Id u = ucol + z * nxy;
+            Id s, v;
+            TR::load(W, u, s, v);
+            if (!(s == u && v == u)) TR::store(W, u, s, repair_walk<WIDE>(W, f, sg, v, s, val(s), &ok));
+            else if (WIDE) TR::store(W, u, s, v);
+            if constexpr (LAB) {
+                uint32_t lab = 0xFFFFFFFFu;
+                if (val(u) <= la.t) {
+                    const uint64_t r = label_walk(W, Field{f, sg}, u, la.t, la.eps);
+                    if (r >> 32) ok = false;
+                    lab = (uint32_t)r;
+                }
+                la.labels[u] = lab;
+            }
         }
     }
     __syncthreads();
 
-    // 4. inner vertices
-    for (uint32_t l0 = 0; l0 < TV; l0 += NT * NB) {
-        uint64_t Tb[NB];
-        float fb[NB];
-#pragma unroll
-        for (uint32_t k = 0; k < NB; k++) {
-            const uint32_t l = l0 + k * NT + threadIdx.x;
-            const uint32_t u = gid_of(l);
-            const bool in = inside(l);
-            Tb[k] = in ? W[u] : tri_pack(u, u);
-            fb[k] = in ? f[u] : 0.0f;
+    // 4. inner vertices, the next row's value and word loaded ahead (rows
+    //    unrolled by 4 or 8 with their loads first measured slower: the
+    //    kernel then waits for instructions)
+    uint32_t lost = 0;                             // bit z: the climb left the forest
+    auto row = [&](uint32_t z, float &fu, uint32_t &m) {
+        const bool in = inx && z < wz, inner = in && !((minima >> z) & 1u);
+        const Id u = ucol + z * nxy;
+        fu = 0.0f, m = 0;
+        if (LAB ? in : inner) fu = val(u);
+        if (inner) m = (uint32_t)W[WIDE ? 2 * u + 1 : u];
+    };
+    float fnext;
+    uint32_t mnext;
+    row(0, fnext, mnext);
+#pragma unroll 1
+    for (uint32_t z = 0; z < wz; z++) {
+        const uint32_t l = col + z * NT;
+        const Id u = ucol + z * nxy;
+        const bool inner = inx && !((minima >> z) & 1u);
+        const float fu = fnext;
+        const uint32_t m = inner ? mnext : l;      // the vertex's minimum
+        row(z + 1, fnext, mnext);
+        const uint32_t ku = order_key(fu);
+        const uint64_t lim = inner ? level_word(ku, l) : 0u;
+        uint32_t x = inner || (LAB && inx && ((minima >> z) & 1u)) ? node[m >> 1] : NN;
+        uint64_t w = word[x];
+        for (uint32_t h = 0; h < 2 * NN; h++) {
+            const bool go = w <= lim;
+            if (!__any_sync(0xffffffffu, go)) {
+                // a link of the same key whose saddle lies outside the tile?
+                bool tie = inner && (uint32_t)(w >> 32) == ku && (uint32_t)w >= 0xFFFF0000u;
+                if (!__any_sync(0xffffffffu, tie)) break;
+                if (tie) tie = saddle_before(x, u);
+                if (!__any_sync(0xffffffffu, tie)) break;
+                x = tie ? link_next(w) : x;
+            } else {
+                x = go ? link_next(w) : x;
+            }
+            w = word[x];
         }
-#pragma unroll
-        for (uint32_t k = 0; k < NB; k++) {
-            const uint32_t l = l0 + k * NT + threadIdx.x;
-            const uint32_t u = gid_of(l);
-            const uint32_t s = tri_s(Tb[k]), t = tri_v(Tb[k]);
-            if (s != u || t == u) {  // a branch minimum, the root, or outside the grid
-                if (LAB && inside(l)) {
-                    if (!(fb[k] <= lt)) la.labels[u] = OUT;
-                    else if (s == u) la.labels[u] = u;  // the root labels itself
-                }
-                continue;
+        const bool leave = inner && (uint32_t)w == (uint32_t)LOST;
+        lost |= (uint32_t)leave << z;
+        if (x != NN && !leave) {
+            if constexpr (LAB) {
+                const uint64_t o = out[x];
+                if (inner) W[u] = tri_pack(u, (uint32_t)o);
+                la.labels[u] = fu <= la.t ? (uint32_t)(o >> 32) : 0xFFFFFFFFu;
+            } else if constexpr (WIDE) {
+                reinterpret_cast<ulonglong2 *>(W)[u] = make_ulonglong2(u, ids[x]);
+            } else {
+                W[u] = tri_pack(u, ids[x]);
             }
-            const uint32_t h = find(t);
-            const uint16_t c = h < HS ? hslot[h] : NOSLOT;
-            uint32_t r = t;
-            bool global = true;
-            if (c != NOSLOT) {
-                const uint32_t b = (uint32_t)c * H;
-                const uint32_t ku = order_key(fb[k]);
-                // number of copied links at or below u (saddles increase)
-                uint32_t lo = 0;
-#pragma unroll
-                for (uint32_t w = H / 2; w > 0; w >>= 1)
-                    if (!kbefore(ku, u, ek[b + lo + w - 1], es[b + lo + w - 1])) lo += w;
-                if (lo < H && !kbefore(ku, u, ek[b + lo], es[b + lo])) lo++;
-                if (lo > 0) r = ev[b + lo - 1];
-                global = lo == H;
-            }
-            if (global) {
-                const uint64_t rr = repair_walk(W, f, r, u, fb[k]);
-                if (rr >> 32) {
-                    ok = false;
-                    continue;
-                }
-                r = (uint32_t)rr;
-            }
-            if (r != t) st_tri(W + u, tri_pack(u, r));
-            // t >= f(u): the walk at t passes the representative at u
-            if (LAB) la.labels[u] = !(fb[k] <= lt) ? OUT : c != NOSLOT ? slab[c] : label_from(r, true);
+        }
+    }
+    // the few that left the forest follow the global chain from their minimum
+    for (; lost; lost &= lost - 1) {
+        const Id u = ucol + (__ffs(lost) - 1) * nxy;
+        const float fu = val(u);
+        const Id r = repair_walk<WIDE>(W, f, sg, id_at((uint32_t)W[WIDE ? 2 * u + 1 : u]), u, fu, &ok);
+        if constexpr (WIDE) reinterpret_cast<ulonglong2 *>(W)[u] = make_ulonglong2(u, r);
+        else W[u] = tri_pack(u, r);
+        if constexpr (LAB) {
+            const uint64_t q = label_walk(W, Field{f, sg}, (uint32_t)r, la.t, la.eps);
+            if (q >> 32) ok = false;
+            la.labels[u] = fu <= la.t ? (uint32_t)q : 0xFFFFFFFFu;
         }
     }
     if (!ok) raise_status(status, ST_TIMEOUT);
@@ -1006,10 +1168,8 @@ __global__ void __launch_bounds__(NT, 3) k_repair(Loc loc, uint32_t *status, con
 
 // Tile shapes. Variant 0: 16 x 16 x 16, 4096 vertices, 44 KB of shared memory,
 // five CTAs of 256 threads per SM. Variant 1: 16 x 16 x 8, for batches of small
-// fields that would leave most of a large tile empty. Variant 2: 32 x 16 x 16
-// bricks of 8192 vertices, the unit of the repair pass of a single field (its
-// shared-memory copies of target chains serve twice as many vertices as in
-// a 16^3 brick) and of the wide-id tile kernel.
+// fields that would leave most of a large tile empty. Variant 2: 32 x 16 x 16,
+// which a single field may choose (MT_CFG_LARGE_TILES).
 template <int V> struct Variant;
 template <> struct Variant<0> { static constexpr int LX = 4, LY = 4, LZ = 4; };
 template <> struct Variant<1> { static constexpr int LX = 4, LY = 4, LZ = 3; };
@@ -1028,12 +1188,12 @@ void tile_shape(int variant, uint32_t &tx, uint32_t &ty, uint32_t &tz)
 }
 
 // Workspace words per tile: one per end of every edge of its six faces, more
-// than the face record takes.
+// than its record takes.
 uint32_t face_words(int variant)
 {
-    static_assert(TileOf<0>::kFaceWords <= 2 * TileOf<0>::FH && TileOf<1>::kFaceWords <= 2 * TileOf<1>::FH &&
-                      TileOf<2>::kFaceWords <= 2 * TileOf<2>::FH,
-                  "the face records fit the workspace");
+    static_assert(TileOf<0>::kTileWords<false> <= 2 * TileOf<0>::FH && TileOf<1>::kTileWords<false> <= 2 * TileOf<1>::FH &&
+                      TileOf<2>::kTileWords<false> <= 2 * TileOf<2>::FH,
+                  "the tile records fit the workspace");
     return 2 * (variant == 1 ? TileOf<1>::FH : variant == 2 ? TileOf<2>::FH : TileOf<0>::FH);
 }
 
@@ -1066,31 +1226,21 @@ static cudaError_t launch_tile(const Loc &loc, uint32_t ntiles, uint32_t *queue,
     return cudaGetLastError();
 }
 
-template <int V, int NT, class Loc, bool LAB>
-static cudaError_t repair_attrs()
-{
-    using VV = Variant<V>;
-    using RS = RepairShape<VV::LX, VV::LY, VV::LZ>;
-    static AttrFlags flags;  // per instantiation
-    int dev;
-    if (!flags.pending(dev)) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(k_repair<VV::LX, VV::LY, VV::LZ, NT, Loc, LAB>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)(LAB ? RS::kSmemLab : RS::kSmem));
-    if (e == cudaSuccess) flags.done(dev);
-    return e;
-}
-
-template <int V, int NT, class Loc, bool LAB = false>
+template <int V, class Loc, bool LAB = false, bool WIDE = false>
 static cudaError_t launch_repair(const Loc &loc, uint32_t ntiles, uint32_t *status, cudaStream_t st,
                                  const LabelArgs &la = LabelArgs{})
 {
     using VV = Variant<V>;
-    using RS = RepairShape<VV::LX, VV::LY, VV::LZ>;
-    cudaError_t e;
-    if ((e = repair_attrs<V, NT, Loc, LAB>()) != cudaSuccess) return e;
-    k_repair<VV::LX, VV::LY, VV::LZ, NT, Loc, LAB><<<ntiles, NT, LAB ? RS::kSmemLab : RS::kSmem, st>>>(loc, status,
-                                                                                                   la);
+    using RS = RepairShape<VV::LX, VV::LY, VV::LZ, LAB, WIDE>;
+    auto kern = k_repair<VV::LX, VV::LY, VV::LZ, Loc, LAB, WIDE>;
+    static AttrFlags flags;  // per instantiation
+    int dev;
+    if (flags.pending(dev)) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS::kSmem);
+        if (e != cudaSuccess) return e;
+        flags.done(dev);
+    }
+    kern<<<ntiles, RS::NT, RS::kSmem, st>>>(loc, status, la);
     count_launch();
     return cudaGetLastError();
 }
@@ -1117,21 +1267,9 @@ static cudaError_t run_build(const Loc &loc, uint32_t ntiles, uint32_t *queue, i
     }
     PhaseScope ps(kRepair, st);
     if constexpr (std::is_same<Loc, OneField>::value) {
-        // a single field is repaired (and labelled) in 32 x 16 x 16 bricks
-        using RV = Variant<2>;
-        OneField rl = loc;
-        rl.d.ntx = (loc.d.nx + (1u << RV::LX) - 1) >> RV::LX;
-        rl.d.nty = (loc.d.ny + (1u << RV::LY) - 1) >> RV::LY;
-        const uint32_t rn = rl.d.ntx * rl.d.nty * ((loc.d.nz + (1u << RV::LZ) - 1) >> RV::LZ);
-        if (la)
-            return (cfg & MT_CFG_REPAIR_256) ? launch_repair<2, 256, Loc, true>(rl, rn, status, st, *la)
-                                             : launch_repair<2, 512, Loc, true>(rl, rn, status, st, *la);
-        return (cfg & MT_CFG_REPAIR_256) ? launch_repair<2, 256>(rl, rn, status, st)
-                                         : launch_repair<2, 512>(rl, rn, status, st);
-    } else {
-        return (cfg & MT_CFG_REPAIR_256) ? launch_repair<V, 256>(loc, ntiles, status, st)
-                                         : launch_repair<V, 512>(loc, ntiles, status, st);
+        if (la) return launch_repair<V, Loc, true>(loc, ntiles, status, st, *la);
     }
+    return launch_repair<V>(loc, ntiles, status, st);
 }
 
 // A single field in the tile shape of variant V (0, or 2 with MT_CFG_LARGE_TILES).
@@ -1162,27 +1300,43 @@ cudaError_t launch_build(const float *f, uint64_t *W, uint32_t nx, uint32_t ny, 
     return build_one<0>(f, W, nx, ny, nz, ws, faces, sg, st, cfg, la);
 }
 
-// The tile kernel with 64-bit ids and 128-bit output words (the wide path):
-// one CTA per 32x16x16 tile (the tiles whose boundaries k_w_cross merges),
-// no face buffer.
-cudaError_t launch_tile_wide(const float *f, uint64_t *W2, uint32_t nx, uint32_t ny, uint32_t nz, float sg,
-                             uint32_t *status, cudaStream_t st)
+// The tile kernel and the repair pass with 64-bit ids and 128-bit words (the
+// wide path), on 16x16x16 tiles; notes: wide_note_words() u32 per tile.
+uint32_t wide_note_words() { return TileOf<0>::kTileWords<true>; }
+
+static bool wide_field(const float *f, uint64_t *W2, uint32_t *notes, uint32_t nx, uint32_t ny, uint32_t nz, float sg,
+                       OneField &loc, uint64_t &ntiles)
 {
-    using VV = Variant<2>;
-    OneField loc;
+    using VV = Variant<0>;
     loc.d = FieldDesc{};
     loc.d.f = f;
     loc.d.W = W2;
-    loc.d.faces = nullptr;
+    loc.d.faces = notes;
     loc.d.sg = sg;
     loc.d.nx = nx, loc.d.ny = ny, loc.d.nz = nz;
     loc.d.n = (uint64_t)nx * ny * nz;
-    loc.d.ntx = (nx + (1u << VV::LX) - 1) >> VV::LX;
-    loc.d.nty = (ny + (1u << VV::LY) - 1) >> VV::LY;
-    const uint64_t ntz = (nz + (1u << VV::LZ) - 1) >> VV::LZ;
-    const uint64_t ntiles = (uint64_t)loc.d.ntx * loc.d.nty * ntz;
-    if (ntiles >= 0x80000000ull) return cudaErrorInvalidValue;
-    return launch_tile<2, OneField, true>(loc, (uint32_t)ntiles, nullptr, 0, status, st);
+    loc.d.ntx = (uint32_t)(((uint64_t)nx + (1u << VV::LX) - 1) >> VV::LX);
+    loc.d.nty = (uint32_t)(((uint64_t)ny + (1u << VV::LY) - 1) >> VV::LY);
+    ntiles = (uint64_t)loc.d.ntx * loc.d.nty * (((uint64_t)nz + (1u << VV::LZ) - 1) >> VV::LZ);
+    return ntiles < 0x80000000ull;
+}
+
+cudaError_t launch_tile_wide(const float *f, uint64_t *W2, uint32_t *notes, uint32_t nx, uint32_t ny, uint32_t nz, float sg,
+                             uint32_t *status, cudaStream_t st)
+{
+    OneField loc;
+    uint64_t ntiles;
+    if (!wide_field(f, W2, notes, nx, ny, nz, sg, loc, ntiles)) return cudaErrorInvalidValue;
+    return launch_tile<0, OneField, true>(loc, (uint32_t)ntiles, nullptr, 0, status, st);
+}
+
+cudaError_t launch_repair_wide(const float *f, uint64_t *W2, uint32_t *notes, uint32_t nx, uint32_t ny, uint32_t nz, float sg,
+                               uint32_t *status, cudaStream_t st)
+{
+    OneField loc;
+    uint64_t ntiles;
+    if (!wide_field(f, W2, notes, nx, ny, nz, sg, loc, ntiles)) return cudaErrorInvalidValue;
+    return launch_repair<0, OneField, false, true>(loc, (uint32_t)ntiles, status, st);
 }
 
 cudaError_t launch_batch_build(const FieldDesc *d_descs, uint32_t nfields, uint32_t ntiles, uint32_t cfg,

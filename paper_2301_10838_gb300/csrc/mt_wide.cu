@@ -8,12 +8,13 @@
 // ids. It computes the same unique triplets as the 32-bit path, in three
 // steps of Algorithm 1 (which merges the edges in any order):
 //   1. the tile kernel of the 32-bit path (mt_build.cu) builds the merge tree
-//      of every 32x16x16 tile in shared memory on 16-bit local ids and writes
+//      of every 16x16x16 tile in shared memory on 16-bit local ids and writes
 //      it with 64-bit ids (launch_tile_wide);
-//   2. k_w_cross merges every edge between neighbouring tiles with the
-//      lock-free Merge (Algorithms 2 and 3) on the global 128-bit words,
-//      starting from the edge's two ends;
-//   3. k_w_repair restores minimality (Algorithms 4 and 5).
+//   2. k_w_cross merges the edges between neighbouring tiles that can matter
+//      with the lock-free Merge (Algorithms 2 and 3) on the global 128-bit
+//      words, starting from the tile minima their ends descend to;
+//   3. the repair pass of the 32-bit path restores minimality (Algorithms 4
+//      and 5; launch_repair_wide).
 //
 // Torn reads. While merges run, every 64-bit half of a word carries the same
 // 30-bit version tag above its 34-bit id; a compare-and-swap writes both
@@ -46,38 +47,45 @@ constexpr uint32_t kWChunk = 4096;         // vertices per pair-compaction chunk
 constexpr int kWThreads = 256;
 
 // Workspace: [0, 256) status word, [256, 512) meta (npairs, roots, root),
-// then per-chunk pair counts (u32) and offsets (u64).
+// then per-chunk pair counts (u32) and offsets (u64), then the notes that the
+// tile kernel leaves for the repair pass.
 struct WideWs {
     uint32_t *status;
     uint64_t *meta;
     uint32_t *counts;
     uint64_t *offsets;
+    uint32_t *notes;
     uint64_t nchunks;
 };
 
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-size_t wide_ws_bytes(uint64_t n)
+constexpr uint32_t kSide = 16;  // side of a tile (of the tile kernel's, too)
+
+struct Geo {
+    uint64_t nx, ny, nz, nxy, n;
+};
+
+size_t wide_ws_bytes(const Geo &g)
 {
-    const uint64_t nchunks = (n + kWChunk - 1) / kWChunk;
-    return 512 + al256(nchunks * 4) + al256(nchunks * 8);
+    const uint64_t nchunks = (g.n + kWChunk - 1) / kWChunk, t = kSide;
+    const uint64_t tiles = ((g.nx + t - 1) / t) * ((g.ny + t - 1) / t) * ((g.nz + t - 1) / t);
+    return 512 + al256(nchunks * 4) + al256(nchunks * 8) + al256(tiles * wide_note_words() * 4);
 }
 
-bool carve(void *base, size_t bytes, uint64_t n, WideWs &ws)
+bool carve(void *base, size_t bytes, const Geo &g, WideWs &ws)
 {
-    if (!base || ((uintptr_t)base & 255) || bytes < wide_ws_bytes(n)) return false;
+    const uint64_t n = g.n;
+    if (!base || ((uintptr_t)base & 255) || bytes < wide_ws_bytes(g)) return false;
     char *p = static_cast<char *>(base);
     ws.nchunks = (n + kWChunk - 1) / kWChunk;
     ws.status = reinterpret_cast<uint32_t *>(p);
     ws.meta = reinterpret_cast<uint64_t *>(p + 256);
     ws.counts = reinterpret_cast<uint32_t *>(p + 512);
     ws.offsets = reinterpret_cast<uint64_t *>(p + 512 + al256(ws.nchunks * 4));
+    ws.notes = reinterpret_cast<uint32_t *>(p + 512 + al256(ws.nchunks * 4) + al256(ws.nchunks * 8));
     return true;
 }
-
-struct Geo {
-    uint64_t nx, ny, nz, nxy, n;
-};
 
 // the values as the order sees them (sg = -1: the tree of -f)
 struct FieldW {
@@ -175,95 +183,85 @@ struct WideMerge {
     }
 };
 
-// One CTA per 32x16x16 tile: the edges from the tile to its +x, +y and +z
-// neighbour tiles, each merged from its two ends at the level of its later
-// end (the tile kernel has already merged every edge inside a tile).
-constexpr uint32_t kTX = 32, kTY = 16, kTZ = 16;
-
+// One CTA per 16x16x16 tile: the edges from the tile to its +x, +y and +z
+// neighbour tiles, merged at the level of their later end (the tile kernel
+// has already merged every edge inside a tile). An edge adds nothing if a
+// parallel edge of its face beside it has a lower level (both its ends are
+// then before the edge's level, and inside the two tiles they are neighbours
+// of the edge's ends), so only the local minima of the level over each face
+// are merged: about 132 of the 768 edges on a lognormal field. They are
+// listed first, so that all lanes have one to merge.
 __global__ void __launch_bounds__(256) k_w_cross(FieldW f, Geo g, uint32_t ntx, uint32_t nty, uint64_t *W,
                                                  uint32_t *status)
 {
-    if (*status) return;  // no barriers below: a per-thread test is enough
-    constexpr uint32_t FX = kTY * kTZ, FY = kTX * kTZ, FZ = kTX * kTY, FH = FX + FY + FZ;
+    if (block_skips(status)) return;
+    constexpr uint32_t F = kSide * kSide;
+    constexpr uint64_t kInner = kIdMask;  // saddle id of an inner vertex's word; its target is then a local id
+    __shared__ uint64_t lev[3][F];        // (order key, order of the id within the face) of each edge's level
+    __shared__ uint16_t list[3 * F];
+    __shared__ uint32_t s_n;
     const WideMerge M{W, f};
     const uint32_t tile = blockIdx.x;
     const uint32_t tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
-    const uint64_t x0 = (uint64_t)tx * kTX, y0 = (uint64_t)ty * kTY, z0 = (uint64_t)tz * kTZ;
-    const uint64_t wx = min((uint64_t)kTX, g.nx - x0), wy = min((uint64_t)kTY, g.ny - y0),
-                   wz = min((uint64_t)kTZ, g.nz - z0);
+    const uint64_t x0 = (uint64_t)tx * kSide, y0 = (uint64_t)ty * kSide, z0 = (uint64_t)tz * kSide;
+    const uint32_t wx = (uint32_t)min((uint64_t)kSide, g.nx - x0), wy = (uint32_t)min((uint64_t)kSide, g.ny - y0),
+                   wz = (uint32_t)min((uint64_t)kSide, g.nz - z0);
     const uint64_t base = z0 * g.nxy + y0 * g.nx + x0;
-    const bool hx = x0 + kTX < g.nx, hy = y0 + kTY < g.ny, hz = z0 + kTZ < g.nz;
+    const uint32_t e = threadIdx.x, c1 = e % kSide, c2 = e / kSide, lane = threadIdx.x & 31;
+    // the ends of edge (c1, c2) of face dir (0, 1, 2: +x, +y, +z)
+    auto ends = [&](uint32_t dir, uint32_t p, uint32_t q, uint64_t &a, uint64_t &b) {
+        if (dir == 0) a = base + q * g.nxy + p * g.nx + (kSide - 1), b = a + 1;
+        else if (dir == 1) a = base + q * g.nxy + (kSide - 1) * g.nx + p, b = a + g.nx;
+        else a = base + (kSide - 1) * g.nxy + q * g.nx + p, b = a + g.nxy;
+    };
+    if (threadIdx.x == 0) s_n = 0;
+    uint64_t mine[3];
+#pragma unroll
+    for (uint32_t dir = 0; dir < 3; dir++) {
+        const bool has = dir == 0 ? x0 + kSide < g.nx : dir == 1 ? y0 + kSide < g.ny : z0 + kSide < g.nz;
+        mine[dir] = ~0ull;
+        if (has && c1 < (dir == 0 ? wy : wx) && c2 < (dir == 2 ? wy : wz)) {
+            uint64_t a, b;
+            ends(dir, c1, c2, a, b);
+            const float fa = f[a], fb = f[b];
+            const uint32_t side = before_w(fa, a, fb, b);  // 1: b is the later end
+            const float fs = side ? fb : fa;
+            const uint32_t bits = fs == 0.0f ? 0u : __float_as_uint(fs);
+            const uint32_t key = (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
+            const uint32_t pos = dir == 0 ? 2 * e + side : dir == 1 ? c2 * 2 * kSide + side * kSide + c1 : side * F + e;
+            mine[dir] = (uint64_t)key << 32 | pos;
+        }
+        lev[dir][e] = mine[dir];
+    }
+    __syncthreads();
+#pragma unroll
+    for (uint32_t dir = 0; dir < 3; dir++) {
+        const uint64_t v = mine[dir], *p = &lev[dir][e];
+        const bool keep = v != ~0ull && !((c1 > 0 && p[-1] < v) || (c1 + 1 < kSide && p[1] < v) ||
+                                          (c2 > 0 && *(p - kSide) < v) || (c2 + 1 < kSide && p[kSide] < v));
+        const uint32_t bal = __ballot_sync(0xffffffffu, keep);
+        uint32_t pos = 0;
+        if (lane == 0) pos = atomicAdd(&s_n, __popc(bal));
+        pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(bal & ((1u << lane) - 1u));
+        if (keep) list[pos] = (uint16_t)(dir * F + e);
+    }
+    __syncthreads();
     bool ok = true;
-    for (uint32_t e = threadIdx.x; e < FH; e += blockDim.x) {
+    for (uint32_t i = threadIdx.x; i < s_n; i += blockDim.x) {
+        const uint32_t en = list[i], dir = en / F, ee = en % F;
         uint64_t a, b;
-        if (e < FX) {
-            const uint64_t ly = e % kTY, lz = e / kTY;
-            if (!hx || ly >= wy || lz >= wz) continue;
-            a = base + lz * g.nxy + ly * g.nx + (kTX - 1);
-            b = a + 1;
-        } else if (e < FX + FY) {
-            const uint64_t k = e - FX, lx = k % kTX, lz = k / kTX;
-            if (!hy || lx >= wx || lz >= wz) continue;
-            a = base + lz * g.nxy + (kTY - 1) * g.nx + lx;
-            b = a + g.nx;
-        } else {
-            const uint64_t k = e - FX - FY, lx = k % kTX, ly = k / kTX;
-            if (!hz || lx >= wx || ly >= wy) continue;
-            a = base + (kTZ - 1) * g.nxy + ly * g.nx + lx;
-            b = a + g.nxy;
-        }
+        ends(dir, ee % kSide, ee / kSide, a, b);
         const uint64_t S = before_w(f[a], a, f[b], b) ? b : a;
-        ok &= M.merge(S, a, b);
-    }
-    if (!ok) raise_status(status, ST_TIMEOUT);
-}
-
-// ---------------------------------------------------------------- repair
-// Representative (Algorithm 4) at level S: hop while the link's saddle is at
-// or below S in the order; return the vertex where the walk stops. Concurrent
-// repairs only move a word's target further along its own chain below the
-// same saddle, so either half may be old or new. The next word is read
-// beside the saddle's value, before the test that decides whether it is
-// needed (the target of a link is a vertex of the grid, so the read stays in
-// bounds); the same in the climbs of the merges, whose reads repeat until
-// both halves carry one tag, measured slower.
-__device__ __forceinline__ uint64_t w_rep(const uint64_t *W, const FieldW &f, uint64_t x, uint64_t S, float fS,
-                                          uint32_t &steps)
-{
-    uint64_t lo, hi;
-    ld_word(W, x, lo, hi);
-    for (;;) {
-        const uint64_t s = lo & kIdMask, v = hi & kIdMask;
-        if (s == x && v == x) return x;
-        const float fs = f[s];
-        uint64_t nlo, nhi;
-        ld_word(W, v, nlo, nhi);
-        if (s != S && !before_w(fs, s, fS, S)) return x;
-        x = v, lo = nlo, hi = nhi;
-        if (++steps > kChaseLimit) return x;
-    }
-}
-
-__global__ void __launch_bounds__(kWThreads) k_w_repair(FieldW f, Geo g, uint64_t *W, uint32_t *status)
-{
-    if (*status) return;
-    bool ok = true;
-    for (uint64_t u = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; u < g.n; u += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t lo, hi;
-        ld_word(W, u, lo, hi);
-        const uint64_t s = lo & kIdMask, v = hi & kIdMask;
-        uint64_t r = v;
-        if (!(s == u && v == u)) {
-            uint32_t steps = 0;
-            // a minimum: its target at its saddle s; an inner vertex: at u itself
-            r = w_rep(W, f, v, s, f[s], steps);
-            if (steps > kChaseLimit) {
-                ok = false;
-                continue;
-            }
-        }
-        if (r != v || lo != s || hi != v)
-            asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(W + 2 * u), "l"(s), "l"(r) : "memory");
+        // climbs start at the tile minima the ends descend to
+        auto start = [&](uint64_t u, uint64_t tbase) -> uint64_t {
+            uint64_t lo, hi;
+            ld_word(W, u, lo, hi);
+            if ((lo & kIdMask) != kInner) return u;
+            const uint32_t l = (uint32_t)hi;
+            return tbase + (uint64_t)(l / F) * g.nxy + (uint64_t)(l / kSide % kSide) * g.nx + l % kSide;
+        };
+        const uint64_t step = dir == 0 ? kSide : dir == 1 ? kSide * g.nx : kSide * g.nxy;
+        ok &= M.merge(S, start(a, base), start(b, base + step));
     }
     if (!ok) raise_status(status, ST_TIMEOUT);
 }
@@ -434,7 +432,7 @@ size_t mt_wide_workspace_bytes(mt_grid g)
 {
     Geo geo;
     if (wide_grid(g, geo) != MT_OK) return 0;
-    return wide_ws_bytes(geo.n);
+    return wide_ws_bytes(geo);
 }
 
 mt_status mt_build_triplets_wide(const float *d_f, mt_grid g, uint64_t *d_W, void *d_ws, size_t ws_bytes,
@@ -446,16 +444,17 @@ mt_status mt_build_triplets_wide(const float *d_f, mt_grid g, uint64_t *d_W, voi
     if (!d_f || !d_W || ((uintptr_t)d_f & 3) || ((uintptr_t)d_W & 15) || (flags & ~MT_SUPERLEVEL))
         return MT_ERR_INVALID;
     WideWs ws;
-    if (!carve(d_ws, ws_bytes, geo.n, ws)) return MT_ERR_INVALID;
+    if (!carve(d_ws, ws_bytes, geo, ws)) return MT_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const float sg = (flags & MT_SUPERLEVEL) ? -1.0f : 1.0f;
     const FieldW f{d_f, sg};
     if (cudaMemsetAsync(ws.status, 0, 512, s) != cudaSuccess) return MT_ERR_CUDA;
     {
         PhaseScope ps(kTile, s);
-        if (launch_tile_wide(d_f, d_W, g.nx, g.ny, g.nz, sg, ws.status, s) != cudaSuccess) return MT_ERR_CUDA;
+        if (launch_tile_wide(d_f, d_W, ws.notes, g.nx, g.ny, g.nz, sg, ws.status, s) != cudaSuccess) return MT_ERR_CUDA;
     }
-    const uint32_t ntx = (g.nx + kTX - 1) / kTX, nty = (g.ny + kTY - 1) / kTY, ntz = (g.nz + kTZ - 1) / kTZ;
+    const uint32_t ntx = (uint32_t)((geo.nx + kSide - 1) / kSide), nty = (uint32_t)((geo.ny + kSide - 1) / kSide),
+                   ntz = (uint32_t)((geo.nz + kSide - 1) / kSide);
     {
         PhaseScope ps(kMerge, s);
         k_w_cross<<<ntx * nty * ntz, 256, 0, s>>>(f, geo, ntx, nty, d_W, ws.status);
@@ -463,8 +462,7 @@ mt_status mt_build_triplets_wide(const float *d_f, mt_grid g, uint64_t *d_W, voi
     }
     {
         PhaseScope ps(kRepair, s);
-        k_w_repair<<<grid_for(geo.n), kWThreads, 0, s>>>(f, geo, d_W, ws.status);
-        count_launch();
+        if (launch_repair_wide(d_f, d_W, ws.notes, g.nx, g.ny, g.nz, sg, ws.status, s) != cudaSuccess) return MT_ERR_CUDA;
     }
     return cudaGetLastError() == cudaSuccess ? MT_OK : MT_ERR_CUDA;
 }
@@ -478,7 +476,7 @@ mt_status mt_persistence_pairs_wide(const uint64_t *d_W, mt_grid g, uint64_t *d_
     if (!d_W || !h_npairs || ((uintptr_t)d_W & 15) || (cap && (!d_pairs || ((uintptr_t)d_pairs & 7))))
         return MT_ERR_INVALID;
     WideWs ws;
-    if (!carve(d_ws, ws_bytes, geo.n, ws)) return MT_ERR_INVALID;
+    if (!carve(d_ws, ws_bytes, geo, ws)) return MT_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(ws.meta, 0, 3 * sizeof(uint64_t), s) != cudaSuccess) return MT_ERR_CUDA;
     {
@@ -510,7 +508,7 @@ mt_status mt_components_at_wide(const float *d_f, const uint64_t *d_W, mt_grid g
         ((uintptr_t)d_labels & 7) || (flags & ~MT_SUPERLEVEL))
         return MT_ERR_INVALID;
     WideWs ws;
-    if (!carve(d_ws, ws_bytes, geo.n, ws)) return MT_ERR_INVALID;
+    if (!carve(d_ws, ws_bytes, geo, ws)) return MT_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const float sg = (flags & MT_SUPERLEVEL) ? -1.0f : 1.0f;
     PhaseScope ps(kLabels, s);
