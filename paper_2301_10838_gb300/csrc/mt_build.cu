@@ -653,17 +653,33 @@ __global__ void __launch_bounds__(Tile<LX, LY, LZ>::NT, Tile<LX, LY, LZ>::kCTAs)
 // left the edges that can matter (the local minima of the level over each
 // face), in the same order in the records of both tiles: the level S, and for
 // each end its tile-local top at S (the deepest vertex of its tile component
-// below S), where the merge's climbs start. The kernel is bound by the latency
-// of those climbs: 6.3 ms for the 132 edges per tile of the 1024^3 lognormal
-// field (6.4 ms when the CTA read all 768 edges of its faces and found those
-// to merge in a hash of the pairs of tops).
+// below S), where the merge's climbs start. Edges with the same pair of tops
+// join the same two tile components, so only the one with the earliest level
+// of each pair is merged (a shared-memory hash with 64-bit atomicMin): about
+// 93 of the 132 edges per tile on a lognormal field.
+//
+// The kernel is bound by the latency of its chains of dependent reads (a
+// quarter of the issue slots used, HBM 12 % busy): 4.8 ms on the 1024^3
+// lognormal field; 6.3 ms with a merge that read a vertex's value and a
+// re-inserted link's level only when it needed them, and without the hash;
+// 5.6 ms with the new merge alone. The fields of a batch are small enough
+// for L2, where the hash costs more than the merges it saves (512 uneven
+// fields: 0.36 ms with it, 0.29 without), and 16 CTAs per SM run better than
+// the 12 that hide most of HBM's latency (0.39 ms with 11 CTAs, 0.29 with 16;
+// single field 4.8 ms with 12, 5.2 with 14).
 template <int LX, int LY, int LZ, class Loc>
-__global__ void __launch_bounds__(128) k_cross(Loc loc, uint32_t *status)
+__global__ void __launch_bounds__(128, std::is_same<Loc, OneField>::value ? 12 : 16) k_cross(Loc loc, uint32_t *status)
 {
     if (block_skips(status)) return;
     using TS = Tile<LX, LY, LZ>;
-    constexpr uint32_t G = TS::G, GX = TS::FX / 32, GY = TS::FY / 32;
-    __shared__ uint32_t off[65];  // first edge of each group
+    constexpr uint32_t G = TS::G, GX = TS::FX / 32, GY = TS::FY / 32, NT = 128;
+    constexpr uint32_t HS = 16 * G > 512 ? 1024 : 512;  // slots for at most 16 edges per group
+    static_assert(16 * G <= HS, "the hash holds every edge");
+    constexpr unsigned long long EMPTY = ~0ull;
+    __shared__ unsigned long long hkey[HS], hlev[HS];  // pair of tops; (key, id) of the earliest level
+    __shared__ uint32_t off[65];                       // first edge of each group
+    __shared__ uint16_t list[HS];
+    __shared__ uint32_t s_n;
     uint32_t tile;
     const FieldDesc fd = loc.tile(blockIdx.x, tile);
     const Field f{fd.f, fd.sg};
@@ -679,11 +695,14 @@ __global__ void __launch_bounds__(128) k_cross(Loc loc, uint32_t *status)
             if (threadIdx.x >= (uint32_t)o) incl += y;
         }
         off[g] = incl - c0 - c1, off[g + 1] = incl - c1;
-        if (threadIdx.x == 31) off[64] = incl;
+        if (threadIdx.x == 31) off[64] = incl, s_n = 0;
     }
+    constexpr bool DEDUP = std::is_same<Loc, OneField>::value;  // see above
+    if (DEDUP)
+        for (uint32_t i = threadIdx.x; i < HS; i += NT) hkey[i] = EMPTY, hlev[i] = EMPTY;
     __syncthreads();
     bool ok = true;
-    for (uint32_t i = threadIdx.x; i < off[64]; i += blockDim.x) {
+    for (uint32_t i = threadIdx.x; i < off[64]; i += NT) {
         uint32_t g = 0;  // the last group whose first edge is at or before i
 #pragma unroll
         for (uint32_t w = 32; w > 0; w >>= 1)
@@ -692,7 +711,29 @@ __global__ void __launch_bounds__(128) k_cross(Loc loc, uint32_t *status)
         const uint32_t nb = g < GX ? 1u : g < GX + GY ? fd.ntx : fd.ntx * fd.nty;  // the neighbour tile
         const uint32_t ta = rec[TS::kFaceHead + p], S = rec[TS::kFaceHead + 2 * TS::kFaceSide + p];
         const uint32_t tb = rec[(size_t)nb * kWords + TS::kFaceHead + TS::kFaceSide + p];
-        ok &= merge(fd.W, f, S, ta, tb);
+        if (!DEDUP) {
+            ok &= merge(fd.W, f, S, f[S], ta, tb);
+            continue;
+        }
+        const unsigned long long key = (unsigned long long)ta << 32 | tb,
+                                 lev = (unsigned long long)order_key(f[S]) << 32 | S;
+        uint32_t h = (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> 54) & (HS - 1);
+        for (uint32_t q = 0; q < HS; q++) {
+            const unsigned long long k0 = atomicCAS(&hkey[h], EMPTY, key);
+            if (k0 == EMPTY) list[atomicAdd(&s_n, 1u)] = (uint16_t)h;
+            if (k0 == EMPTY || k0 == key) {
+                atomicMin(&hlev[h], lev);
+                break;
+            }
+            h = (h + 1) & (HS - 1);
+        }
+    }
+    if (DEDUP) __syncthreads();
+    for (uint32_t j = threadIdx.x; DEDUP && j < s_n; j += NT) {
+        const uint32_t h = list[j], kS = (uint32_t)(hlev[h] >> 32);
+        // the value with order key kS
+        const float fS = __uint_as_float((kS & 0x80000000u) ? kS ^ 0x80000000u : ~kS);
+        ok &= merge(fd.W, f, (uint32_t)hlev[h], fS, (uint32_t)(hkey[h] >> 32), (uint32_t)hkey[h]);
     }
     if (!ok) raise_status(status, ST_TIMEOUT);
 }
@@ -803,7 +844,10 @@ struct RepairShape {
     static constexpr size_t kSmem = (size_t)(kNodes + 4) * 8 + (size_t)kNodes * (LAB || WIDE ? 8 : 4) +
                                     (size_t)kHash * (WIDE ? 8 : 4) + (size_t)TV / 2 * 2 + (size_t)kHash * 2;
     static constexpr int kFit = (int)(227 * 1024 / (kSmem + 1024));
-    static constexpr int kCTAs = kFit < (int)(1536 / NT) ? kFit : (int)(1536 / NT);
+    // CTAs per SM the registers are limited for: 7 of 256 threads (36
+    // registers) take 8.4 ms without labels on the 1024^3 field, 6 take 9.7;
+    // with labels 6 (40 registers) take 10.8 ms and 7 take 11.0
+    static constexpr int kWant = (LAB || WIDE ? 1536 : 1792) / NT, kCTAs = kFit < kWant ? kFit : kWant;
 };
 
 template <int LX, int LY, int LZ, class Loc, bool LAB, bool WIDE = false>
@@ -1245,13 +1289,11 @@ static cudaError_t launch_repair(const Loc &loc, uint32_t ntiles, uint32_t *stat
     return cudaGetLastError();
 }
 
-// Build steps with tile variant V and the knobs of cfg (MT_CFG_* bits of
-// include/mt.h): the CTA size of the repair kernel (MT_CFG_FOUR_ROUNDS chooses
-// nothing: the tile kernel has no rounds). Every configuration gives the same
-// triplets.
+// Build steps with tile variant V (of the knobs in include/mt.h the tile shapes
+// alone choose anything).
 template <int V, class Loc>
 static cudaError_t run_build(const Loc &loc, uint32_t ntiles, uint32_t *queue, int persistent_grid, uint32_t *status,
-                             cudaStream_t st, uint32_t cfg, const LabelArgs *la = nullptr)
+                             cudaStream_t st, const LabelArgs *la = nullptr)
 {
     using VV = Variant<V>;
     cudaError_t e;
@@ -1275,7 +1317,7 @@ static cudaError_t run_build(const Loc &loc, uint32_t ntiles, uint32_t *queue, i
 // A single field in the tile shape of variant V (0, or 2 with MT_CFG_LARGE_TILES).
 template <int V>
 static cudaError_t build_one(const float *f, uint64_t *W, uint32_t nx, uint32_t ny, uint32_t nz, Workspace &ws,
-                             uint32_t *faces, float sg, cudaStream_t st, uint32_t cfg, const LabelArgs *la)
+                             uint32_t *faces, float sg, cudaStream_t st, const LabelArgs *la)
 {
     using VV = Variant<V>;
     OneField loc;
@@ -1290,14 +1332,14 @@ static cudaError_t build_one(const float *f, uint64_t *W, uint32_t nx, uint32_t 
     loc.d.nty = (ny + (1u << VV::LY) - 1) >> VV::LY;
     const uint32_t ntz = (nz + (1u << VV::LZ) - 1) >> VV::LZ;
     const uint64_t ntiles = (uint64_t)loc.d.ntx * loc.d.nty * ntz;
-    return run_build<V>(loc, (uint32_t)ntiles, nullptr, 0, ws.status, st, cfg, la);
+    return run_build<V>(loc, (uint32_t)ntiles, nullptr, 0, ws.status, st, la);
 }
 
 cudaError_t launch_build(const float *f, uint64_t *W, uint32_t nx, uint32_t ny, uint32_t nz, Workspace &ws,
                          uint32_t *faces, float sg, cudaStream_t st, uint32_t cfg, const LabelArgs *la)
 {
-    if (cfg & MT_CFG_LARGE_TILES) return build_one<2>(f, W, nx, ny, nz, ws, faces, sg, st, cfg, la);
-    return build_one<0>(f, W, nx, ny, nz, ws, faces, sg, st, cfg, la);
+    if (cfg & MT_CFG_LARGE_TILES) return build_one<2>(f, W, nx, ny, nz, ws, faces, sg, st, la);
+    return build_one<0>(f, W, nx, ny, nz, ws, faces, sg, st, la);
 }
 
 // The tile kernel and the repair pass with 64-bit ids and 128-bit words (the
@@ -1349,8 +1391,8 @@ cudaError_t launch_batch_build(const FieldDesc *d_descs, uint32_t nfields, uint3
     const bool small = cfg & MT_CFG_SMALL_TILES;
     const int per_sm = small ? TileOf<1>::kCTAs : TileOf<0>::kCTAs;
     const int grid = device_sms() * per_sm;
-    if (small) return run_build<1>(loc, ntiles, queue, grid, status, st, cfg);
-    return run_build<0>(loc, ntiles, queue, grid, status, st, cfg);
+    if (small) return run_build<1>(loc, ntiles, queue, grid, status, st);
+    return run_build<0>(loc, ntiles, queue, grid, status, st);
 }
 
 }  // namespace mt

@@ -85,39 +85,11 @@ struct Field {
     __device__ __forceinline__ float operator[](uint32_t i) const { return sg * __ldg(f + i); }
 };
 
-// Climbs (Algorithm 3): follow the triplet links from a vertex while the
-// link's saddle is at or below level S (vertex order), i.e. walk to the
-// deepest vertex that the current tree connects to it below S. A root word
-// (x, x) always stops a walk (the paper's pseudocode has no guard for it).
-// Both climbs of a merge side by side, so that their loads overlap: each
-// round reads, for every walk still going, its saddle's value and (before the
-// level test) its next vertex's word.
-__device__ __forceinline__ void climb2(const uint64_t *W, const Field f, uint32_t &u, uint32_t &v, uint32_t S,
-                                       float fS, uint64_t &Tu, uint64_t &Tv, uint32_t &steps)
-{
-    Tu = ld_tri(W + u);
-    Tv = ld_tri(W + v);
-    bool du = false, dv = false;
-    for (;;) {
-        const uint32_t su = tri_s(Tu), tu = tri_v(Tu), sv = tri_s(Tv), tv = tri_v(Tv);
-        du = du || (su == u && tu == u);
-        dv = dv || (sv == v && tv == v);
-        float fsu = 0.0f, fsv = 0.0f;
-        uint64_t Tnu = 0, Tnv = 0;
-        if (!du) fsu = f[su], Tnu = ld_tri(W + tu);
-        if (!dv) fsv = f[sv], Tnv = ld_tri(W + tv);
-        du = du || (su != S && !before(fsu, su, fS, S));
-        dv = dv || (sv != S && !before(fsv, sv, fS, S));
-        if (du && dv) return;
-        if (!du) u = tu, Tu = Tnu;
-        if (!dv) v = tv, Tv = Tnv;
-        if (++steps > kMergeStepLimit) return;
-    }
-}
-
-// Algorithm 3 (Merge), lock-free: make a and b connected at level S in the
-// triplet forest, given that they are connected below S in the graph.
-//   1. climb a and b to their deepest vertices u, v below S;
+// Algorithm 3 (Merge), lock-free: make a and b connected at level S (value fS)
+// in the triplet forest, given that they are connected below S in the graph.
+//   1. climb a and b to their deepest vertices u, v below S: follow links
+//      while their saddle is at or below S in the vertex order (a root word
+//      (x, x) always stops a walk; the paper's pseudocode has no guard for it);
 //   2. if they coincide the edge adds nothing;
 //   3. otherwise order them so that u comes first and swing v's link to
 //      (S, u) with one 64-bit CAS (Algorithm 2);
@@ -125,61 +97,48 @@ __device__ __forceinline__ void climb2(const uint64_t *W, const Field f, uint32_
 //      root, continue by merging u and tv at level sv. (A displaced root
 //      carries no link, so the merge ends there.)
 //   5. if the CAS fails another thread moved v first: climb again.
+// A merge is a chain of dependent reads, so everything a step may need is
+// read with the step before it: both climbs advance side by side, a vertex's
+// own value (to order u and v) is read beside its word, a link's saddle
+// value beside the next vertex's word and value, and the displaced link's
+// saddle value is the one its level test has read.
 // Returns false if the step budget ran out.
-__device__ __forceinline__ bool merge(uint64_t *W, const Field f, uint32_t S, uint32_t a, uint32_t b)
+__device__ __forceinline__ bool merge(uint64_t *W, const Field f, uint32_t S, float fS, uint32_t a, uint32_t b)
 {
-    float fS = f[S];
     uint32_t u = a, v = b;
-    uint32_t steps = 0;
-    for (;;) {
-        uint64_t Tu, Tv;
-        climb2(W, f, u, v, S, fS, Tu, Tv, steps);
-        if (++steps > kMergeStepLimit) return false;
+    uint64_t Tu = ld_tri(W + u), Tv = ld_tri(W + v);
+    float fu = f[u], fv = f[v];
+    for (uint32_t steps = 0; steps < kMergeStepLimit; steps++) {
         if (u == v) return true;
-        if (before(f[v], v, f[u], u)) {
-            uint32_t tx = u;
-            u = v;
-            v = tx;
-            uint64_t tT = Tu;
-            Tu = Tv;
-            Tv = tT;
+        const uint32_t su = tri_s(Tu), tu = tri_v(Tu), sv = tri_s(Tv), tv = tri_v(Tv);
+        const bool ru = su == u && tu == u, rv = sv == v && tv == v;
+        // saddle values, and the words and values behind the links (a root's
+        // lead to itself)
+        const float fsu = f[su], fsv = f[sv], ftu = f[tu], ftv = f[tv];
+        const uint64_t Tnu = ld_tri(W + tu), Tnv = ld_tri(W + tv);
+        const bool mu = !ru && (su == S || before(fsu, su, fS, S)), mv = !rv && (sv == S || before(fsv, sv, fS, S));
+        if (mu || mv) {
+            if (mu) u = tu, Tu = Tnu, fu = ftu;
+            if (mv) v = tv, Tv = Tnv, fv = ftv;
+            continue;
         }
-        const uint64_t old = cas_tri(W + v, Tv, tri_pack(S, u));
-        if (old == Tv) {
-            const uint32_t sv = tri_s(Tv), tv = tri_v(Tv);
-            if (sv == v && tv == v) return true;  // displaced a root
-            S = sv;
-            fS = f[sv];
-            v = tv;
+        const bool sw = before(fv, v, fu, u);  // v is the earlier one: link u under it
+        const uint32_t lo = sw ? v : u, hi = sw ? u : v;
+        const uint64_t Thi = sw ? Tu : Tv;
+        const uint64_t old = cas_tri(W + hi, Thi, tri_pack(S, lo));
+        if (old == Thi) {
+            if (sw ? ru : rv) return true;  // displaced a root
+            // go on with the link that hi held: merge lo and its target there
+            S = sw ? su : sv, fS = sw ? fsu : fsv;
+            if (sw) u = tu, Tu = Tnu, fu = ftu;
+            else v = tv, Tv = Tnv, fv = ftv;
+        } else if (sw) {
+            Tu = old;
+        } else {
+            Tv = old;
         }
     }
-}
-
-// Representative (Algorithm 4) of x at level S given as a vertex: the deepest
-// vertex of x's component below S. Hops while the link's saddle s' satisfies
-// s' <= S in the vertex order and returns the vertex where it stops (the
-// printed algorithm returns one hop further; the vertex itself is the one
-// the definition asks for). Ordinary (L1-cacheable) loads: it serves passes
-// in which the entries only ever move further along their own chains
-// (repair), where a stale copy still leads to the same representative. The
-// triplet of the next vertex is loaded together with the value of the
-// current saddle, before the level test decides whether it is needed, so that
-// a hop costs one memory latency instead of two (the extra load reads a valid
-// entry either way).
-__device__ __forceinline__ uint32_t representative_cached(const uint64_t *W, const Field f, uint32_t x, uint32_t S,
-                                                          float fS, uint32_t &steps)
-{
-    uint64_t T = W[x];
-    for (;;) {
-        const uint32_t s = tri_s(T), t = tri_v(T);
-        if (s == x && t == x) return x;
-        const float fs = f[s];
-        const uint64_t Tn = W[t];
-        if (s != S && !before(fs, s, fS, S)) return x;
-        x = t;
-        T = Tn;
-        if (++steps > kChaseLimit) return x;
-    }
+    return false;
 }
 
 }  // namespace mt
