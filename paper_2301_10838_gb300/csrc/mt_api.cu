@@ -45,6 +45,10 @@ bool carve_workspace(void *base, size_t bytes, uint64_t n, Workspace &ws)
     ws.meta = reinterpret_cast<uint64_t *>(p + 256);
     ws.counts = reinterpret_cast<uint32_t *>(p + 512);
     ws.nchunks = (n + kCompactChunk - 1) / kCompactChunk;
+    // the pair compaction's bits take the place of the build's tile records,
+    // which are done with by then, if the workspace has room for them
+    const size_t need = workspace_bytes(n) + ws.nchunks * (kCompactChunk / 8);
+    ws.mask = bytes >= need ? reinterpret_cast<uint32_t *>(p + workspace_bytes(n)) : nullptr;
     return true;
 }
 

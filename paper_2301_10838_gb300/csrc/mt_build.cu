@@ -187,35 +187,6 @@ __device__ __noinline__ bool sm_merge_rare(uint64_t *L, const uint32_t *K, const
     return false;
 }
 
-// A triplet in global memory: one 64-bit word of two 32-bit ids, or (WIDE) two
-// 64-bit words whose ids carry the merges' tags in their upper 30 bits.
-template <bool WIDE>
-struct Tri {
-    using Id = typename std::conditional<WIDE, uint64_t, uint32_t>::type;
-    static constexpr uint64_t kMask = (1ull << 34) - 1;
-    // saddle id of the word of a tile's inner vertex between the tile kernel
-    // and the repair pass; the word's other id is then the local id of
-    // the tile minimum the vertex descends to (no merge reads such words:
-    // every target of a link is a minimum of its tile)
-    static constexpr Id kInner = WIDE ? (Id)kMask : (Id)0xFFFFFFFFu;
-    static __device__ __forceinline__ void load(const uint64_t *W, Id u, Id &s, Id &v)
-    {
-        if constexpr (WIDE) {
-            const ulonglong2 w = reinterpret_cast<const ulonglong2 *>(W)[u];
-            s = w.x & kMask, v = w.y & kMask;
-        } else {
-            const uint64_t w = W[u];
-            s = tri_s(w), v = tri_v(w);
-        }
-    }
-    static __device__ __forceinline__ void store(uint64_t *W, Id u, Id s, Id v)
-    {
-        if constexpr (WIDE)
-            asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(W + 2 * u), "l"(s), "l"(v) : "memory");
-        else st_tri(W + u, tri_pack(s, v));
-    }
-};
-
 // WIDE: the triplets leave the tile as 128-bit words of two 64-bit ids
 // (W[2u] = s, W[2u + 1] = v) for grids of 2^32 vertices and more; the work
 // inside the tile, on 16-bit local ids, is the same, and no face record is
@@ -1140,7 +1111,7 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
 
     // 4. inner vertices, the next row's value and word loaded ahead (rows
     //    unrolled by 4 or 8 with their loads first measured slower: the
-    //    kernel then waits for instructions)
+    //    kernel then waits for instructions; two rows ahead: no faster)
     uint32_t lost = 0;                             // bit z: the climb left the forest
     auto row = [&](uint32_t z, float &fu, uint32_t &m) {
         const bool in = inx && z < wz, inner = in && !((minima >> z) & 1u);

@@ -6,6 +6,7 @@
 // Order:         a < b  <=>  f[a] < f[b] || (f[a] == f[b] && a < b).
 #pragma once
 #include <cstdint>
+#include <type_traits>
 
 namespace mt {
 
@@ -25,11 +26,11 @@ enum : uint32_t {
 #ifdef MT_STRESS_TABLES
 constexpr int kTileListShrink = 64;       // k_tile: edge list 64x smaller
 constexpr uint32_t kRepairShrink = 64;    // k_repair: hash, copies and minima list 64x smaller
-constexpr uint32_t kLabelHashLog = 6;     // k_labels: 64 chain starts per brick
+constexpr uint32_t kLabelShrink = 64;     // k_labels: hash of chain starts 64x smaller
 #else
 constexpr int kTileListShrink = 1;
 constexpr uint32_t kRepairShrink = 1;
-constexpr uint32_t kLabelHashLog = 12;    // 4096 chain starts per brick
+constexpr uint32_t kLabelShrink = 1;
 #endif
 
 // Limits of the bounded device loops. A merge that needs more steps than this
@@ -75,6 +76,35 @@ __device__ __forceinline__ bool block_skips(const uint32_t *status)
 {
     return __syncthreads_or(threadIdx.x == 0 && *(const volatile uint32_t *)status != 0) != 0;
 }
+
+// A triplet in global memory: one 64-bit word of two 32-bit ids, or (WIDE) two
+// 64-bit words whose ids carry the merges' tags in their upper 30 bits.
+template <bool WIDE>
+struct Tri {
+    using Id = typename std::conditional<WIDE, uint64_t, uint32_t>::type;
+    static constexpr uint64_t kMask = (1ull << 34) - 1;
+    // saddle id of the word of a tile's inner vertex between the tile kernel
+    // and the repair pass; the word's other id is then the local id of
+    // the tile minimum the vertex descends to (no merge reads such words:
+    // every target of a link is a minimum of its tile)
+    static constexpr Id kInner = WIDE ? (Id)kMask : (Id)0xFFFFFFFFu;
+    static __device__ __forceinline__ void load(const uint64_t *W, Id u, Id &s, Id &v)
+    {
+        if constexpr (WIDE) {
+            const ulonglong2 w = reinterpret_cast<const ulonglong2 *>(W)[u];
+            s = w.x & kMask, v = w.y & kMask;
+        } else {
+            const uint64_t w = W[u];
+            s = tri_s(w), v = tri_v(w);
+        }
+    }
+    static __device__ __forceinline__ void store(uint64_t *W, Id u, Id s, Id v)
+    {
+        if constexpr (WIDE)
+            asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(W + 2 * u), "l"(s), "l"(v) : "memory");
+        else st_tri(W + u, tri_pack(s, v));
+    }
+};
 
 // The values as the order sees them: f itself (sublevel sets), or -f (sg =
 // -1) for the tree of the superlevel sets, the split tree. Multiplying by -1

@@ -44,6 +44,7 @@ struct Workspace {
     uint64_t *meta;    // [0] npairs, [1] number of roots, [2] root
     uint32_t *faces;   // per tile: tile-local tops of the cross-edge ends, or null vertex
     uint32_t *counts;  // per-chunk counts, then exclusive offsets in place
+    uint32_t *mask;    // a bit per vertex for the pair compaction, or null
     uint64_t nchunks;
 };
 
@@ -127,5 +128,8 @@ cudaError_t launch_batch_pairs(const FieldDesc *d_descs, uint32_t nfields, uint6
 void tile_shape(int variant, uint32_t &tx, uint32_t &ty, uint32_t &tz);
 cudaError_t launch_labels(const float *f, const uint64_t *W, uint32_t nx, uint32_t ny, uint32_t nz, float t,
                           float sg, uint32_t *labels, Workspace &ws, cudaStream_t st, float eps = 0.0f);
+
+cudaError_t launch_labels_wide(const float *f, const uint64_t *W2, uint32_t nx, uint32_t ny, uint32_t nz, float t,
+                               float sg, uint64_t *labels, uint32_t *status, cudaStream_t st);
 
 }  // namespace mt

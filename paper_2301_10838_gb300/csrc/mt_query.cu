@@ -18,30 +18,60 @@ namespace mt {
 // owns the contiguous slice [w * 512, (w + 1) * 512) of the chunk and reads it
 // in 16 coalesced rows of 32. A pass counts the pairs of each chunk (and finds
 // the roots), a scan per field turns the counts into offsets, and a second
-// pass writes each chunk's pairs at its offset in order: every warp keeps its
-// 16 triplets in registers, ranks its flags with ballots, and one barrier
-// combines the 8 warp totals, which keeps the ascending order.
+// pass writes each chunk's pairs at its offset in order: every warp ranks its
+// flags with ballots, and one barrier combines the 8 warp totals, which keeps
+// the ascending order.
+//
+// Both passes are bound by HBM, so the first one leaves a bit per vertex
+// (`mask`, 1/64 of the triplets' size, where the caller has the room) and the
+// second reads the triplets of pairs only, one vertex in ten on a lognormal
+// field: 2.8 -> 2.7 ms at 1024^3, 68 -> 61 us at 256^3. With a persistence to
+// keep (eps > 0) it also saves reading f at the saddles a second time, and
+// those reads are issued for eight rows at a time: 585 -> 256 us at 400^3. A
+// batch's fields mostly stay in L2 between the passes, where the bits cost
+// more than they save (512 uneven fields: 345 us with them, 325 without).
 constexpr int kCompactThreads = 256;
-
-// Persistence simplification (SIMP): the pair (u, s) of a branch minimum u is
-// kept when its persistence f(s) - f(u), computed in float32 on the values
-// the order sees (sg * f), is at least eps. Without SIMP every pair is kept
-// and f is not read (a separate instantiation, so that the plain kernels
-// keep their loads of all rows ahead of any use).
-template <bool SIMP>
-__device__ __forceinline__ bool keep_pair(const FieldDesc &fd, uint64_t T, uint32_t u, float eps)
-{
-    if (tri_s(T) == u) return false;
-    if (!SIMP) return true;
-    const float fu = fd.sg * __ldg(fd.f + u), fs = fd.sg * __ldg(fd.f + tri_s(T));
-    return fs - fu >= eps;
-}
 constexpr int kCompactWarps = kCompactThreads / 32;
 constexpr int kCompactRows = kCompactChunk / kCompactThreads;  // rows of 32 per warp
 static_assert(kCompactRows * 32 * kCompactWarps == kCompactChunk, "chunk = warps x rows x 32");
+static_assert(kCompactRows <= 32, "a lane per row holds the row's mask");
+
+// Which of the vertices u0 + 32 r + lane with triplets T[r] begin a pair: bit
+// r of the result. Persistence simplification (SIMP): the pair (u, s) of a
+// branch minimum u is kept when its persistence f(s) - f(u), computed in
+// float32 on the values the order sees (sg * f), is at least eps; the values
+// of a few rows are read together, without a branch between them. Without SIMP
+// every pair is kept and f is not read.
+template <bool SIMP>
+__device__ __forceinline__ uint32_t keep_rows(const FieldDesc &fd, const uint64_t *T, uint64_t u0, float eps)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t keep = 0;
+    constexpr int RB = SIMP ? 8 : kCompactRows;
+#pragma unroll
+    for (int q = 0; q < kCompactRows; q += RB) {
+        float fu[RB], fs[RB];
+        if (SIMP) {
+#pragma unroll
+            for (int r = 0; r < RB; r++) {
+                const uint32_t u = (uint32_t)(u0 + (q + r) * 32 + lane), s = tri_s(T[q + r]);
+                fu[r] = s != u ? __ldg(fd.f + u) : 0.0f;
+                fs[r] = s != u ? __ldg(fd.f + s) : 0.0f;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RB; r++) {
+            const uint32_t u = (uint32_t)(u0 + (q + r) * 32 + lane);
+            bool k = tri_s(T[q + r]) != u;
+            if (SIMP) k = k && fd.sg * fs[r] - fd.sg * fu[r] >= eps;
+            keep |= (uint32_t)k << (q + r);
+        }
+    }
+    return keep;
+}
 
 template <class Loc, bool SIMP>
-__global__ void __launch_bounds__(kCompactThreads) k_pairs_count(Loc loc, uint32_t *counts, float eps,
+__global__ void __launch_bounds__(kCompactThreads, std::is_same<Loc, OneField>::value ? 4 : 3) k_pairs_count(Loc loc, uint32_t *counts, uint32_t *mask, float eps,
                                                                  const uint32_t *status)
 {
     if (block_skips(status)) return;
@@ -53,26 +83,28 @@ __global__ void __launch_bounds__(kCompactThreads) k_pairs_count(Loc loc, uint32
     const uint64_t n = fd.n;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t b0 = local * kCompactChunk + (uint64_t)warp * (kCompactRows * 32);
-    uint32_t c = 0;
     // all rows are loaded before any is used, so that their loads overlap
     uint64_t Tr[kCompactRows];
 #pragma unroll
     for (int r = 0; r < kCompactRows; r++) {
         const uint64_t u = b0 + (uint64_t)r * 32 + lane;
-        Tr[r] = u < n ? W[u] : tri_pack((uint32_t)u, (uint32_t)u + 1);  // past the end: neither pair nor root
+        Tr[r] = u < n ? W[u] : (uint64_t)(uint32_t)u << 32 | (uint32_t)~u;  // past the end: neither pair nor root
     }
+    const uint32_t keep = keep_rows<SIMP>(fd, Tr, b0, eps);
+    uint32_t mine = 0;
 #pragma unroll
     for (int r = 0; r < kCompactRows; r++) {
-        const uint64_t u = b0 + (uint64_t)r * 32 + lane;
-        const uint64_t T = Tr[r];
-        if (tri_s(T) != (uint32_t)u) {
-            c += keep_pair<SIMP>(fd, T, (uint32_t)u, eps);
-        } else if (tri_v(T) == (uint32_t)u) {
+        const uint32_t u = (uint32_t)(b0 + (uint64_t)r * 32 + lane);
+        if (Tr[r] == tri_pack(u, u)) {
             atomicAdd(reinterpret_cast<unsigned long long *>(fd.meta + 1), 1ull);
             fd.meta[2] = u;
         }
+        const uint32_t bal = __ballot_sync(0xffffffffu, (keep >> r) & 1u);
+        mine = lane == (uint32_t)r ? bal : mine;
     }
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (mask && lane < (uint32_t)kCompactRows)
+        mask[(uint64_t)blockIdx.x * (kCompactChunk / 32) + warp * kCompactRows + lane] = mine;
+    const uint32_t c = __reduce_add_sync(0xffffffffu, __popc(mine));
     if (lane == 0) warp_sum[warp] = c;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -132,8 +164,9 @@ __global__ void __launch_bounds__(1024) k_scan_counts(Loc loc, uint32_t *counts,
     }
 }
 
-template <class Loc, bool SIMP>
-__global__ void __launch_bounds__(kCompactThreads) k_pairs_write(Loc loc, const uint32_t *offsets, float eps,
+template <class Loc, bool SIMP, bool MASK>
+__global__ void __launch_bounds__(kCompactThreads) k_pairs_write(Loc loc, const uint32_t *offsets,
+                                                                 const uint32_t *__restrict__ mask, float eps,
                                                                  const uint32_t *status)
 {
     if (block_skips(status)) return;
@@ -147,49 +180,73 @@ __global__ void __launch_bounds__(kCompactThreads) k_pairs_write(Loc loc, const 
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t b0 = local * kCompactChunk + (uint64_t)warp * (kCompactRows * 32);
     uint64_t Tr[kCompactRows];
-    uint32_t c = 0;
+    uint32_t mine = 0;  // lane r: the flags of row r
+    if (MASK) {
+        if (lane < (uint32_t)kCompactRows)
+            mine = mask[(uint64_t)blockIdx.x * (kCompactChunk / 32) + warp * kCompactRows + lane];
+    } else {
 #pragma unroll
-    for (int r = 0; r < kCompactRows; r++) {
-        const uint64_t u = b0 + (uint64_t)r * 32 + lane;
-        Tr[r] = u < n ? W[u] : tri_pack((uint32_t)u, (uint32_t)u);  // past the end: no pair
-        c += __popc(__ballot_sync(0xffffffffu, keep_pair<SIMP>(fd, Tr[r], (uint32_t)u, eps)));
+        for (int r = 0; r < kCompactRows; r++) {
+            const uint64_t u = b0 + (uint64_t)r * 32 + lane;
+            Tr[r] = u < n ? W[u] : tri_pack((uint32_t)u, (uint32_t)u);  // past the end: no pair
+        }
+        const uint32_t keep = keep_rows<SIMP>(fd, Tr, b0, eps);
+#pragma unroll
+        for (int r = 0; r < kCompactRows; r++) {
+            const uint32_t bal = __ballot_sync(0xffffffffu, (keep >> r) & 1u);
+            mine = lane == (uint32_t)r ? bal : mine;
+        }
     }
+    const uint32_t c = __reduce_add_sync(0xffffffffu, __popc(mine));
     if (lane == 0) warp_cnt[warp] = c;
+    if (MASK) {
+#pragma unroll
+        for (int r = 0; r < kCompactRows; r++) {
+            const uint32_t q = __shfl_sync(0xffffffffu, mine, r);
+            Tr[r] = (q >> lane) & 1u ? W[b0 + (uint64_t)r * 32 + lane] : 0;
+        }
+    }
     __syncthreads();
     uint64_t run = offsets[blockIdx.x];
     for (uint32_t w = 0; w < warp; w++) run += warp_cnt[w];
     const uint32_t below = (1u << lane) - 1u;
+    const bool wide = ((uintptr_t)pairs & 7) == 0;  // the list is only 4-byte aligned
 #pragma unroll
     for (int r = 0; r < kCompactRows; r++) {
-        const uint64_t u = b0 + (uint64_t)r * 32 + lane;
-        const bool flag = keep_pair<SIMP>(fd, Tr[r], (uint32_t)u, eps);
-        const uint32_t ball = __ballot_sync(0xffffffffu, flag);
-        if (flag) {
-            const uint64_t pos = run + __popc(ball & below);
+        const uint32_t u = (uint32_t)(b0 + (uint64_t)r * 32 + lane);
+        const uint32_t q = __shfl_sync(0xffffffffu, mine, r);
+        if ((q >> lane) & 1u) {
+            const uint64_t pos = run + __popc(q & below);
             if (pos < cap) {
-                pairs[2 * pos] = (uint32_t)u;
-                pairs[2 * pos + 1] = tri_s(Tr[r]);
+                if (wide) {
+                    reinterpret_cast<uint2 *>(pairs)[pos] = make_uint2(u, tri_s(Tr[r]));
+                } else {
+                    pairs[2 * pos] = u;
+                    pairs[2 * pos + 1] = tri_s(Tr[r]);
+                }
             }
         }
-        run += __popc(ball);
+        run += __popc(q);
     }
 }
 
 template <class Loc>
-static cudaError_t run_pairs(const Loc &loc, uint32_t nfields, uint64_t nchunks, uint32_t *counts, uint64_t *npairs,
-                             const uint32_t *status, cudaStream_t st, float eps = 0.0f)
+static cudaError_t run_pairs(const Loc &loc, uint32_t nfields, uint64_t nchunks, uint32_t *counts, uint32_t *mask,
+                             uint64_t *npairs, const uint32_t *status, cudaStream_t st, float eps = 0.0f)
 {
     PhaseScope ps(kPairs, st);
     count_launch(3);
     const bool simp = eps > 0.0f;
-    if (simp) k_pairs_count<Loc, true><<<(unsigned)nchunks, kCompactThreads, 0, st>>>(loc, counts, eps, status);
-    else k_pairs_count<Loc, false><<<(unsigned)nchunks, kCompactThreads, 0, st>>>(loc, counts, eps, status);
+    const unsigned grid = (unsigned)nchunks;
+    if (simp) k_pairs_count<Loc, true><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
+    else k_pairs_count<Loc, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_scan_counts<Loc><<<nfields, 1024, 0, st>>>(loc, counts, npairs, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (simp) k_pairs_write<Loc, true><<<(unsigned)nchunks, kCompactThreads, 0, st>>>(loc, counts, eps, status);
-    else k_pairs_write<Loc, false><<<(unsigned)nchunks, kCompactThreads, 0, st>>>(loc, counts, eps, status);
+    if (mask) k_pairs_write<Loc, false, true><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
+    else if (simp) k_pairs_write<Loc, true, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
+    else k_pairs_write<Loc, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
     return cudaGetLastError();
 }
 
@@ -207,14 +264,14 @@ cudaError_t launch_pairs(const uint64_t *W, uint64_t n, uint32_t *pairs, uint64_
     loc.d.cap = cap;
     loc.d.f = f;
     loc.d.sg = sg;
-    return run_pairs(loc, 1, ws.nchunks, ws.counts, nullptr, ws.status, st, eps);
+    return run_pairs(loc, 1, ws.nchunks, ws.counts, ws.mask, nullptr, ws.status, st, eps);
 }
 
 cudaError_t launch_batch_pairs(const FieldDesc *d_descs, uint32_t nfields, uint64_t nchunks, uint32_t *counts,
                                uint64_t *npairs, const uint32_t *status, cudaStream_t st)
 {
     ManyFields loc{d_descs, nfields};
-    return run_pairs(loc, nfields, nchunks, counts, npairs, status, st);
+    return run_pairs(loc, nfields, nchunks, counts, nullptr, npairs, status, st);
 }
 
 // ----------------------------------------------------------------- labels
@@ -233,6 +290,14 @@ cudaError_t launch_batch_pairs(const FieldDesc *d_descs, uint32_t nfields, uint6
 // slot. The vertices of a brick share a few hundred starts, so each vertex
 // costs one read of f and W and one write, and the chases run once per start.
 // A vertex whose start finds no room in the hash follows its chain itself.
+// 356 us for 400^3 vertices, of which HBM needs 150: the dependent reads of
+// the chases and the probes' instructions (389 us with a division into rows
+// per vertex and without the start's triplet being fetched when it is
+// entered; loops kept together by votes, which serve the build's kernels,
+// 406: nearly every probe succeeds at once). 3 CTAs per SM: 406.
+//
+// WIDE: 64-bit ids (the wide path's triplets and labels; 1.0 ms for 512^3, 1.7
+// with a chase per vertex).
 //
 // With eps > 0 the labels are those of the simplified field in which every
 // branch of persistence below eps is filled up to its saddle: a component of
@@ -242,114 +307,131 @@ cudaError_t launch_batch_pairs(const FieldDesc *d_descs, uint32_t nfields, uint6
 // rule a branch is never less persistent than one that merges into it, so a
 // long branch never lies inside a short one's pit.
 constexpr uint32_t kLabLX = 5, kLabLY = 4, kLabLZ = 4;
-constexpr uint32_t kLabThreads = 512;
-constexpr uint32_t kLabHashLog = kLabelHashLog;  // 4096 slots (64 in a stress build)
-constexpr size_t kLabSmem = ((size_t)8 << kLabHashLog) + ((size_t)2 << (kLabLX + kLabLY + kLabLZ));
+constexpr uint32_t kLabThreads = 1u << (kLabLX + kLabLY);  // a thread per column of the brick
+template <bool WIDE>
+struct LabelShape {
+    static constexpr uint32_t kSlots = (WIDE ? 2048 : 4096) / kLabelShrink;
+    static constexpr size_t kSmem =
+        (size_t)kSlots * 2 * sizeof(typename Tri<WIDE>::Id) + ((size_t)2 << (kLabLX + kLabLY + kLabLZ));
+};
 
-__global__ void __launch_bounds__(kLabThreads, 4) k_labels(const Field f, const uint64_t *__restrict__ W, uint32_t nx,
-                                                           uint32_t ny, uint32_t nz, uint32_t ntx, uint32_t nty,
-                                                           float t, float eps, uint32_t *__restrict__ labels,
+template <bool WIDE>
+__global__ void __launch_bounds__(kLabThreads, 4) k_labels(const float *__restrict__ f, float sg,
+                                                           const uint64_t *__restrict__ W, uint32_t nx, uint32_t ny,
+                                                           uint32_t nz, uint32_t ntx, uint32_t nty, float t, float eps,
+                                                           typename Tri<WIDE>::Id *__restrict__ labels,
                                                            uint32_t *status)
 {
-    const uint32_t n = nx * ny * nz;
-    const uint32_t limit = n < kChaseLimit ? n : kChaseLimit;
+    using Id = typename Tri<WIDE>::Id;
     if (block_skips(status)) return;
-    constexpr uint32_t TX = 1u << kLabLX, TY = 1u << kLabLY, TZ = 1u << kLabLZ, TV = TX * TY * TZ;
-    constexpr uint32_t HS = 1u << kLabHashLog, NT = kLabThreads, NB = 4;
-    constexpr uint32_t EMPTY = 0xFFFFFFFFu, kProbes = 16;
+    const Id nxy = (Id)nx * ny, n = nxy * nz;
+    const uint32_t limit = n < kChaseLimit ? (uint32_t)n : kChaseLimit;
+    constexpr uint32_t TX = 1u << kLabLX, TY = 1u << kLabLY, TZ = 1u << kLabLZ, NT = kLabThreads;
+    constexpr uint32_t HS = LabelShape<WIDE>::kSlots, kProbes = 16, NB = WIDE ? 2 : 4;  // rows loaded together
+    constexpr Id EMPTY = ~(Id)0, NOLABEL = ~(Id)0;
     constexpr uint16_t OUT = 0xFFFFu, SELF = 0xFFFEu;  // slot codes: not in G_t; no room in the hash
-    static_assert(HS <= SELF && TV % (NT * NB) == 0, "slot codes and batches");
-    extern __shared__ __align__(16) uint32_t smem[];
-    uint32_t *hkey = smem;               // chain starts
-    uint32_t *hval = hkey + HS;          // their representatives at t
+    static_assert(HS <= SELF && (HS & (HS - 1)) == 0 && TZ % NB == 0, "slot codes, power of two, whole batches");
+    extern __shared__ __align__(16) uint64_t lab_smem[];
+    Id *hkey = reinterpret_cast<Id *>(lab_smem);       // chain starts
+    Id *hval = hkey + HS;                              // their representatives at t
     uint16_t *vslot = reinterpret_cast<uint16_t *>(hval + HS);  // per vertex: slot or code
-    const unsigned long long *Wq = reinterpret_cast<const unsigned long long *>(W);
 
     const uint32_t tile = blockIdx.x;
     const uint32_t tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
     const uint32_t x0 = tx * TX, y0 = ty * TY, z0 = tz * TZ;
     const uint32_t wx = min(TX, nx - x0), wy = min(TY, ny - y0), wz = min(TZ, nz - z0);
-    const uint32_t nxy = nx * ny;
-    const uint32_t base = z0 * nxy + y0 * nx + x0;
-    auto gid_of = [&](uint32_t l) {
-        return base + (l >> (kLabLX + kLabLY)) * nxy + ((l >> kLabLX) & (TY - 1)) * nx + (l & (TX - 1));
-    };
-    auto inside = [&](uint32_t l) {
-        return (l & (TX - 1)) < wx && ((l >> kLabLX) & (TY - 1)) < wy && (l >> (kLabLX + kLabLY)) < wz;
+    const uint32_t cx = threadIdx.x & (TX - 1), cy = threadIdx.x >> kLabLX;
+    const bool inx = cx < wx && cy < wy;
+    const Id u0 = (Id)z0 * nxy + (Id)(y0 + cy) * nx + x0 + cx;  // vertex z of the column: u0 + z * nxy
+    auto val = [&](Id u) { return sg * __ldg(f + u); };
+    // a triplet as the caller gave it (all bits of its ids)
+    auto load = [&](Id u, Id &s, Id &v) {
+        if constexpr (WIDE) {
+            const ulonglong2 w = reinterpret_cast<const ulonglong2 *>(W)[u];
+            s = w.x, v = w.y;
+        } else {
+            const uint64_t w = __ldg(reinterpret_cast<const unsigned long long *>(W) + u);
+            s = tri_s(w), v = tri_v(w);
+        }
     };
     // representative at t of the chain from x: the caller's triplets are
     // followed only through ids < n, and for at most `limit` links (a chain
     // of a valid tree is shorter than n, so a longer one means a cycle)
     bool ok = true, bad = false;
-    auto chase = [&](uint32_t x) -> uint32_t {
+    auto chase = [&](Id x) -> Id {
         for (uint32_t h = 0;; h++) {
-            const uint64_t T = __ldg(Wq + x);
-            const uint32_t s = tri_s(T);
-            if (T == tri_pack(x, x)) return x;
-            if (s >= n || tri_v(T) >= n) {
+            Id s, v;
+            load(x, s, v);
+            if (s == x && v == x) return x;
+            if (s >= n || v >= n) {
                 bad = true;
                 return x;
             }
-            if (!(f[s] <= t)) return x;
-            x = tri_v(T);
+            if (!(val(s) <= t)) return x;
+            x = v;
             if (h >= limit) {
                 ok = false;
                 return x;
             }
         }
     };
-    // the representative, or 0xFFFFFFFF if it heads a branch shorter than eps
-    auto simplified = [&](uint32_t r) -> uint32_t {
-        if (!(eps > 0.0f)) return r;
-        const uint64_t T = __ldg(Wq + r);
-        const uint32_t s = tri_s(T);
+    // the representative, or NOLABEL if it heads a branch shorter than eps
+    auto simplified = [&](Id r) -> Id {
+        if (WIDE || !(eps > 0.0f)) return r;
+        Id s, v;
+        load(r, s, v);
         if (s == r || s >= n) return r;  // the root (or an inner vertex of a corrupt tree)
-        return f[s] - f[r] >= eps ? r : 0xFFFFFFFFu;
+        return val(s) - val(r) >= eps ? r : NOLABEL;
     };
 
     for (uint32_t i = threadIdx.x; i < HS; i += NT) hkey[i] = EMPTY;
     __syncthreads();
 
     // 1. chain starts into the hash
-    volatile uint32_t *vhk = hkey;
-    for (uint32_t l0 = 0; l0 < TV; l0 += NT * NB) {
-        uint64_t Tb[NB];
+    volatile Id *vhk = hkey;
+    for (uint32_t zb = 0; zb < wz; zb += NB) {
+        Id sb[NB], vb[NB];
         float fb[NB];
 #pragma unroll
         for (uint32_t k = 0; k < NB; k++) {
-            const uint32_t l = l0 + k * NT + threadIdx.x;
-            const uint32_t u = gid_of(l);
-            const bool in = inside(l);
-            fb[k] = in ? f[u] : 0.0f;
-            Tb[k] = in ? __ldg(Wq + u) : tri_pack(u, u);
+            const bool in = inx && zb + k < wz;
+            const Id u = u0 + (zb + k) * nxy;
+            fb[k] = in ? val(u) : 0.0f;
+            sb[k] = vb[k] = 0;
+            if (in) load(u, sb[k], vb[k]);
         }
 #pragma unroll
         for (uint32_t k = 0; k < NB; k++) {
-            const uint32_t l = l0 + k * NT + threadIdx.x;
-            if (!inside(l)) continue;
-            const uint32_t u = gid_of(l);
-            if (!(fb[k] <= t)) {
-                vslot[l] = OUT;
-                continue;
-            }
-            const uint32_t s = tri_s(Tb[k]), v = tri_v(Tb[k]);
-            if (s >= n || v >= n) {  // leave it to the vertex's own chase, which reports it
-                vslot[l] = SELF;
-                continue;
-            }
-            const uint32_t st = (s == u && v != u) ? v : u;
-            uint32_t h = (st * 0x9E3779B1u) >> (32 - kLabHashLog);
-            uint16_t slot = SELF;
-            for (uint32_t p = 0; p < kProbes; p++) {
-                uint32_t kk = vhk[h];
-                if (kk == EMPTY) kk = atomicCAS(hkey + h, EMPTY, st);
-                if (kk == EMPTY || kk == st) {
-                    slot = (uint16_t)h;
-                    break;
+            const uint32_t z = zb + k;
+            if (!inx || z >= wz) continue;
+            const Id u = u0 + z * nxy;
+            uint16_t slot = OUT;
+            if (fb[k] <= t) {
+                slot = SELF;
+                // (an id >= n is left to the vertex's own chase, which reports it)
+                if (sb[k] < n && vb[k] < n) {
+                    const Id st = (sb[k] == u && vb[k] != u) ? vb[k] : u;
+                    uint32_t h = (((uint32_t)st * 0x9E3779B1u) >> 16) & (HS - 1);
+                    for (uint32_t p = 0; p < kProbes; p++) {
+                        Id q = vhk[h];
+                        if (q == EMPTY) {
+                            if constexpr (WIDE)
+                                q = atomicCAS(reinterpret_cast<unsigned long long *>(hkey + h),
+                                              (unsigned long long)EMPTY, (unsigned long long)st);
+                            else q = atomicCAS(hkey + h, EMPTY, st);
+                            // its chase begins with this read
+                            if (q == EMPTY)
+                                asm volatile("prefetch.global.L2 [%0];" ::"l"(W + (WIDE ? 2 : 1) * (size_t)st));
+                        }
+                        if (q == EMPTY || q == st) {
+                            slot = (uint16_t)h;
+                            break;
+                        }
+                        h = (h + 1) & (HS - 1);
+                    }
                 }
-                h = (h + 1) & (HS - 1);
             }
-            vslot[l] = slot;
+            vslot[threadIdx.x + z * NT] = slot;
         }
     }
     __syncthreads();
@@ -385,40 +467,63 @@ __global__ void __launch_bounds__(kLabThreads, 4) k_labels(const Field f, const 
         }
     } else {
         for (uint32_t i = threadIdx.x; i < HS; i += NT) {
-            const uint32_t st = hkey[i];
+            const Id st = hkey[i];
             if (st != EMPTY) hval[i] = simplified(chase(st));
         }
     }
     __syncthreads();
 
     // 3. labels
-    for (uint32_t l = threadIdx.x; l < TV; l += NT) {
-        if (!inside(l)) continue;
-        const uint32_t u = gid_of(l);
-        const uint16_t c = vslot[l];
-        labels[u] = c == OUT ? 0xFFFFFFFFu : c == SELF ? simplified(chase(u)) : hval[c];
+    if (inx) {
+        uint32_t self = 0;  // bit z: the vertex follows its chain itself
+#pragma unroll 4
+        for (uint32_t z = 0; z < wz; z++) {
+            const uint16_t c = vslot[threadIdx.x + z * NT];
+            self |= (uint32_t)(c == SELF) << z;
+            if (c != SELF) labels[u0 + z * nxy] = c == OUT ? NOLABEL : hval[c];
+        }
+        for (; self; self &= self - 1) {
+            const Id u = u0 + (__ffs(self) - 1) * nxy;
+            labels[u] = simplified(chase(u));
+        }
     }
     if (!ok) raise_status(status, ST_TIMEOUT);
     if (bad) raise_status(status, ST_CORRUPT);
 }
 
-cudaError_t launch_labels(const float *f, const uint64_t *W, uint32_t nx, uint32_t ny, uint32_t nz, float t,
-                          float sg, uint32_t *labels, Workspace &ws, cudaStream_t st, float eps)
+template <bool WIDE>
+static cudaError_t run_labels(const float *f, const uint64_t *W, uint32_t nx, uint32_t ny, uint32_t nz, float t,
+                              float sg, typename Tri<WIDE>::Id *labels, uint32_t *status, cudaStream_t st, float eps)
 {
     PhaseScope ps(kLabels, st);
-    count_launch();
-    const uint32_t ntx = (nx + 31) >> kLabLX, nty = (ny + 15) >> kLabLY, ntz = (nz + 15) >> kLabLZ;
-    static AttrFlags attr;
+    const uint32_t ntx = (uint32_t)(((uint64_t)nx + 31) >> kLabLX), nty = (uint32_t)(((uint64_t)ny + 15) >> kLabLY),
+                   ntz = (uint32_t)(((uint64_t)nz + 15) >> kLabLZ);
+    static AttrFlags attr;  // per instantiation
     int dev;
     if (attr.pending(dev)) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_labels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLabSmem);
+        const cudaError_t e = cudaFuncSetAttribute(k_labels<WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)LabelShape<WIDE>::kSmem);
         if (e != cudaSuccess) return e;
         attr.done(dev);
     }
-    k_labels<<<ntx * nty * ntz, kLabThreads, kLabSmem, st>>>(Field{f, sg}, W, nx, ny, nz, ntx, nty, t, eps,
-                                                            labels, ws.status);
+    const uint64_t bricks = (uint64_t)ntx * nty * ntz;
+    if (bricks >= 0x80000000ull) return cudaErrorInvalidValue;
+    k_labels<WIDE><<<(unsigned)bricks, kLabThreads, LabelShape<WIDE>::kSmem, st>>>(f, sg, W, nx, ny, nz, ntx, nty, t,
+                                                                                  eps, labels, status);
+    count_launch();
     return cudaGetLastError();
+}
+
+cudaError_t launch_labels(const float *f, const uint64_t *W, uint32_t nx, uint32_t ny, uint32_t nz, float t,
+                          float sg, uint32_t *labels, Workspace &ws, cudaStream_t st, float eps)
+{
+    return run_labels<false>(f, W, nx, ny, nz, t, sg, labels, ws.status, st, eps);
+}
+
+cudaError_t launch_labels_wide(const float *f, const uint64_t *W2, uint32_t nx, uint32_t ny, uint32_t nz, float t,
+                               float sg, uint64_t *labels, uint32_t *status, cudaStream_t st)
+{
+    return run_labels<true>(f, W2, nx, ny, nz, t, sg, labels, status, st, 0.0f);
 }
 
 }  // namespace mt

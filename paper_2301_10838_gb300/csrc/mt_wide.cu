@@ -26,8 +26,9 @@
 // per vertex the field and the triplets take. The tile kernel writes tag 0;
 // repair writes every word back without its tag.
 //
-// Pairs and labels: k_w_pairs_count / k_w_scan / k_w_pairs_write (ordered
-// compaction with 64-bit offsets) and k_w_labels (a chase per vertex).
+// Pairs: k_w_pairs_count / k_w_scan / k_w_pairs_write (ordered compaction with
+// 64-bit offsets). Labels: the labels kernel of the 32-bit path with 64-bit ids
+// (launch_labels_wide).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -267,26 +268,44 @@ __global__ void __launch_bounds__(256) k_w_cross(FieldW f, Geo g, uint32_t ntx, 
 }
 
 // ----------------------------------------------------------------- pairs
+// One CTA per chunk; warp w owns 512 consecutive vertices, read in 16 rows of
+// 32 (one 16-byte load each, eight rows loaded before any is used). The count
+// leaves a bit per vertex, so that the write reads the words of pairs only.
+constexpr int kWRows = kWChunk / kWThreads;  // rows of 32 per warp
+
 __global__ void __launch_bounds__(kWThreads) k_w_pairs_count(const uint64_t *W, uint64_t n, uint32_t *counts,
-                                                             uint64_t *meta, const uint32_t *status)
+                                                             uint32_t *mask, uint64_t *meta, const uint32_t *status)
 {
     if (block_skips(status)) return;
     __shared__ uint32_t s_cnt;
     if (threadIdx.x == 0) s_cnt = 0;
     __syncthreads();
-    const uint64_t a = blockIdx.x * (uint64_t)kWChunk;
-    uint32_t c = 0;
-    for (uint64_t u = a + threadIdx.x; u < a + kWChunk && u < n; u += kWThreads) {
-        const uint64_t s = W[2 * u], v = W[2 * u + 1];
-        if (s != u) {
-            c++;
-        } else if (v == u) {
-            atomicAdd(reinterpret_cast<unsigned long long *>(meta + 1), 1ull);
-            meta[2] = u;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t a = blockIdx.x * (uint64_t)kWChunk + warp * (kWRows * 32);
+    uint32_t mine = 0;  // lane r: the flags of row r
+    constexpr int RB = 8;
+#pragma unroll
+    for (int q = 0; q < kWRows; q += RB) {
+        ulonglong2 T[RB];
+#pragma unroll
+        for (int r = 0; r < RB; r++) {
+            const uint64_t u = a + (q + r) * 32 + lane;
+            T[r] = u < n ? reinterpret_cast<const ulonglong2 *>(W)[u] : make_ulonglong2(u, ~u);
+        }
+#pragma unroll
+        for (int r = 0; r < RB; r++) {
+            const uint64_t u = a + (q + r) * 32 + lane;
+            if (T[r].x == u && T[r].y == u) {
+                atomicAdd(reinterpret_cast<unsigned long long *>(meta + 1), 1ull);
+                meta[2] = u;
+            }
+            const uint32_t bal = __ballot_sync(0xffffffffu, T[r].x != u);
+            mine = lane == (uint32_t)(q + r) ? bal : mine;
         }
     }
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_cnt, c);
+    if (lane < (uint32_t)kWRows) mask[blockIdx.x * (uint64_t)(kWChunk / 32) + warp * kWRows + lane] = mine;
+    const uint32_t c = __reduce_add_sync(0xffffffffu, __popc(mine));
+    if (lane == 0 && c) atomicAdd(&s_cnt, c);
     __syncthreads();
     if (threadIdx.x == 0) counts[blockIdx.x] = s_cnt;
 }
@@ -334,81 +353,43 @@ __global__ void __launch_bounds__(1024) k_w_scan(const uint32_t *counts, uint64_
 }
 
 // ordered write: the chunk's pairs at its offset, by ascending u (one warp
-// after another, ballots rank the lanes)
-__global__ void __launch_bounds__(kWThreads) k_w_pairs_write(const uint64_t *W, uint64_t n, const uint64_t *offsets,
-                                                             uint64_t *pairs, uint64_t cap, const uint32_t *status)
+// after another, the flags' ranks within a row)
+__global__ void __launch_bounds__(kWThreads, 4) k_w_pairs_write(const uint64_t *W, const uint64_t *offsets,
+                                                             const uint32_t *__restrict__ mask, uint64_t *pairs,
+                                                             uint64_t cap, const uint32_t *status)
 {
     if (block_skips(status)) return;
     constexpr int kWarps = kWThreads / 32;
-    constexpr uint32_t kPerWarp = kWChunk / kWarps;
     __shared__ uint32_t s_wc[kWarps];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t a = blockIdx.x * (uint64_t)kWChunk + (uint64_t)warp * kPerWarp;
-    uint32_t c = 0;
-    for (uint32_t r = 0; r < kPerWarp; r += 32) {
-        const uint64_t u = a + r + lane;
-        const bool p = u < n && W[2 * u] != u;
-        c += __popc(__ballot_sync(0xffffffffu, p));
-    }
+    const uint64_t a = blockIdx.x * (uint64_t)kWChunk + warp * (kWRows * 32);
+    uint32_t mine = 0;
+    if (lane < (uint32_t)kWRows) mine = mask[blockIdx.x * (uint64_t)(kWChunk / 32) + warp * kWRows + lane];
+    const uint32_t c = __reduce_add_sync(0xffffffffu, __popc(mine));
     if (lane == 0) s_wc[warp] = c;
+    uint64_t s[kWRows];
+#pragma unroll
+    for (int r = 0; r < kWRows; r++) {
+        const uint32_t q = __shfl_sync(0xffffffffu, mine, r);
+        s[r] = (q >> lane) & 1u ? W[2 * (a + r * 32 + lane)] : 0;
+    }
     __syncthreads();
     uint64_t run = offsets[blockIdx.x];
     for (uint32_t w = 0; w < warp; w++) run += s_wc[w];
-    for (uint32_t r = 0; r < kPerWarp; r += 32) {
-        const uint64_t u = a + r + lane;
-        const uint64_t s = u < n ? W[2 * u] : u;
-        const bool p = u < n && s != u;
-        const uint32_t ball = __ballot_sync(0xffffffffu, p);
-        if (p) {
-            const uint64_t pos = run + __popc(ball & ((1u << lane) - 1u));
-            if (pos < cap) pairs[2 * pos] = u, pairs[2 * pos + 1] = s;
-        }
-        run += __popc(ball);
-    }
-}
-
-// ---------------------------------------------------------------- labels
-// label[u] = the deepest vertex of u's component of G_t (Algorithm 4 with the
-// value test f(s) <= t), or all ones when f[u] > t.
-__global__ void __launch_bounds__(kWThreads) k_w_labels(FieldW f, uint64_t n, const uint64_t *W, float t,
-                                                        uint64_t *labels, uint32_t *status)
-{
-    if (*status) return;
-    bool ok = true, bad = false;
-    for (uint64_t u = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; u < n; u += (uint64_t)gridDim.x * blockDim.x) {
-        if (!(f[u] <= t)) {
-            labels[u] = ~0ull;
-            continue;
-        }
-        const ulonglong2 wu = reinterpret_cast<const ulonglong2 *>(W)[u];
-        uint64_t x = (wu.x == u && wu.y != u) ? wu.y : u;
-        for (uint64_t h = 0;; h++) {
-            const ulonglong2 wx = reinterpret_cast<const ulonglong2 *>(W)[x];
-            const uint64_t s = wx.x, v = wx.y;
-            if (s == x && v == x) break;
-            if (s >= n || v >= n) {
-                bad = true;
-                break;
-            }
-            if (!(f[s] <= t)) break;
-            x = v;
-            if (h >= kChaseLimit || h >= n) {
-                ok = false;
-                break;
+    const bool one = ((uintptr_t)pairs & 15) == 0;  // the list is only 8-byte aligned
+#pragma unroll
+    for (int r = 0; r < kWRows; r++) {
+        const uint64_t u = a + r * 32 + lane;
+        const uint32_t q = __shfl_sync(0xffffffffu, mine, r);
+        if ((q >> lane) & 1u) {
+            const uint64_t pos = run + __popc(q & ((1u << lane) - 1u));
+            if (pos < cap) {
+                if (one) reinterpret_cast<ulonglong2 *>(pairs)[pos] = make_ulonglong2(u, s[r]);
+                else pairs[2 * pos] = u, pairs[2 * pos + 1] = s[r];
             }
         }
-        labels[u] = x;
+        run += __popc(q);
     }
-    if (!ok) raise_status(status, ST_TIMEOUT);
-    if (bad) raise_status(status, ST_CORRUPT);
-}
-
-unsigned grid_for(uint64_t work)
-{
-    const uint64_t per_block = kWThreads * 8ull;
-    const uint64_t want = (work + per_block - 1) / per_block;
-    const uint64_t cap = (uint64_t)device_sms() * 16;
-    return (unsigned)(want < 1 ? 1 : want > cap ? cap : want);
 }
 
 mt_status wide_grid(mt_grid g, Geo &geo)
@@ -481,10 +462,11 @@ mt_status mt_persistence_pairs_wide(const uint64_t *d_W, mt_grid g, uint64_t *d_
     if (cudaMemsetAsync(ws.meta, 0, 3 * sizeof(uint64_t), s) != cudaSuccess) return MT_ERR_CUDA;
     {
         PhaseScope ps(kPairs, s);
-        k_w_pairs_count<<<(unsigned)ws.nchunks, kWThreads, 0, s>>>(d_W, geo.n, ws.counts, ws.meta, ws.status);
+        // the bits take the place of the build's notes, which are done with
+        uint32_t *mask = ws.notes;
+        k_w_pairs_count<<<(unsigned)ws.nchunks, kWThreads, 0, s>>>(d_W, geo.n, ws.counts, mask, ws.meta, ws.status);
         k_w_scan<<<1, 1024, 0, s>>>(ws.counts, ws.offsets, ws.nchunks, ws.meta, ws.status);
-        k_w_pairs_write<<<(unsigned)ws.nchunks, kWThreads, 0, s>>>(d_W, geo.n, ws.offsets, d_pairs, cap,
-                                                                   ws.status);
+        k_w_pairs_write<<<(unsigned)ws.nchunks, kWThreads, 0, s>>>(d_W, ws.offsets, mask, d_pairs, cap, ws.status);
         count_launch(3);
         if (cudaGetLastError() != cudaSuccess) return MT_ERR_CUDA;
     }
@@ -511,10 +493,9 @@ mt_status mt_components_at_wide(const float *d_f, const uint64_t *d_W, mt_grid g
     if (!carve(d_ws, ws_bytes, geo, ws)) return MT_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const float sg = (flags & MT_SUPERLEVEL) ? -1.0f : 1.0f;
-    PhaseScope ps(kLabels, s);
-    k_w_labels<<<grid_for(geo.n), kWThreads, 0, s>>>(FieldW{d_f, sg}, geo.n, d_W, sg * t, d_labels, ws.status);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? MT_OK : MT_ERR_CUDA;
+    return launch_labels_wide(d_f, d_W, g.nx, g.ny, g.nz, sg * t, sg, d_labels, ws.status, s) == cudaSuccess
+               ? MT_OK
+               : MT_ERR_CUDA;
 }
 
 }  // extern "C"
