@@ -25,32 +25,38 @@ struct OneField {
     __device__ __forceinline__ FieldDesc field(uint32_t) const { return d; }
 };
 
+// A field is found by whole warps: 32 lanes read the first tiles (chunks) of 32
+// evenly spaced fields at a time, so that a batch of 512 fields takes two
+// dependent reads instead of the nine of a binary search.
 struct ManyFields {
     const FieldDesc *d;
     uint32_t nfields;
-    // last field whose first tile is <= g (fields with no tiles cannot occur)
+    // last field whose first(field) is <= g (fields with no tiles cannot occur)
+    template <class First>
+    __device__ __forceinline__ uint32_t find(uint64_t g, First first) const
+    {
+        const uint32_t lane = threadIdx.x & 31;
+        uint32_t lo = 0, len = nfields;  // the answer is in [lo, lo + len)
+        while (len > 1) {
+            const uint32_t step = (len + 31) / 32, i = lo + lane * step;
+            const bool le = lane * step < len && first(d[i]) <= g;
+            const uint32_t k = __popc(__ballot_sync(0xffffffffu, le)) - 1;  // (field lo is always one)
+            lo += k * step;
+            len = len - k * step < step ? len - k * step : step;
+        }
+        return lo;
+    }
     __device__ __forceinline__ FieldDesc tile(uint32_t g, uint32_t &local) const
     {
-        uint32_t lo = 0, hi = nfields;
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (d[mid].tile0 <= g) lo = mid;
-            else hi = mid;
-        }
-        local = g - d[lo].tile0;
-        return d[lo];
+        const uint32_t i = find(g, [](const FieldDesc &f) -> uint64_t { return f.tile0; });
+        local = g - d[i].tile0;
+        return d[i];
     }
     __device__ __forceinline__ FieldDesc chunk(uint64_t g, uint64_t &local, uint32_t &fi) const
     {
-        uint32_t lo = 0, hi = nfields;
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (d[mid].chunk0 <= g) lo = mid;
-            else hi = mid;
-        }
-        local = g - d[lo].chunk0;
-        fi = lo;
-        return d[lo];
+        fi = find(g, [](const FieldDesc &f) -> uint64_t { return f.chunk0; });
+        local = g - d[fi].chunk0;
+        return d[fi];
     }
     __device__ __forceinline__ FieldDesc field(uint32_t i) const { return d[i]; }
 };
