@@ -306,13 +306,14 @@ Server::Admit Server::admit(Slot &s, const Request &r, mt_status &fail)
     bool ok = carve_workspace(s.ws, s.ws_bytes, n, ws);
     if (builds) {
         ok = ok && cudaMemcpyAsync(s.f, r.h_f, 4 * n, cudaMemcpyHostToDevice, st) == cudaSuccess;
-        ok = ok && mt_build_triplets(s.f, g, s.W, s.ws, s.ws_bytes, st) == MT_OK;
+        // the labels come out of the build's repair pass
+        ok = ok && mt_build_components(s.f, g, s.W, r.t, 0.0f, 0u, 0u, s.labels, s.ws, s.ws_bytes, st) == MT_OK;
         ok = ok && launch_pairs(s.W, n, s.pairs, cap, ws, st) == cudaSuccess;
     } else {
         s.h_meta[0] = res->npairs, s.h_meta[1] = res->nroots, s.h_meta[2] = res->root;
         ok = ok && cudaMemsetAsync(ws.status, 0, 256, st) == cudaSuccess;
+        ok = ok && mt_components_at(s.f, s.W, g, r.t, s.labels, s.ws, s.ws_bytes, st) == MT_OK;
     }
-    ok = ok && mt_components_at(s.f, s.W, g, r.t, s.labels, s.ws, s.ws_bytes, st) == MT_OK;
     if (builds)
         ok = ok && cudaMemcpyAsync(s.h_meta, ws.meta, 3 * sizeof(uint64_t), cudaMemcpyDeviceToHost, st) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(s.h_meta + 3, ws.status, sizeof(uint32_t), cudaMemcpyDeviceToHost, st) == cudaSuccess;
