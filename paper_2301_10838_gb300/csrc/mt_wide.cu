@@ -133,54 +133,63 @@ __device__ __forceinline__ bool wload(const uint64_t *W, uint64_t u, uint64_t &l
 }
 
 // ----------------------------------------------------------------- merge
-// Climb (Algorithm 3): from x, follow links whose saddle is at or below
-// (fS, S) in the order; a root stops the walk. Returns false if a read
-// stayed torn or the step budget ran out.
+// Merge(S, a, b): make a and b connected at level S, value fS (Algorithm 3), as
+// in the 32-bit path: both climbs side by side, everything a step may need
+// read with the step before it. A word read ahead may be torn; it is read
+// again, until its halves carry one tag, when the climb moves to it. Returns
+// false if a read stayed torn or the step budget ran out.
+// 512^3 lognormal: k_w_cross 0.97 ms, 1.31 ms with one climb after the other.
 struct WideMerge {
     uint64_t *W;
     FieldW f;
 
-    __device__ __forceinline__ bool climb(uint64_t &x, uint64_t S, float fS, uint64_t &lo, uint64_t &hi,
-                                          uint32_t &steps) const
+    struct Node {
+        uint64_t x, lo, hi;  // vertex, its word
+        float fx;            // its value
+    };
+
+    __device__ __forceinline__ bool settle(Node &a) const
     {
-        if (!wload(W, x, lo, hi)) return false;
-        for (;;) {
-            const uint64_t s = lo & kIdMask, v = hi & kIdMask;
-            if (s == x && v == x) return true;
-            if (s != S && !before_w(f[s], s, fS, S)) return true;
-            x = v;
-            if (!wload(W, x, lo, hi) || ++steps > kMergeStepLimit) return false;
-        }
+        return (a.lo >> kIdBits) == (a.hi >> kIdBits) || wload(W, a.x, a.lo, a.hi);
     }
 
-    // Merge(S, a, b): make a and b connected at level S (Algorithm 3).
-    __device__ bool merge(uint64_t S, uint64_t a, uint64_t b) const
+    __device__ bool merge(uint64_t S, float fS, uint64_t a, uint64_t b) const
     {
-        float fS = f[S];
-        uint64_t u = a, v = b;
-        uint32_t steps = 0;
-        for (;;) {
-            uint64_t ulo, uhi, vlo, vhi;
-            if (!climb(u, S, fS, ulo, uhi, steps) || !climb(v, S, fS, vlo, vhi, steps)) return false;
-            if (++steps > kMergeStepLimit) return false;
-            if (u == v) return true;
-            if (before_w(f[v], v, f[u], u)) {
-                uint64_t t = u;
-                u = v, v = t;
-                t = ulo, ulo = vlo, vlo = t;
-                t = uhi, uhi = vhi, vhi = t;
-            }
-            const uint64_t tag = (uint64_t)(((vlo >> kIdBits) + 1) & kTagMask) << kIdBits;
+        Node u{a, 0, 0, f[a]}, v{b, 0, 0, f[b]};
+        ld_word(W, a, u.lo, u.hi);
+        ld_word(W, b, v.lo, v.hi);
+        for (uint32_t steps = 0; steps < kMergeStepLimit; steps++) {
+            if (u.x == v.x) return true;
+            if (!settle(u) || !settle(v)) return false;
+            const uint64_t su = u.lo & kIdMask, sv = v.lo & kIdMask;
+            Node nu{u.hi & kIdMask, 0, 0, 0.0f}, nv{v.hi & kIdMask, 0, 0, 0.0f};  // behind the links
+            const bool ru = su == u.x && nu.x == u.x, rv = sv == v.x && nv.x == v.x;
+            const float fsu = f[su], fsv = f[sv];
+            nu.fx = f[nu.x], nv.fx = f[nv.x];
+            ld_word(W, nu.x, nu.lo, nu.hi);
+            ld_word(W, nv.x, nv.lo, nv.hi);
+            const bool mu = !ru && (su == S || before_w(fsu, su, fS, S)),
+                       mv = !rv && (sv == S || before_w(fsv, sv, fS, S));
+            if (mu) u = nu;
+            if (mv) v = nv;
+            if (mu || mv) continue;
+            const bool sw = before_w(v.fx, v.x, u.fx, u.x);  // v is the earlier one: link u under it
+            const Node hi = sw ? u : v;
+            const uint64_t tag = (uint64_t)(((hi.lo >> kIdBits) + 1) & kTagMask) << kIdBits;
             uint64_t olo, ohi;
-            cas128(W + 2 * v, vlo, vhi, S | tag, u | tag, olo, ohi);
-            if (olo == vlo && ohi == vhi) {
-                const uint64_t sv = vlo & kIdMask, tv = vhi & kIdMask;
-                if (sv == v && tv == v) return true;  // displaced a root: it carries no link
-                S = sv;                                // re-insert the displaced link
-                fS = f[sv];
-                v = tv;
+            cas128(W + 2 * hi.x, hi.lo, hi.hi, S | tag, (sw ? v.x : u.x) | tag, olo, ohi);
+            if (olo == hi.lo && ohi == hi.hi) {
+                if (sw ? ru : rv) return true;  // displaced a root: it carries no link
+                S = sw ? su : sv, fS = sw ? fsu : fsv;  // re-insert the displaced link
+                if (sw) u = nu;
+                else v = nv;
+            } else if (sw) {
+                u.lo = olo, u.hi = ohi;
+            } else {
+                v.lo = olo, v.hi = ohi;
             }
         }
+        return false;
     }
 };
 
@@ -252,7 +261,8 @@ __global__ void __launch_bounds__(256) k_w_cross(FieldW f, Geo g, uint32_t ntx, 
         const uint32_t en = list[i], dir = en / F, ee = en % F;
         uint64_t a, b;
         ends(dir, ee % kSide, ee / kSide, a, b);
-        const uint64_t S = before_w(f[a], a, f[b], b) ? b : a;
+        const float fa = f[a], fb = f[b];
+        const bool up = before_w(fa, a, fb, b);
         // climbs start at the tile minima the ends descend to
         auto start = [&](uint64_t u, uint64_t tbase) -> uint64_t {
             uint64_t lo, hi;
@@ -262,7 +272,7 @@ __global__ void __launch_bounds__(256) k_w_cross(FieldW f, Geo g, uint32_t ntx, 
             return tbase + (uint64_t)(l / F) * g.nxy + (uint64_t)(l / kSide % kSide) * g.nx + l % kSide;
         };
         const uint64_t step = dir == 0 ? kSide : dir == 1 ? kSide * g.nx : kSide * g.nxy;
-        ok &= M.merge(S, start(a, base), start(b, base + step));
+        ok &= M.merge(up ? b : a, up ? fb : fa, start(a, base), start(b, base + step));
     }
     if (!ok) raise_status(status, ST_TIMEOUT);
 }
