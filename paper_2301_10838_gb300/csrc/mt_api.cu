@@ -85,8 +85,8 @@ __global__ void k_readback(const uint64_t *meta, const uint32_t *status, volatil
     out[3] = *status;
 }
 
-// out[0..2] = meta (if given), out[3] = status word; synchronises s
-cudaError_t readback(const uint64_t *meta, const uint32_t *status, cudaStream_t s, uint64_t out[4])
+// The calling thread's buffer, by its host and device addresses.
+static cudaError_t readback_buffer(uint64_t *&host, uint64_t *&dev)
 {
     thread_local uint64_t *h = nullptr, *d = nullptr;
     if (!h) {
@@ -99,14 +99,48 @@ cudaError_t readback(const uint64_t *meta, const uint32_t *status, cudaStream_t 
         }
         h = static_cast<uint64_t *>(hp), d = static_cast<uint64_t *>(dp);
     }
-    k_readback<<<1, 1, 0, s>>>(meta, status, d);
-    count_launch();
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    host = h, dev = d;
+    return cudaSuccess;
+}
+
+static cudaError_t readback_wait(const uint64_t *h, cudaStream_t s, uint64_t out[4])
+{
+    const cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
     const volatile uint64_t *vh = h;
     for (int i = 0; i < 4; i++) out[i] = vh[i];
     return cudaSuccess;
+}
+
+// out[0..2] = meta (if given), out[3] = status word; synchronises s
+cudaError_t readback(const uint64_t *meta, const uint32_t *status, cudaStream_t s, uint64_t out[4])
+{
+    uint64_t *h, *d;
+    cudaError_t e = readback_buffer(h, d);
+    if (e != cudaSuccess) return e;
+    k_readback<<<1, 1, 0, s>>>(meta, status, d);
+    count_launch();
+    e = cudaGetLastError();
+    return e == cudaSuccess ? readback_wait(h, s, out) : e;
+}
+
+// The pair compaction of a call that synchronises: its last kernel leaves the
+// counters and the status word in the thread's buffer.
+static mt_status pairs_and_wait(const uint64_t *d_W, uint64_t n, uint32_t *d_pairs, uint64_t cap, Workspace &ws,
+                                cudaStream_t s, const float *f, float sg, float eps, bool clear, uint64_t *h_npairs,
+                                uint32_t *h_root)
+{
+    uint64_t *h, *d, meta[4];
+    if (readback_buffer(h, d) != cudaSuccess ||
+        launch_pairs(d_W, n, d_pairs, cap, ws, s, f, sg, eps, d, clear) != cudaSuccess ||
+        readback_wait(h, s, meta) != cudaSuccess)
+        return MT_ERR_CUDA;
+    const uint32_t bits = (uint32_t)meta[3];
+    if (bits) return status_from_bits(bits);
+    *h_npairs = meta[0];
+    if (h_root) *h_root = meta[1] == 1 ? (uint32_t)meta[2] : 0xFFFFFFFFu;
+    if (meta[1] != 1) return MT_ERR_INVALID;  // not a tree of a connected grid
+    return meta[0] > cap ? MT_ERR_CAPACITY : MT_OK;
 }
 
 mt_status status_from_bits(uint32_t bits)
@@ -211,20 +245,12 @@ mt_status mt_build_step(const float *d_f, mt_grid g, uint64_t *d_W, float t, flo
     if (ws_bytes < build_workspace_bytes(g.nx, g.ny, g.nz) || !carve_workspace(d_ws, ws_bytes, n, ws))
         return MT_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(ws.status, 0, 256, s) != cudaSuccess) return MT_ERR_CUDA;
+    if (cudaMemsetAsync(ws.status, 0, 512, s) != cudaSuccess) return MT_ERR_CUDA;  // and the pair counters
     const float sg = (flags & MT_SUPERLEVEL) ? -1.0f : 1.0f;
     const LabelArgs la{d_labels, sg * t, eps};
     if (launch_build(d_f, d_W, g.nx, g.ny, g.nz, ws, build_faces(d_ws, n), sg, s, cfg, &la) != cudaSuccess)
         return MT_ERR_CUDA;
-    if (launch_pairs(d_W, n, d_pairs, cap, ws, s, d_f, sg, eps) != cudaSuccess) return MT_ERR_CUDA;
-    uint64_t meta[4];
-    if (readback(ws.meta, ws.status, s, meta) != cudaSuccess) return MT_ERR_CUDA;
-    const uint32_t bits = (uint32_t)meta[3];
-    if (bits) return status_from_bits(bits);
-    *h_npairs = meta[0];
-    if (h_root) *h_root = meta[1] == 1 ? (uint32_t)meta[2] : 0xFFFFFFFFu;
-    if (meta[1] != 1) return MT_ERR_INVALID;  // not a tree of a connected grid
-    return meta[0] > cap ? MT_ERR_CAPACITY : MT_OK;
+    return pairs_and_wait(d_W, n, d_pairs, cap, ws, s, d_f, sg, eps, false, h_npairs, h_root);
 }
 
 mt_status mt_build_autotune(const float *d_f, mt_grid g, uint64_t *d_W, void *d_ws, size_t ws_bytes, uint32_t flags,
@@ -281,15 +307,7 @@ mt_status mt_persistence_pairs(const float *d_f, const uint64_t *d_W, mt_grid g,
     Workspace ws;
     if (!carve_workspace(d_ws, ws_bytes, n, ws)) return MT_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (launch_pairs(d_W, n, d_pairs, cap, ws, s) != cudaSuccess) return MT_ERR_CUDA;
-    uint64_t meta[4];
-    if (readback(ws.meta, ws.status, s, meta) != cudaSuccess) return MT_ERR_CUDA;
-    const uint32_t bits = (uint32_t)meta[3];
-    if (bits) return status_from_bits(bits);
-    *h_npairs = meta[0];
-    if (h_root) *h_root = meta[1] == 1 ? (uint32_t)meta[2] : 0xFFFFFFFFu;
-    if (meta[1] != 1) return MT_ERR_INVALID;  // not a tree of a connected grid
-    return meta[0] > cap ? MT_ERR_CAPACITY : MT_OK;
+    return pairs_and_wait(d_W, n, d_pairs, cap, ws, s, nullptr, 1.0f, 0.0f, true, h_npairs, h_root);
 }
 
 mt_status mt_simplified_pairs(const float *d_f, const uint64_t *d_W, mt_grid g, float eps, uint32_t flags,
@@ -306,15 +324,7 @@ mt_status mt_simplified_pairs(const float *d_f, const uint64_t *d_W, mt_grid g, 
     if (!carve_workspace(d_ws, ws_bytes, n, ws)) return MT_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const float sg = (flags & MT_SUPERLEVEL) ? -1.0f : 1.0f;
-    if (launch_pairs(d_W, n, d_pairs, cap, ws, s, d_f, sg, eps) != cudaSuccess) return MT_ERR_CUDA;
-    uint64_t meta[4];
-    if (readback(ws.meta, ws.status, s, meta) != cudaSuccess) return MT_ERR_CUDA;
-    const uint32_t bits = (uint32_t)meta[3];
-    if (bits) return status_from_bits(bits);
-    *h_npairs = meta[0];
-    if (h_root) *h_root = meta[1] == 1 ? (uint32_t)meta[2] : 0xFFFFFFFFu;
-    if (meta[1] != 1) return MT_ERR_INVALID;  // not a tree of a connected grid
-    return meta[0] > cap ? MT_ERR_CAPACITY : MT_OK;
+    return pairs_and_wait(d_W, n, d_pairs, cap, ws, s, d_f, sg, eps, true, h_npairs, h_root);
 }
 
 mt_status mt_simplified_components_at(const float *d_f, const uint64_t *d_W, mt_grid g, float t, float eps,

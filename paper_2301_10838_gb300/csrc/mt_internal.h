@@ -108,9 +108,12 @@ cudaError_t launch_build(const float *f, uint64_t *W, uint32_t nx, uint32_t ny, 
                          uint32_t *faces, float sg, cudaStream_t st, uint32_t cfg = 0,
                          const LabelArgs *la = nullptr);
 // f, sg, eps: persistence simplification (pairs of persistence below eps
-// dropped; eps <= 0 keeps all and does not read f)
+// dropped; eps <= 0 keeps all and does not read f). out: mapped host memory
+// that receives meta[0..2] and the status word (as readback's), or null.
+// clear: clear the counters first (false: the caller has)
 cudaError_t launch_pairs(const uint64_t *W, uint64_t n, uint32_t *pairs, uint64_t cap, Workspace &ws,
-                         cudaStream_t st, const float *f = nullptr, float sg = 1.0f, float eps = 0.0f);
+                         cudaStream_t st, const float *f = nullptr, float sg = 1.0f, float eps = 0.0f,
+                         uint64_t *out = nullptr, bool clear = true);
 
 // Batched build and pairs over a packed descriptor table already in device
 // memory; cfg holds the MT_CFG_* knobs (mt_build.cu, mt_query.cu).

@@ -164,13 +164,22 @@ __global__ void __launch_bounds__(1024) k_scan_counts(Loc loc, uint32_t *counts,
     }
 }
 
-template <class Loc, bool SIMP, bool MASK>
+// SUM: `offsets` still holds the chunks' counts, and every CTA adds up those
+// before its own. For a single field of up to kSumChunks chunks that costs less
+// than the scan's launch. The last CTA of a single field also leaves the
+// counters and the status word at `out` (mapped host memory, or null).
+constexpr uint64_t kSumChunks = 4096;
+
+template <class Loc, bool SIMP, bool MASK, bool SUM>
 __global__ void __launch_bounds__(kCompactThreads) k_pairs_write(Loc loc, const uint32_t *offsets,
                                                                  const uint32_t *__restrict__ mask, float eps,
-                                                                 const uint32_t *status)
+                                                                 const uint32_t *status, volatile uint64_t *out)
 {
-    if (block_skips(status)) return;
-    __shared__ uint32_t warp_cnt[kCompactWarps];
+    if (block_skips(status)) {
+        if (out && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[3] = *status;
+        return;
+    }
+    __shared__ uint32_t warp_cnt[kCompactWarps], warp_sum[kCompactWarps];
     uint64_t local;
     uint32_t fi;
     const FieldDesc fd = loc.chunk(blockIdx.x, local, fi);
@@ -206,8 +215,22 @@ __global__ void __launch_bounds__(kCompactThreads) k_pairs_write(Loc loc, const 
             Tr[r] = (q >> lane) & 1u ? W[b0 + (uint64_t)r * 32 + lane] : 0;
         }
     }
+    if (SUM) {
+        uint32_t s = 0;
+        for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kCompactThreads) s += offsets[i];
+        s = __reduce_add_sync(0xffffffffu, s);
+        if (lane == 0) warp_sum[warp] = s;
+    }
     __syncthreads();
-    uint64_t run = offsets[blockIdx.x];
+    uint64_t run = SUM ? 0 : offsets[blockIdx.x];
+    if (SUM)
+        for (int w = 0; w < kCompactWarps; w++) run += warp_sum[w];
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0 && (SUM || out)) {
+        uint64_t total = run;
+        for (int w = 0; w < kCompactWarps; w++) total += warp_cnt[w];
+        if (SUM) fd.meta[0] = total;
+        if (out) out[0] = total, out[1] = fd.meta[1], out[2] = fd.meta[2], out[3] = *status;
+    }
     for (uint32_t w = 0; w < warp; w++) run += warp_cnt[w];
     const uint32_t below = (1u << lane) - 1u;
     const bool wide = ((uintptr_t)pairs & 7) == 0;  // the list is only 4-byte aligned
@@ -232,29 +255,39 @@ __global__ void __launch_bounds__(kCompactThreads) k_pairs_write(Loc loc, const 
 
 template <class Loc>
 static cudaError_t run_pairs(const Loc &loc, uint32_t nfields, uint64_t nchunks, uint32_t *counts, uint32_t *mask,
-                             uint64_t *npairs, const uint32_t *status, cudaStream_t st, float eps = 0.0f)
+                             uint64_t *npairs, const uint32_t *status, cudaStream_t st, float eps = 0.0f,
+                             uint64_t *out = nullptr)
 {
     PhaseScope ps(kPairs, st);
-    count_launch(3);
     const bool simp = eps > 0.0f;
     const unsigned grid = (unsigned)nchunks;
     if (simp) k_pairs_count<Loc, true><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
     else k_pairs_count<Loc, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    if constexpr (std::is_same<Loc, OneField>::value) {
+        if (mask && nchunks <= kSumChunks) {
+            k_pairs_write<Loc, false, true, true><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
+            count_launch(2);
+            return cudaGetLastError();
+        }
+    }
     k_scan_counts<Loc><<<nfields, 1024, 0, st>>>(loc, counts, npairs, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (mask) k_pairs_write<Loc, false, true><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
-    else if (simp) k_pairs_write<Loc, true, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
-    else k_pairs_write<Loc, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
+    if (mask) k_pairs_write<Loc, false, true, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
+    else if (simp) k_pairs_write<Loc, true, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
+    else k_pairs_write<Loc, false, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
+    count_launch(3);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pairs(const uint64_t *W, uint64_t n, uint32_t *pairs, uint64_t cap, Workspace &ws,
-                         cudaStream_t st, const float *f, float sg, float eps)
+                         cudaStream_t st, const float *f, float sg, float eps, uint64_t *out, bool clear)
 {
-    cudaError_t e = cudaMemsetAsync(ws.meta, 0, 3 * sizeof(uint64_t), st);
-    if (e != cudaSuccess) return e;
+    if (clear) {
+        const cudaError_t e = cudaMemsetAsync(ws.meta, 0, 3 * sizeof(uint64_t), st);
+        if (e != cudaSuccess) return e;
+    }
     OneField loc;
     loc.d = FieldDesc{};
     loc.d.W = const_cast<uint64_t *>(W);
@@ -264,7 +297,7 @@ cudaError_t launch_pairs(const uint64_t *W, uint64_t n, uint32_t *pairs, uint64_
     loc.d.cap = cap;
     loc.d.f = f;
     loc.d.sg = sg;
-    return run_pairs(loc, 1, ws.nchunks, ws.counts, ws.mask, nullptr, ws.status, st, eps);
+    return run_pairs(loc, 1, ws.nchunks, ws.counts, ws.mask, nullptr, ws.status, st, eps, out);
 }
 
 cudaError_t launch_batch_pairs(const FieldDesc *d_descs, uint32_t nfields, uint64_t nchunks, uint32_t *counts,
