@@ -127,12 +127,12 @@ cudaError_t readback(const uint64_t *meta, const uint32_t *status, cudaStream_t 
 // The pair compaction of a call that synchronises: its last kernel leaves the
 // counters and the status word in the thread's buffer.
 static mt_status pairs_and_wait(const uint64_t *d_W, uint64_t n, uint32_t *d_pairs, uint64_t cap, Workspace &ws,
-                                cudaStream_t s, const float *f, float sg, float eps, bool clear, uint64_t *h_npairs,
-                                uint32_t *h_root)
+                                cudaStream_t s, const float *f, float sg, float eps, bool clear, bool marked,
+                                uint64_t *h_npairs, uint32_t *h_root)
 {
     uint64_t *h, *d, meta[4];
     if (readback_buffer(h, d) != cudaSuccess ||
-        launch_pairs(d_W, n, d_pairs, cap, ws, s, f, sg, eps, d, clear) != cudaSuccess ||
+        launch_pairs(d_W, n, d_pairs, cap, ws, s, f, sg, eps, d, clear, marked) != cudaSuccess ||
         readback_wait(h, s, meta) != cudaSuccess)
         return MT_ERR_CUDA;
     const uint32_t bits = (uint32_t)meta[3];
@@ -223,7 +223,7 @@ mt_status mt_build_components(const float *d_f, mt_grid g, uint64_t *d_W, float 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(ws.status, 0, 256, s) != cudaSuccess) return MT_ERR_CUDA;
     const float sg = (flags & MT_SUPERLEVEL) ? -1.0f : 1.0f;
-    const LabelArgs la{d_labels, sg * t, eps};
+    const LabelArgs la{d_labels, sg * t, eps, nullptr, nullptr};
     if (launch_build(d_f, d_W, g.nx, g.ny, g.nz, ws, build_faces(d_ws, n), sg, s, cfg, &la) != cudaSuccess)
         return MT_ERR_CUDA;
     return MT_OK;
@@ -247,10 +247,11 @@ mt_status mt_build_step(const float *d_f, mt_grid g, uint64_t *d_W, float t, flo
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(ws.status, 0, 512, s) != cudaSuccess) return MT_ERR_CUDA;  // and the pair counters
     const float sg = (flags & MT_SUPERLEVEL) ? -1.0f : 1.0f;
-    const LabelArgs la{d_labels, sg * t, eps};
-    if (launch_build(d_f, d_W, g.nx, g.ny, g.nz, ws, build_faces(d_ws, n), sg, s, cfg, &la) != cudaSuccess)
-        return MT_ERR_CUDA;
-    return pairs_and_wait(d_W, n, d_pairs, cap, ws, s, d_f, sg, eps, false, h_npairs, h_root);
+    uint32_t *faces = build_faces(d_ws, n), *mask = build_mask(faces, g.nx, g.ny, g.nz, cfg);
+    const LabelArgs la{d_labels, sg * t, eps, mask, ws.meta};
+    if (launch_build(d_f, d_W, g.nx, g.ny, g.nz, ws, faces, sg, s, cfg, &la) != cudaSuccess) return MT_ERR_CUDA;
+    if (mask) ws.mask = mask;
+    return pairs_and_wait(d_W, n, d_pairs, cap, ws, s, d_f, sg, eps, false, mask != nullptr, h_npairs, h_root);
 }
 
 mt_status mt_build_autotune(const float *d_f, mt_grid g, uint64_t *d_W, void *d_ws, size_t ws_bytes, uint32_t flags,
@@ -307,7 +308,7 @@ mt_status mt_persistence_pairs(const float *d_f, const uint64_t *d_W, mt_grid g,
     Workspace ws;
     if (!carve_workspace(d_ws, ws_bytes, n, ws)) return MT_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    return pairs_and_wait(d_W, n, d_pairs, cap, ws, s, nullptr, 1.0f, 0.0f, true, h_npairs, h_root);
+    return pairs_and_wait(d_W, n, d_pairs, cap, ws, s, nullptr, 1.0f, 0.0f, true, false, h_npairs, h_root);
 }
 
 mt_status mt_simplified_pairs(const float *d_f, const uint64_t *d_W, mt_grid g, float eps, uint32_t flags,
@@ -324,7 +325,7 @@ mt_status mt_simplified_pairs(const float *d_f, const uint64_t *d_W, mt_grid g, 
     if (!carve_workspace(d_ws, ws_bytes, n, ws)) return MT_ERR_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const float sg = (flags & MT_SUPERLEVEL) ? -1.0f : 1.0f;
-    return pairs_and_wait(d_W, n, d_pairs, cap, ws, s, d_f, sg, eps, true, h_npairs, h_root);
+    return pairs_and_wait(d_W, n, d_pairs, cap, ws, s, d_f, sg, eps, true, false, h_npairs, h_root);
 }
 
 mt_status mt_simplified_components_at(const float *d_f, const uint64_t *d_W, mt_grid g, float t, float eps,

@@ -737,13 +737,16 @@ __global__ void __launch_bounds__(128, std::is_same<Loc, OneField>::value ? 12 :
 // Tables that are full (more than kMin minima, a crowded hash) leave a link
 // without a node; whoever needs it goes on along the global chain.
 //
-// What it costs, on the 1024^3 lognormal field: 9.7 ms, 10.8 ms with labels
+// What it costs, on the 1024^3 lognormal field: 8.4 ms, 10.9 ms with labels
 // (11.7 and 14.2 ms with copies of each target's first 8 links found through
 // a hash per vertex, from triplets that the tile kernel had repaired itself
-// at 3.8 ms more): numbering 1.0, links 3.2 (chains of dependent reads),
-// targets and labels 0.7 to 1.2, inner vertices 4.9 to 5.4 (16 to 24 bytes
-// each way per vertex, 130 thread instructions). Issue slots are 60 % busy.
-// Climbing the forest before its targets are repaired costs 1.4 ms more.
+// at 3.8 ms more), 11.4 ms with labels and the pairs marked, which saves 1.2 ms
+// of the pair compaction. With 6 CTAs per SM: numbering 1.0, links 3.2 (chains
+// of dependent reads), targets and labels 0.7 to 1.2, inner vertices 4.9 to
+// 5.4 (16 to 24 bytes each way per vertex, 130 thread instructions). Issue
+// slots are 60 % busy. Climbing the forest before its targets are repaired
+// costs 1.4 ms more; marking the pairs in the loop over the inner vertices 1.0
+// ms more than from the list of minima.
 //
 // With LAB the pass also labels the components of G_t (the labels of
 // k_labels) where it already stands. The representative of u at level t is
@@ -811,9 +814,11 @@ struct RepairShape {
     // shared memory: link word and global id (with LAB also the label) of
     // every node (and of the one that stands for none), hash keys, the node of
     // each minimum by x-adjacent pair, the foreign nodes in the order they
-    // were entered
+    // were entered; with LAB the local id of each minimum, a bit per vertex
     static constexpr size_t kSmem = (size_t)(kNodes + 4) * 8 + (size_t)kNodes * (LAB || WIDE ? 8 : 4) +
-                                    (size_t)kHash * (WIDE ? 8 : 4) + (size_t)TV / 2 * 2 + (size_t)kHash * 2;
+                                    (size_t)kHash * (WIDE ? 8 : 4) + (size_t)TV / 2 * 2 + (size_t)kHash * 2 +
+                                    (LAB ? (size_t)kMin * 2 + TV / 8 : 0);
+    static_assert((kMin + kHash) % 2 == 0, "the bits after the 16-bit arrays are 4-byte aligned");
     static constexpr int kFit = (int)(227 * 1024 / (kSmem + 1024));
     // CTAs per SM the registers are limited for: 7 of 256 threads (36
     // registers) take 8.4 ms without labels on the 1024^3 field, 6 take 9.7;
@@ -847,6 +852,8 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
     Id *hkey = reinterpret_cast<Id *>(out + (LAB || WIDE ? NN : NN / 2));
     uint16_t *node = reinterpret_cast<uint16_t *>(hkey + HS);  // of the minimum of each x-adjacent pair
     uint16_t *order = node + TV / 2;
+    uint16_t *lid = order + HS;                    // LAB: local ids of the minima
+    uint32_t *pbits = reinterpret_cast<uint32_t *>(lid + MIN);  // LAB: a bit per vertex that begins a pair
     __shared__ uint32_t s_nmin, s_nf;
     auto id_of = [&](uint32_t x) -> Id {
         if constexpr (LAB) return (uint32_t)out[x];
@@ -903,6 +910,8 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
         }
     }
     for (uint32_t i = threadIdx.x; i < HS; i += NT) hkey[i] = EMPTY;
+    if (LAB)
+        for (uint32_t i = threadIdx.x; i < TV / 32; i += NT) pbits[i] = 0;
     if (threadIdx.x == 0) s_nmin = 0, s_nf = 0, word[NN] = LOST;
     __syncthreads();
 
@@ -924,7 +933,7 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
             const uint32_t z = __ffs(m) - 1;
             node[(col + z * NT) >> 1] = (uint16_t)(pos < MIN ? pos : NN);
             if (pos < MIN) {
-                if constexpr (LAB) out[pos] = ucol + z * nxy;
+                if constexpr (LAB) out[pos] = ucol + z * nxy, lid[pos] = (uint16_t)(col + z * NT);
                 else ids[pos] = ucol + z * nxy;
             }
         }
@@ -1027,6 +1036,18 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
     //    that follow) and, for the tile's minima, in W. A node whose link has
     //    a node lies at or below the tile's highest key, and so do the links it
     //    follows; a minimum with a higher saddle goes along the global chain.
+    //    With la.mask the minima that begin a pair are marked on the way: those
+    //    whose saddle is not the minimum itself (the cross-tile merges make
+    //    that of a minimum of the tile that is none of the grid) and, with
+    //    eps, lies high enough above it.
+    auto mark = [&](uint32_t l, Id u, Id sd, float fs) {
+        if (sd == u || (la.eps > 0.0f && !(fs - val(u) >= la.eps))) return;
+        atomicOr(pbits + (l >> 5), 1u << (l & 31));
+    };
+    auto mark_root = [&](Id u) {
+        atomicAdd(reinterpret_cast<unsigned long long *>(la.meta + 1), 1ull);
+        la.meta[2] = u;
+    };
     const uint32_t nf = s_nf, nall = nmin + nf;
     volatile uint64_t *vword = word;
     for (uint32_t i0 = 0; i0 < nall; i0 += NT) {
@@ -1057,11 +1078,18 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
         }
         const bool left = link && (uint32_t)wx_ == (uint32_t)LOST;  // further along the global chain
         if (link && !left && x != x0) vword[n] = (w & ~(uint64_t)0xFFFFu) | x;
-        if (i >= nmin || (ks == kNoKey && w != LOST)) continue;     // foreign, or the root
+        if (i >= nmin) continue;                   // foreign
         const Id u = id_of(n);
+        if (ks == kNoKey && w != LOST) {           // the root
+            if (LAB && la.mask) mark_root(u);
+            continue;
+        }
         Id s, v = 0;
         if (!link || left || sl == NONE) TR::load(W, u, s, v);
         else s = id_at(sl);
+        if constexpr (LAB) {
+            if (la.mask) mark(lid[n], u, s, la.eps > 0.0f ? val(s) : 0.0f);
+        }
         if (!link || left) TR::store(W, u, s, repair_walk<WIDE>(W, f, sg, left ? id_of(x) : v, s, val(s), &ok));
         else if (x != x0 || WIDE) TR::store(W, u, s, id_of(x));
     }
@@ -1097,6 +1125,10 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
             if (!(s == u && v == u)) TR::store(W, u, s, repair_walk<WIDE>(W, f, sg, v, s, val(s), &ok));
             else if (WIDE) TR::store(W, u, s, v);
             if constexpr (LAB) {
+                if (la.mask && s == u && v == u) mark_root(u);
+                else if (la.mask) mark(col + z * NT, u, s, val(s));
+            }
+            if constexpr (LAB) {
                 uint32_t lab = 0xFFFFFFFFu;
                 if (val(u) <= la.t) {
                     const uint64_t r = label_walk(W, Field{f, sg}, u, la.t, la.eps);
@@ -1108,6 +1140,21 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
         }
     }
     __syncthreads();
+    if constexpr (LAB) {
+        // the bits row by row: 16 or 32 vertices (build_mask sees to it that
+        // they fill whole pieces)
+        constexpr uint32_t ROW = TX, rows = TV / ROW;
+        if (la.mask && threadIdx.x < rows) {
+            static_assert(ROW == 16 || ROW == 32, "rows of 16 or 32 vertices");
+            const uint32_t r = threadIdx.x, y = r & (TY - 1), z = r >> LY;
+            const Id u = base + (Id)z * nxy + (Id)y * nx;
+            if (y < wy && z < wz) {
+                if constexpr (ROW == 16)
+                    reinterpret_cast<uint16_t *>(la.mask)[u >> 4] = reinterpret_cast<const uint16_t *>(pbits)[r];
+                else la.mask[u >> 5] = pbits[r];
+            }
+        }
+    }
 
     // 4. inner vertices, the next row's value and word loaded ahead (rows
     //    unrolled by 4 or 8 with their loads first measured slower: the
@@ -1283,6 +1330,19 @@ static cudaError_t run_build(const Loc &loc, uint32_t ntiles, uint32_t *queue, i
         if (la) return launch_repair<V, Loc, true>(loc, ntiles, status, st, *la);
     }
     return launch_repair<V>(loc, ntiles, status, st);
+}
+
+uint32_t *build_mask(uint32_t *faces, uint32_t nx, uint32_t ny, uint32_t nz, uint32_t cfg)
+{
+    const int v = cfg & MT_CFG_LARGE_TILES ? 2 : 0;
+    uint32_t tx, ty, tz;
+    tile_shape(v, tx, ty, tz);
+    if (nx % tx != 0) return nullptr;
+    constexpr int w0 = TileOf<0>::kTileWords<false>, w2 = TileOf<2>::kTileWords<false>;
+    static_assert(2 * TileOf<0>::FH - w0 >= TileOf<0>::TV / 32 && 2 * TileOf<2>::FH - w2 >= TileOf<2>::TV / 32,
+                  "a bit per vertex fits behind the records");
+    static_assert(w0 % 4 == 0 && w2 % 4 == 0, "16-byte aligned");
+    return faces + tile_count(v, nx, ny, nz) * (v == 2 ? w2 : w0);
 }
 
 // A single field in the tile shape of variant V (0, or 2 with MT_CFG_LARGE_TILES).

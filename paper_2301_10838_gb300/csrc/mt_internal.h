@@ -36,6 +36,10 @@ struct LabelArgs {
     uint32_t *labels;  // uint32[n]
     float t;           // threshold on the values the order sees (sg * f)
     float eps;         // persistence simplification; <= 0: none
+    // pairs marked on the way (build_mask), or null: a bit per vertex that
+    // begins a pair of persistence >= eps, and the roots counted in meta[1..2]
+    uint32_t *mask;
+    uint64_t *meta;
 };
 
 // Views into the caller's workspace (layout fixed by carve_workspace).
@@ -72,6 +76,10 @@ bool carve_workspace(void *base, size_t bytes, uint64_t n, Workspace &ws);
 // buffers of k_tile / k_cross (build_faces points at them).
 size_t build_workspace_bytes(uint32_t nx, uint32_t ny, uint32_t nz);
 uint32_t *build_faces(void *base, uint64_t n);
+// Where a build of configuration cfg may leave its pairs' bits, behind the tile
+// records in the workspace; null if the rows of its tiles do not fill whole
+// 16-bit pieces of them.
+uint32_t *build_mask(uint32_t *faces, uint32_t nx, uint32_t ny, uint32_t nz, uint32_t cfg);
 // u32 entries of one tile's face buffer for tile variant v, and tile counts
 uint32_t face_words(int variant);
 uint64_t tile_count(int variant, uint32_t nx, uint32_t ny, uint32_t nz);
@@ -110,10 +118,11 @@ cudaError_t launch_build(const float *f, uint64_t *W, uint32_t nx, uint32_t ny, 
 // f, sg, eps: persistence simplification (pairs of persistence below eps
 // dropped; eps <= 0 keeps all and does not read f). out: mapped host memory
 // that receives meta[0..2] and the status word (as readback's), or null.
-// clear: clear the counters first (false: the caller has)
+// clear: clear the counters first (false: the caller has); marked: ws.mask and
+// the roots are there already (LabelArgs)
 cudaError_t launch_pairs(const uint64_t *W, uint64_t n, uint32_t *pairs, uint64_t cap, Workspace &ws,
                          cudaStream_t st, const float *f = nullptr, float sg = 1.0f, float eps = 0.0f,
-                         uint64_t *out = nullptr, bool clear = true);
+                         uint64_t *out = nullptr, bool clear = true, bool marked = false);
 
 // Batched build and pairs over a packed descriptor table already in device
 // memory; cfg holds the MT_CFG_* knobs (mt_build.cu, mt_query.cu).

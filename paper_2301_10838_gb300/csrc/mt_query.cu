@@ -114,6 +114,31 @@ __global__ void __launch_bounds__(kCompactThreads, std::is_same<Loc, OneField>::
     }
 }
 
+// Counts of the chunks whose bits the build has left (a warp per chunk); the
+// bits past the field's end are cleared.
+__global__ void __launch_bounds__(kCompactThreads) k_mask_count(uint32_t *mask, uint64_t n, uint64_t nchunks,
+                                                                uint32_t *counts, const uint32_t *status)
+{
+    if (block_skips(status)) return;
+    const uint64_t c = (uint64_t)blockIdx.x * kCompactWarps + (threadIdx.x >> 5);
+    if (c >= nchunks) return;
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t *m = mask + c * (kCompactChunk / 32), sum = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < kCompactChunk / 32; k += 32) {
+        const uint64_t u = c * kCompactChunk + (k + lane) * 32;  // the word's first vertex
+        uint32_t w = 0;
+        if (u < n) w = m[k + lane];
+        if (u + 32 > n) {
+            if (u < n) w &= (1u << (n - u)) - 1u;
+            m[k + lane] = w;
+        }
+        sum += __popc(w);
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) counts[c] = sum;
+}
+
 // Exclusive scan of one field's chunk counts in place (one CTA of 1024
 // threads per field); the field's total goes to its meta[0] and, in a batch,
 // to npairs[field]. Warp w owns a contiguous range of chunks and reads it in
@@ -256,12 +281,15 @@ __global__ void __launch_bounds__(kCompactThreads) k_pairs_write(Loc loc, const 
 template <class Loc>
 static cudaError_t run_pairs(const Loc &loc, uint32_t nfields, uint64_t nchunks, uint32_t *counts, uint32_t *mask,
                              uint64_t *npairs, const uint32_t *status, cudaStream_t st, float eps = 0.0f,
-                             uint64_t *out = nullptr)
+                             uint64_t *out = nullptr, uint64_t marked = 0)
 {
     PhaseScope ps(kPairs, st);
     const bool simp = eps > 0.0f;
     const unsigned grid = (unsigned)nchunks;
-    if (simp) k_pairs_count<Loc, true><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
+    if (marked)  // the number of vertices
+        k_mask_count<<<(unsigned)((nchunks + kCompactWarps - 1) / kCompactWarps), kCompactThreads, 0, st>>>(
+            mask, marked, nchunks, counts, status);
+    else if (simp) k_pairs_count<Loc, true><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
     else k_pairs_count<Loc, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -282,7 +310,7 @@ static cudaError_t run_pairs(const Loc &loc, uint32_t nfields, uint64_t nchunks,
 }
 
 cudaError_t launch_pairs(const uint64_t *W, uint64_t n, uint32_t *pairs, uint64_t cap, Workspace &ws,
-                         cudaStream_t st, const float *f, float sg, float eps, uint64_t *out, bool clear)
+                         cudaStream_t st, const float *f, float sg, float eps, uint64_t *out, bool clear, bool marked)
 {
     if (clear) {
         const cudaError_t e = cudaMemsetAsync(ws.meta, 0, 3 * sizeof(uint64_t), st);
@@ -297,7 +325,7 @@ cudaError_t launch_pairs(const uint64_t *W, uint64_t n, uint32_t *pairs, uint64_
     loc.d.cap = cap;
     loc.d.f = f;
     loc.d.sg = sg;
-    return run_pairs(loc, 1, ws.nchunks, ws.counts, ws.mask, nullptr, ws.status, st, eps, out);
+    return run_pairs(loc, 1, ws.nchunks, ws.counts, ws.mask, nullptr, ws.status, st, eps, out, marked ? n : 0);
 }
 
 cudaError_t launch_batch_pairs(const FieldDesc *d_descs, uint32_t nfields, uint64_t nchunks, uint32_t *counts,
