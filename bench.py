@@ -132,17 +132,19 @@ class ClockSampler:
 
 # ------------------------------------------------------------ algorithmic bytes
 def algorithmic_bytes(n: int, shape, npairs: int, tile=(16, 16, 16), fused: bool = True) -> dict:
-    """Bytes the method must move per step, by kernel:
-      tile    init: read f (4n) + write W (8n); plus two triplet reads per
-              merged edge inside the tiles, 16 (E' - C)
-      merge   (k_cross) two triplet reads per edge between tiles: 16 C
+    """Bytes the step cannot do without, by kernel:
+      tile    read f (4n) + write W (8n); the edges inside a tile are merged
+              in shared memory
+      merge   (k_cross) the values of both ends of every edge between tiles:
+              8 C (most of these edges are then left out)
       repair  read + write W (16n); labelling inside it (fused): + read f
               (4n) + write labels (4n)
-      pairs   scan W (8n) + write pairs (8 npairs)
+      pairs   fused: the bits the repair pass left (n/8), the triplets of
+              pairs (8 npairs) and the pairs (8 npairs); else scan W (8n) +
+              write pairs (8 npairs)
       labels  (separate pass) read f (4n) + W (8n), write labels (4n)
-    E' = E - (n - #minima) (edges that are not steepest-descent seeds: the
-    per-edge cost of the edge loop of Algorithm 1) and C the edges between
-    tiles; tile + merge together are 12n + 16E'.
+    E' = E - (n - #minima) is the number of edges that are not descent seeds,
+    C the number of edges between tiles.
     """
     nz, ny, nx = shape
     tz, ty, tx = tile
@@ -150,9 +152,9 @@ def algorithmic_bytes(n: int, shape, npairs: int, tile=(16, 16, 16), fused: bool
     nmin = npairs + 1
     Ep = E - (n - nmin)
     C = ((nx - 1) // tx) * ny * nz + ((ny - 1) // ty) * nx * nz + ((nz - 1) // tz) * nx * ny
-    return {"tile": 12 * n + 16 * (Ep - C), "merge": 16 * C, "repair": 24 * n if fused else 16 * n,
-            "pairs": 8 * n + 8 * npairs, "labels": 0 if fused else 16 * n, "E": E, "E_prime": Ep,
-            "cross_edges": C}
+    return {"tile": 12 * n, "merge": 8 * C, "repair": 24 * n if fused else 16 * n,
+            "pairs": n // 8 + 16 * npairs if fused else 8 * n + 8 * npairs, "labels": 0 if fused else 16 * n,
+            "E": E, "E_prime": Ep, "cross_edges": C}
 
 
 def kernel_source_digest(kernel: str) -> str:

@@ -17,8 +17,10 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 //   [0, 256)     status word, round flag
 //   [256, 512)   meta: npairs, number of roots, root
 //   [512, ...)   per-chunk counts of the ordered compaction
-//   then, for a build, the face buffers (face_words(v) u32 per tile of the
-//   tile shape v in use: 16^3, or 32x16x16 with MT_CFG_LARGE_TILES)
+//   then, for a build, face_words(v) u32 per tile of the tile shape v in use
+//   (16^3, or 32x16x16 with MT_CFG_LARGE_TILES): the tiles' records one after
+//   another, then a bit per vertex (build_mask). The pair compaction of a
+//   later call puts its own bits over the records.
 size_t workspace_bytes(uint64_t n)
 {
     const uint64_t nchunks = (n + kCompactChunk - 1) / kCompactChunk;

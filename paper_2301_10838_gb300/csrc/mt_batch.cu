@@ -26,7 +26,7 @@ size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 //   descriptor tables for tile variants 0 and 1 (nfields each)
 //   per-field meta (npairs, number of roots, root)
 //   per-chunk counts of the pair compaction
-//   face buffers of the tiles (sized for the larger of the two variants)
+//   records of the tiles (sized for the larger of the two variants)
 struct Layout {
     size_t descs[2], meta, counts, faces, total;
     uint32_t tiles[2];

@@ -1,7 +1,7 @@
 // Kernels that build the triplet merge tree (Algorithm 1 of the paper):
-//   k_tile     per tile, in shared memory: initialisation seeded with the
-//              lowest lower neighbour, descent pointer jumping, Merge of the
-//              in-tile edges, Repair
+//   k_tile     per tile, in shared memory: initialisation seeded with a lower
+//              neighbour, descent pointer jumping, Merge of the in-tile
+//              edges, Repair of the tile's minima
 //   k_cross    Merge (Algorithm 3) of the edges between tiles, 64-bit CAS
 //   k_repair   Repair (Algorithm 5) via Representative (Algorithm 4); in
 //              mt_build_components also the components of G_t
@@ -23,8 +23,8 @@ namespace mt {
 // Algorithm 1 may merge the edges in any order. This kernel merges first the
 // edges inside each tile: it loads the tile's values into shared memory
 // (coalesced float4 rows), builds the triplet tree of the tile's own subgraph
-// with the lock-free Merge (32-bit CAS on shared memory, local ids packed as
-// (s << 16) | v), repairs it, and writes it out as global triplets. Local ids
+// with the lock-free Merge (64-bit CAS on link words in shared memory), repairs
+// its minima and writes these out as global triplets. Local ids
 // l = lx + TX * (ly + TY * lz) order the tile's vertices exactly as their
 // global linear indices do, so ties break identically. Values are kept as
 // 32-bit keys whose unsigned order is the float order (-0 and +0 share one
@@ -52,25 +52,27 @@ namespace mt {
 // shared memory, and the components are then flooded for all vertices of the
 // column at once, one LOP3 per word and square.
 //
-// Repair. After the merges the branch minima are repaired (Algorithm 5), then
-// every inner vertex l climbs from its descent minimum to its final tile
-// triplet (l, deepest vertex below l), 1.6 links on average, which goes
-// straight to global memory.
+// What leaves the kernel. After the merges the branch minima are repaired
+// (Algorithm 5) and written as global triplets: a valid normalised triplet
+// tree of the minima in the full grid minus the edges between tiles, which
+// k_cross merges next. An inner vertex takes no part in those merges, so its
+// word only says which minimum of the tile it descends to (kInner, local id);
+// k_repair gives it its triplet, once, when the tree is whole. (Repaired here
+// as well it climbed 1.6 links on average, for 3.8 ms at 1024^3.)
 //
 // What it costs. The kernel is bound by instruction issue (75 % of the issue
-// slots, HBM 7 % busy): 12.5 warp instructions per vertex. On the 1024^3
-// lognormal field it takes 14.5 ms: loads 1.2, relations 0.7, components 1.0,
-// edge list 0.7, descent 1.1, merges 3.5, minima 0.6, inner vertices 3.8,
-// faces 1.8. The earlier design, which kept every edge whose ends descend to
-// different minima and settled most of them by comparing cached climbs in 8
-// rounds over level buckets, took 31.5 ms (29 warp instructions per vertex).
+// slots, HBM 16 % busy). On the 1024^3 lognormal field it takes 11.7 ms: loads
+// 1.2, relations 0.7, components 1.0, edge list 0.7, descent 1.1, merges 3.5,
+// minima 0.6, faces and the words of the inner vertices 2.9. The earlier
+// design, which kept every edge whose ends descend to different minima and
+// settled most of them by comparing cached climbs in 8 rounds over level
+// buckets, took 31.5 ms (29 warp instructions per vertex).
 // The climbs and merges are loops whose lanes stay together by votes: with
-// ordinary divergent loops the same algorithm took 24.0 ms, since a warp
-// whose lanes left a loop one by one ran what follows it once per group.
-//
-// What leaves the kernel is, for every vertex, its triplet in the subgraph
-// induced by its tile: a valid normalised triplet tree of the full grid minus
-// the edges between tiles, which k_cross merges next.
+// ordinary divergent loops the same algorithm took 24.0 ms against 14.5, since
+// a warp whose lanes left a loop one by one ran what follows it once per
+// group. The merges by 4, 3 or 2 of the 8 warps took 12.0, 11.9 and 14.1 ms,
+// merges from each column's own words without the list 13.6, the faces'
+// values loaded before the merges or before the minima's repair 12.5 and 12.7.
 constexpr int log2i(int x) { return x <= 1 ? 0 : 1 + log2i(x / 2); }
 
 template <int LX, int LY, int LZ>

@@ -21,7 +21,7 @@ struct FieldDesc {
     uint64_t *W;       // triplets, field-local vertex ids
     uint32_t *pairs;   // pair output ([cap][2]) or null
     uint64_t *meta;    // [0] npairs, [1] number of roots, [2] root
-    uint32_t *faces;   // per tile: tile-local tops of the cross-edge ends, or null
+    uint32_t *faces;   // the tiles' records (kept edges of their faces, notes for the repair pass)
     uint64_t n, cap;   // vertices, pair capacity
     uint64_t chunk0;   // first compaction chunk of the field
     uint32_t nx, ny, nz;
@@ -46,7 +46,6 @@ struct LabelArgs {
 struct Workspace {
     uint32_t *status;  // status bits (ST_*)
     uint64_t *meta;    // [0] npairs, [1] number of roots, [2] root
-    uint32_t *faces;   // per tile: tile-local tops of the cross-edge ends, or null vertex
     uint32_t *counts;  // per-chunk counts, then exclusive offsets in place
     uint32_t *mask;    // a bit per vertex for the pair compaction, or null
     uint64_t nchunks;
@@ -72,15 +71,16 @@ class PhaseScope {
 // The pair-compaction part of a workspace (status, counters, chunk counts)...
 size_t workspace_bytes(uint64_t n);
 bool carve_workspace(void *base, size_t bytes, uint64_t n, Workspace &ws);
-// ...and the whole workspace a build needs: that part followed by the face
-// buffers of k_tile / k_cross (build_faces points at them).
+// ...and the whole workspace a build needs: that part followed by the tiles'
+// records (build_faces points at them).
 size_t build_workspace_bytes(uint32_t nx, uint32_t ny, uint32_t nz);
 uint32_t *build_faces(void *base, uint64_t n);
 // Where a build of configuration cfg may leave its pairs' bits, behind the tile
 // records in the workspace; null if the rows of its tiles do not fill whole
 // 16-bit pieces of them.
 uint32_t *build_mask(uint32_t *faces, uint32_t nx, uint32_t ny, uint32_t nz, uint32_t cfg);
-// u32 entries of one tile's face buffer for tile variant v, and tile counts
+// u32 entries the workspace has per tile of variant v (its record, stored
+// without gaps, and a bit per vertex behind all records), and tile counts
 uint32_t face_words(int variant);
 uint64_t tile_count(int variant, uint32_t nx, uint32_t ny, uint32_t nz);
 int device_sms();
