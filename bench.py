@@ -89,13 +89,18 @@ class ClockSampler:
     def start(self):
         try:
             self.proc = subprocess.Popen(
-                ["nvidia-smi", f"--query-gpu={self.FIELDS}", "--format=csv,noheader,nounits", "-lms", "200",
+                ["nvidia-smi", f"--query-gpu={self.FIELDS}", "--format=csv,noheader,nounits", "-lms", "100",
                  "-i", str(self.index)], stdout=subprocess.PIPE, stderr=subprocess.DEVNULL, text=True)
         except OSError:
             self.proc = None
             return
         self.t = threading.Thread(target=self._read, daemon=True)
         self.t.start()
+        # nvidia-smi's own start holds up launches (40 ms of ten 29 ms steps):
+        # the timed region begins with its first sample
+        end = time.time() + 5
+        while not self.lines and time.time() < end and self.proc.poll() is None:
+            time.sleep(0.01)
 
     def _read(self):
         for line in self.proc.stdout:
@@ -301,8 +306,8 @@ def run_ours(args):
     mt.mt_trace_enable(True)
     mt.mt_trace_read(reset=True)
     launches0 = mt.mt_kernel_launches()
-    barrier()
     clocks.start()
+    barrier()
     ev0 = torch.cuda.Event(enable_timing=True)
     ev1 = torch.cuda.Event(enable_timing=True)
     ev0.record(stream)

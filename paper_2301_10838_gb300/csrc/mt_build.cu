@@ -60,8 +60,8 @@ namespace mt {
 // k_repair gives it its triplet, once, when the tree is whole. (Repaired here
 // as well it climbed 1.6 links on average, for 3.8 ms at 1024^3.)
 //
-// What it costs. The kernel is bound by instruction issue (75 % of the issue
-// slots, HBM 16 % busy). On the 1024^3 lognormal field it takes 11.7 ms: loads
+// What it costs. The kernel is bound by instruction issue (73 % of the issue
+// slots, HBM 15 % busy). On the 1024^3 lognormal field it takes 11.7 ms: loads
 // 1.2, relations 0.7, components 1.0, edge list 0.7, descent 1.1, merges 3.5,
 // minima 0.6, faces and the words of the inner vertices 2.9. The earlier
 // design, which kept every edge whose ends descend to different minima and
