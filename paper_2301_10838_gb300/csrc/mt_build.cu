@@ -828,11 +828,56 @@ struct RepairShape {
     static constexpr int kWant = (LAB || WIDE ? 1536 : 1792) / NT, kCTAs = kFit < kWant ? kFit : kWant;
 };
 
+// A build that failed (a value is not finite, a loop ran out of steps) leaves
+// valid ids behind too: the inner vertices of the tile, whose words still hold
+// local ids, become roots, so that a later call on the triplets reads nothing
+// out of range. The repair kernel of a single field does this where it skips;
+// in batches and with wide ids the call made it spill registers (687 -> 718,
+// 1406 -> 1490 us), so there a kernel of its own looks at the status word, 5 us.
+template <class Loc, bool WIDE>
+constexpr bool kLeaveApart = WIDE || !std::is_same<Loc, OneField>::value;
+
+template <int LX, int LY, int LZ, bool WIDE>
+__device__ __noinline__ void leave_valid(uint64_t *W, uint32_t nx, uint32_t ny, uint32_t nz, uint32_t ntx, uint32_t nty,
+                                         uint32_t tile)
+{
+    using TR = Tri<WIDE>;
+    using Id = typename TR::Id;
+    constexpr uint32_t TX = 1u << LX, TY = 1u << LY, TZ = 1u << LZ;
+    const uint32_t x = tile % ntx * TX + (threadIdx.x & (TX - 1)),
+                   y = tile / ntx % nty * TY + (threadIdx.x >> LX), z0 = tile / (ntx * nty) * TZ;
+    if (x >= nx || y >= ny) return;
+    for (uint32_t z = z0; z < min(z0 + TZ, nz); z++) {
+        const Id u = ((Id)z * ny + y) * nx + x;
+        Id s, v;
+        TR::load(W, u, s, v);
+        if (s == TR::kInner) s = v = u;
+        TR::store(W, u, s, v);  // wide: without the merges' tags
+    }
+}
+template <int LX, int LY, int LZ, class Loc, bool WIDE>
+__global__ void __launch_bounds__(1 << (LX + LY)) k_leave_valid(Loc loc, uint32_t ntiles, const uint32_t *status)
+{
+    if (block_skips(status))
+        for (uint32_t b = blockIdx.x; b < ntiles; b += gridDim.x) {
+            uint32_t t;
+            const FieldDesc d = loc.tile(b, t);
+            leave_valid<LX, LY, LZ, WIDE>(d.W, d.nx, d.ny, d.nz, d.ntx, d.nty, t);
+        }
+}
+
 template <int LX, int LY, int LZ, class Loc, bool LAB, bool WIDE = false>
 __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, WIDE>::kCTAs)
     k_repair(Loc loc, uint32_t *status, const LabelArgs la)
 {
-    if (block_skips(status)) return;
+    if (block_skips(status)) {
+        if constexpr (!kLeaveApart<Loc, WIDE>) {
+            uint32_t t;
+            const FieldDesc d = loc.tile(blockIdx.x, t);
+            leave_valid<LX, LY, LZ, WIDE>(d.W, d.nx, d.ny, d.nz, d.ntx, d.nty, t);
+        }
+        return;
+    }
     static_assert(!(LAB && WIDE), "labels have 32-bit ids");
     using RS = RepairShape<LX, LY, LZ, LAB, WIDE>;
     using TR = Tri<WIDE>;
@@ -1306,6 +1351,11 @@ static cudaError_t launch_repair(const Loc &loc, uint32_t ntiles, uint32_t *stat
     }
     kern<<<ntiles, RS::NT, RS::kSmem, st>>>(loc, status, la);
     count_launch();
+    if constexpr (kLeaveApart<Loc, WIDE>) {
+        const uint32_t grid = ntiles < 608u ? ntiles : 608u;
+        k_leave_valid<VV::LX, VV::LY, VV::LZ, Loc, WIDE><<<grid, RS::NT, 0, st>>>(loc, ntiles, status);
+        count_launch();
+    }
     return cudaGetLastError();
 }
 
