@@ -1071,7 +1071,11 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
     // below a level, a comparison of the words as in the tile kernel. Where the
     // link's saddle or the level's lies outside the tile, its local id is NONE
     // and the comparison is by key alone; on equal keys the ids decide, read
-    // from W.
+    // from W. While a lane can go on by the words alone, lanes that need the ids
+    // wait, so a warp's rounds may add up to all its lanes' links, each lane
+    // passing a node at most once; a climb that is not done by then raises
+    // ST_TIMEOUT.
+    constexpr uint32_t kRounds = 32 * (NN + 1);
     auto link_next = [](uint64_t w) { return (uint32_t)w & 0xFFFFu; };
     auto saddle_before = [&](uint32_t x, Id S) -> bool {
         Id s, v;
@@ -1106,7 +1110,11 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
         const uint64_t lim = sl != NONE ? w | 0xFFFFu : ((uint64_t)ks << 32) - 1;
         uint32_t x = link ? x0 : NN;
         uint64_t wx_ = vword[x];
-        for (uint32_t h = 0; h < 2 * NN; h++) {
+        for (uint32_t h = 0;; h++) {
+            if (h == kRounds) {
+                ok = false;
+                break;
+            }
             const bool go = wx_ <= lim && link;
             if (!__any_sync(0xffffffffu, go)) {
                 bool tie = link && (uint32_t)(wx_ >> 32) == ks && (sl == NONE || (uint32_t)wx_ >= 0xFFFF0000u);
@@ -1229,7 +1237,11 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
         const uint64_t lim = inner ? level_word(ku, l) : 0u;
         uint32_t x = inner || (LAB && inx && ((minima >> z) & 1u)) ? node[m >> 1] : NN;
         uint64_t w = word[x];
-        for (uint32_t h = 0; h < 2 * NN; h++) {
+        for (uint32_t h = 0;; h++) {
+            if (h == kRounds) {
+                ok = false;
+                break;
+            }
             const bool go = w <= lim;
             if (!__any_sync(0xffffffffu, go)) {
                 // a link of the same key whose saddle lies outside the tile?
