@@ -11,6 +11,7 @@
 
 #include "mt_device.cuh"
 #include "mt_fields.cuh"
+#include "mt_index.h"
 #include "mt_internal.h"
 
 namespace mt {
@@ -885,7 +886,7 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
     constexpr uint32_t TX = 1u << LX, TY = 1u << LY, TZ = 1u << LZ, TV = RS::TV, NT = RS::NT, MIN = RS::kMin,
                        HS = RS::kHash, NN = RS::kNodes;
     static_assert((HS & (HS - 1)) == 0, "power of two");
-    constexpr uint32_t NONE = 0xFFFFu;             // no node, no local id
+    constexpr uint32_t NONE = kNoLocal;            // no node, no local id
     constexpr Id EMPTY = ~(Id)0;                   // free hash slot (no vertex id)
     constexpr uint32_t kProbes = 16;
     // word of a node whose target found no node, and of node NN, which stands
@@ -923,24 +924,9 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
     const Id ucol = base + (Id)cy * nx + cx;       // vertex z of the column: ucol + z * nxy
     bool ok = true;
     auto val = [&](Id u) { return sg * __ldg(f + u); };
-    // local id of vertex v, NONE outside the tile. Within the tile's span the
-    // quotients are below 16, so a product with the reciprocal is off by at
-    // most one, which the remainder shows.
+    // local id of vertex v, NONE outside the tile
     const float rnxy = 1.0f / (float)nxy, rnx = 1.0f / (float)nx;
-    auto local_of = [&](Id v) -> uint32_t {
-        const Id rel = v - base;                   // wraps far beyond the tile for an earlier vertex
-        if ((uint64_t)rel >= (uint64_t)TZ * nxy) return NONE;
-        uint32_t dz = (uint32_t)((float)rel * rnxy);
-        if ((Id)dz * nxy > rel) dz--;
-        Id r = rel - (Id)dz * nxy;
-        if (r >= nxy) dz++, r -= nxy;
-        if ((uint64_t)r >= (uint64_t)TY * nx) return NONE;
-        uint32_t dy = (uint32_t)((float)(uint32_t)r * rnx);
-        if (dy * nx > (uint32_t)r) dy--;
-        uint32_t dx = (uint32_t)r - dy * nx;
-        if (dx >= nx) dy++, dx -= nx;
-        return dx < wx && dy < wy && dz < wz ? dx + TX * (dy + TY * dz) : NONE;
-    };
+    auto local_of = [&](Id v) -> uint32_t { return tile_local<LX, LY, LZ, Id>(v - base, nxy, nx, rnxy, rnx, wx, wy, wz); };
     auto id_at = [&](uint32_t l) -> Id {
         return base + (Id)(l >> (LX + LY)) * nxy + (Id)((l >> LX) & (TY - 1)) * nx + (l & (TX - 1));
     };

@@ -1,0 +1,40 @@
+// Index arithmetic of the kernels that depends on nothing of the GPU, so that
+// the tests can run it on the CPU over grids of any size.
+#pragma once
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define MT_HD __host__ __device__ __forceinline__
+#else
+#define MT_HD inline
+#endif
+
+namespace mt {
+
+constexpr uint32_t kNoLocal = 0xFFFFu;  // no vertex of the tile
+
+// Local id, in a tile of (1 << LX, 1 << LY, 1 << LZ) vertices of which the
+// first (wx, wy, wz) lie in the grid, of the vertex whose id is `rel` above
+// that of the tile's first vertex (an Id that has wrapped for an earlier one);
+// kNoLocal outside the tile. Within the tile's span the quotients by nxy and
+// nx are at most 16, so a product with the reciprocal (rnxy, rnx) is off by at
+// most one, which the remainder shows. With 64-bit ids the remainder by nxy
+// may itself need more than 32 bits (nx above 2^28).
+template <int LX, int LY, int LZ, class Id>
+MT_HD uint32_t tile_local(Id rel, Id nxy, uint32_t nx, float rnxy, float rnx, uint32_t wx, uint32_t wy, uint32_t wz)
+{
+    constexpr uint32_t TX = 1u << LX, TY = 1u << LY, TZ = 1u << LZ;
+    if ((uint64_t)rel >= (uint64_t)TZ * nxy) return kNoLocal;
+    uint32_t dz = (uint32_t)((float)rel * rnxy);
+    if ((Id)dz * nxy > rel) dz--;
+    Id r = rel - (Id)dz * nxy;
+    if (r >= nxy) dz++, r -= nxy;
+    if ((uint64_t)r >= (uint64_t)TY * nx) return kNoLocal;
+    uint32_t dy = (uint32_t)((float)r * rnx);
+    if ((Id)dy * nx > r) dy--;
+    Id dx = r - (Id)dy * nx;
+    if (dx >= nx) dy++, dx -= nx;
+    return dx < wx && dy < wy && dz < wz ? (uint32_t)dx + TX * (dy + TY * dz) : kNoLocal;
+}
+
+}  // namespace mt
