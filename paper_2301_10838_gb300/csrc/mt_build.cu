@@ -848,8 +848,9 @@ __device__ __noinline__ void leave_valid(uint64_t *W, uint32_t nx, uint32_t ny, 
     const uint32_t x = tile % ntx * TX + (threadIdx.x & (TX - 1)),
                    y = tile / ntx % nty * TY + (threadIdx.x >> LX), z0 = tile / (ntx * nty) * TZ;
     if (x >= nx || y >= ny) return;
-    for (uint32_t z = z0; z < min(z0 + TZ, nz); z++) {
-        const Id u = ((Id)z * ny + y) * nx + x;
+    const uint32_t wz = tile_side(z0, TZ, nz);
+    for (uint32_t z = 0; z < wz; z++) {
+        const Id u = ((Id)(z0 + z) * ny + y) * nx + x;
         Id s, v;
         TR::load(W, u, s, v);
         if (s == TR::kInner) s = v = u;

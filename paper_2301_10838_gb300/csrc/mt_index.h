@@ -13,6 +13,10 @@ namespace mt {
 
 constexpr uint32_t kNoLocal = 0xFFFFu;  // no vertex of the tile
 
+// Vertices of the grid, n along an axis, in a tile of T that begins at o < n.
+// (o + T may wrap where n is within T of 2^32.)
+MT_HD uint32_t tile_side(uint32_t o, uint32_t T, uint32_t n) { return n - o < T ? n - o : T; }
+
 // Local id, in a tile of (1 << LX, 1 << LY, 1 << LZ) vertices of which the
 // first (wx, wy, wz) lie in the grid, of the vertex whose id is `rel` above
 // that of the tile's first vertex (an Id that has wrapped for an earlier one);

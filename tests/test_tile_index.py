@@ -1,4 +1,4 @@
-"""The repair pass's local ids against exact division, on the CPU.
+"""The repair pass's local ids and tile sides against exact arithmetic, on the CPU.
 
 csrc/mt_index.h finds a vertex's place in its tile by reciprocals; here it is
 compiled for the host and compared with 64-bit division, with 32-bit and 64-bit
@@ -70,6 +70,14 @@ void both(u64 nx, u64 ny, u64 nz)
 
 int main()
 {
+    // the last tiles of axes up to 2^32 - 1 long
+    const u64 axis[] = {1, 15, 16, 17, 4294967279u, 4294967280u, 4294967281u, 4294967295u};
+    for (u64 n : axis)
+        for (u64 o = n > 64 ? (n - 64) / 16 * 16 : 0; o < n; o += 16) {
+            const u64 want = n - o < 16 ? n - o : 16;
+            if (tile_side((uint32_t)o, 16, (uint32_t)n) != want && bad++ < 5)
+                printf("axis of %llu: not %llu vertices in the tile at %llu\n", n, want, o);
+        }
     const u64 side[] = {1, 2, 3, 15, 16, 17, 33, 509, 1024, 65535, 65536, (1u << 28) - 1, (1u << 28) + 1,
                         (1u << 29) + 16, 1431655764, 2147483648u, 3000000019u, 4294967295u};
     for (u64 a : side)
