@@ -357,8 +357,8 @@ cudaError_t launch_batch_pairs(const FieldDesc *d_descs, uint32_t nfields, uint6
 // entered; loops kept together by votes, which serve the build's kernels,
 // 406: nearly every probe succeeds at once). 3 CTAs per SM: 406.
 //
-// WIDE: 64-bit ids (the wide path's triplets and labels; 1.0 ms for 512^3, 1.7
-// with a chase per vertex).
+// WIDE: 64-bit ids (the wide path's triplets and labels). Grids of which a
+// brick holds too little take k_labels_each instead (see bricks_pay).
 //
 // With eps > 0 the labels are those of the simplified field in which every
 // branch of persistence below eps is filled up to its saddle: a component of
@@ -552,6 +552,57 @@ __global__ void __launch_bounds__(kLabThreads, 4) k_labels(const float *__restri
     if (bad) raise_status(status, ST_CORRUPT);
 }
 
+// The labels of a wide field, each vertex following its own chain. Where many
+// vertices of a neighbourhood share their chains the bricks of k_labels read
+// them less often, but a brick with few vertices in it, or a field whose
+// triplets stay in L2, costs less this way.
+__global__ void __launch_bounds__(256) k_labels_each(const float *f, float sg, const uint64_t *W, uint64_t n, float t,
+                                                     uint64_t *labels, uint32_t *status)
+{
+    if (*status) return;
+    bool ok = true, bad = false;
+    for (uint64_t u = blockIdx.x * 256ull + threadIdx.x; u < n; u += gridDim.x * 256ull) {
+        if (!(sg * __ldg(f + u) <= t)) {
+            labels[u] = ~0ull;
+            continue;
+        }
+        const ulonglong2 wu = reinterpret_cast<const ulonglong2 *>(W)[u];
+        uint64_t x = wu.x == u && wu.y != u && wu.y < n ? wu.y : u;
+        for (uint64_t h = 0;; h++) {
+            const ulonglong2 w = reinterpret_cast<const ulonglong2 *>(W)[x];
+            if (w.x == x && w.y == x) break;
+            if (w.x >= n || w.y >= n) {
+                bad = true;
+                break;
+            }
+            if (!(sg * __ldg(f + w.x) <= t)) break;
+            x = w.y;
+            if (h >= kChaseLimit || h >= n) {
+                ok = false;
+                break;
+            }
+        }
+        labels[u] = x;
+    }
+    if (!ok) raise_status(status, ST_TIMEOUT);
+    if (bad) raise_status(status, ST_CORRUPT);
+}
+
+// Whether wide labels take the bricks: from 2^23 vertices, four planes and
+// columns of which three in four lie in the grid. Measured in us, each vertex
+// by itself against bricks, white noise at its median: 160^3 83 and 114, 256^3
+// 252 and 201, 512^3 2516 and 1424; planes of 8192^2 741 and 1294, 4 of them
+// 7044 and 2952; 1024 x 1024 rows of 8 132 and 184, of 24 426 and 292, of 33
+// 612 and 477 (16 levels: 382 and 432). Smooth fields, where every chain is
+// short, lose up to 9 % to the bricks (320^3 148 and 161), fields of which
+// half the vertices are minima up to a factor of two (512^3 829 and 1672).
+static bool bricks_pay(uint32_t nx, uint32_t ny, uint32_t nz, uint32_t ntx, uint32_t nty)
+{
+    if (kLabelShrink > 1) return true;  // the tests' small tables are meant to be reached by small fields
+    const uint64_t n = (uint64_t)nx * ny * nz;
+    return n >= 1u << 23 && nz >= 4 && 4 * (uint64_t)nx * ny >= 3 * (uint64_t)ntx * nty * kLabThreads;
+}
+
 template <bool WIDE>
 static cudaError_t run_labels(const float *f, const uint64_t *W, uint32_t nx, uint32_t ny, uint32_t nz, float t,
                               float sg, typename Tri<WIDE>::Id *labels, uint32_t *status, cudaStream_t st, float eps)
@@ -559,6 +610,14 @@ static cudaError_t run_labels(const float *f, const uint64_t *W, uint32_t nx, ui
     PhaseScope ps(kLabels, st);
     const uint32_t ntx = (uint32_t)(((uint64_t)nx + 31) >> kLabLX), nty = (uint32_t)(((uint64_t)ny + 15) >> kLabLY),
                    ntz = (uint32_t)(((uint64_t)nz + 15) >> kLabLZ);
+    if constexpr (WIDE) {
+        if (!bricks_pay(nx, ny, nz, ntx, nty)) {
+            const uint64_t n = (uint64_t)nx * ny * nz, want = (n + 2047) / 2048, most = (uint64_t)device_sms() * 16;
+            k_labels_each<<<(unsigned)(want < most ? want : most), 256, 0, st>>>(f, sg, W, n, t, labels, status);
+            count_launch();
+            return cudaGetLastError();
+        }
+    }
     static AttrFlags attr;  // per instantiation
     int dev;
     if (attr.pending(dev)) {
