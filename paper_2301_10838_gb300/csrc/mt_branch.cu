@@ -65,7 +65,7 @@ constexpr uint64_t kSortFew = 1u << 21;
 // Counters in the workspace.
 struct BranchMeta {
     uint32_t root, rstart;              // the root's branch and where its group starts
-    uint32_t nlarge, pad;               // large branches other than one sorted apart
+    uint32_t nlarge, lstart0;           // large branches other than one sorted apart, where the first starts
     uint32_t nbranch, nl[2];            // branches; vertices of the root's branch and of the large ones
     uint32_t kor[2], kand[2];           // OR and AND of their keys
 };
@@ -298,6 +298,7 @@ __global__ void __launch_bounds__(256) k_br_starts(uint32_t *cnt, const uint32_t
             } else if (c[r] > kSmall) {
                 const uint32_t k = atomicAdd(&meta->nlarge, 1u);
                 lstart[k] = start, lsize[k] = c[r];
+                if (k == 0) meta->lstart0 = start;
                 atomicOr(lbits + (u >> 5), 1u << (u & 31));
                 cnt[u] = k;
             } else {
@@ -858,23 +859,26 @@ mt_status mt_branch_decomposition(const float *d_f, const uint64_t *d_W, mt_grid
     if (bits) return status_from_bits(bits);
     const uint64_t n0 = m.nl[0], n1 = m.nl[1];
     // arrays of the sorts, carved from the pool (at most 16 bytes per vertex;
-    // 64 words of slack for alignment): the root's branch keeps its ids in
-    // its own place in d_order every other pass, so that they end there
+    // 64 words of slack for alignment). The root's branch, and a single large
+    // one, keep their ids in their own place in d_order every other pass, so
+    // that they end there.
     uint32_t *p = bw.pool;
     auto carve = [&](uint64_t words) {
         uint32_t *q = p;
         p += (words + 31) & ~31ull;
         return q;
     };
+    const bool one = m.nlarge == 1;
     uint32_t *ka = carve(n0), *kb = carve(n0), *ia = carve(n0), *ib = d_order + m.rstart;
-    uint32_t *ka1 = carve(n1), *kb1 = carve(n1), *ia1 = carve(n1), *ib1 = carve(n1);
+    uint32_t *ka1 = carve(n1), *kb1 = carve(n1), *ia1 = carve(n1), *ib1 = one ? d_order + m.lstart0 : carve(n1);
     uint32_t sh0[4], sh1[4];
     const int p0 = n0 ? digits(m.kor[0] ^ m.kand[0], sh0) : 0, p1 = n1 ? digits(m.kor[1] ^ m.kand[1], sh1) : 0;
-    if (p0 % 2 == 0) {  // an even number of passes starts in place
-        uint32_t *t = ka;
-        ka = kb, kb = t;
-        t = ia, ia = ib, ib = t;
-    }
+    auto swap = [](uint32_t *&a, uint32_t *&b) {
+        uint32_t *t = a;
+        a = b, b = t;
+    };
+    if (p0 % 2 == 0) swap(ka, kb), swap(ia, ib);  // an even number of passes starts in place
+    if (one && p1 % 2 == 0) swap(ka1, kb1), swap(ia1, ib1);
     if (n0 + n1) {
         k_br_compact<<<nchunks, 256, 0, st>>>(f, bw.mask0, bw.mask1, bw.heads, bw.sizes, n, ka, ia, ka1, ia1);
         count_launch();
@@ -883,35 +887,27 @@ mt_status mt_branch_decomposition(const float *d_f, const uint64_t *d_W, mt_grid
     for (int i = 0; i < p0 && e == cudaSuccess; i++) {
         e = i + 1 < p0 ? radix_pass<false>(ka, ia, kb, ib, (uint32_t)n0, sh0[i], bw, st)
                        : radix_pass<true>(ka, ia, kb, ib, (uint32_t)n0, sh0[i], bw, st);
-        uint32_t *t = ka;
-        ka = kb, kb = t;
-        t = ia, ia = ib, ib = t;
+        swap(ka, kb), swap(ia, ib);
     }
-    if (n1 && e == cudaSuccess) {
-        for (int i = 0; i < p1 && e == cudaSuccess; i++) {
-            e = i + 1 < p1 ? radix_pass<false>(ka1, ia1, kb1, ib1, (uint32_t)n1, sh1[i], bw, st)
-                           : radix_pass<true>(ka1, ia1, kb1, ib1, (uint32_t)n1, sh1[i], bw, st);
-            uint32_t *t = ka1;
-            ka1 = kb1, kb1 = t;
-            t = ia1, ia1 = ib1, ib1 = t;
-        }
+    for (int i = 0; i < p1 && e == cudaSuccess; i++) {
+        e = i + 1 < p1 ? radix_pass<false>(ka1, ia1, kb1, ib1, (uint32_t)n1, sh1[i], bw, st)
+                       : radix_pass<true>(ka1, ia1, kb1, ib1, (uint32_t)n1, sh1[i], bw, st);
+        swap(ka1, kb1), swap(ia1, ib1);
+    }
+    if (m.nlarge > 1 && e == cudaSuccess) {
         // then by branch: the keys become branch numbers; lsize becomes the
         // first place of each branch in the sorted array
         const uint64_t wantr = (n1 + 255) / 256, mostr = (uint64_t)device_sms() * 8;
-        if (e == cudaSuccess) {
-            k_br_rank<<<(unsigned)(wantr < mostr ? wantr : mostr), 256, 0, st>>>(d_W, n, bw.cnt, ia1, (uint32_t)n1, ka1);
-            k_br_scan2<<<1, 1024, 0, st>>>(bw.lsize, bw.lsize, m.nlarge, nullptr, nullptr);
-            count_launch(2);
-            e = cudaGetLastError();
-        }
+        k_br_rank<<<(unsigned)(wantr < mostr ? wantr : mostr), 256, 0, st>>>(d_W, n, bw.cnt, ia1, (uint32_t)n1, ka1);
+        k_br_scan2<<<1, 1024, 0, st>>>(bw.lsize, bw.lsize, m.nlarge, nullptr, nullptr);
+        count_launch(2);
+        e = cudaGetLastError();
         uint32_t last = 0;  // the highest digit of the branch numbers
         while (last < 24 && ((m.nlarge - 1) >> (last + 8))) last += 8;
         for (uint32_t s = 0; s <= last && e == cudaSuccess; s += 8) {
             e = s < last ? radix_pass<false>(ka1, ia1, kb1, ib1, (uint32_t)n1, s, bw, st)
                          : radix_pass<true>(ka1, ia1, kb1, d_order, (uint32_t)n1, s, bw, st, bw.lstart, bw.lsize);
-            uint32_t *t = ka1;
-            ka1 = kb1, kb1 = t;
-            t = ia1, ia1 = ib1, ib1 = t;
+            swap(ka1, kb1), swap(ia1, ib1);
         }
     }
     if (e != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return MT_ERR_CUDA;
