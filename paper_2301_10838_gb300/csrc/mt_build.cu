@@ -633,16 +633,30 @@ __global__ void __launch_bounds__(Tile<LX, LY, LZ>::NT, Tile<LX, LY, LZ>::kCTAs)
 // 93 of the 132 edges per tile on a lognormal field.
 //
 // The kernel is bound by the latency of its chains of dependent reads (a
-// quarter of the issue slots used, HBM 12 % busy): 4.8 ms on the 1024^3
-// lognormal field; 6.3 ms with a merge that read a vertex's value and a
-// re-inserted link's level only when it needed them, and without the hash;
-// 5.6 ms with the new merge alone. The fields of a batch are small enough
+// quarter of the issue slots used, HBM 12 % busy): 4.3 ms on the 1024^3
+// lognormal field, 4.6 with the tiles in order instead of scattered (256^3
+// white noise 143 and 155 us, of 16 values 165 and 240, a line of 2^18 constant
+// vertices 55 and 390); 6.3 ms with a merge that read a vertex's value and a
+// re-inserted link's level only when it needed them, in order and without the
+// hash; 5.6 ms with the new merge alone. The fields of a batch are small enough
 // for L2, where the hash costs more than the merges it saves (512 uneven
 // fields: 0.36 ms with it, 0.29 without), and 16 CTAs per SM run better than
 // the 12 that hide most of HBM's latency (0.39 ms with 11 CTAs, 0.29 with 16;
 // single field 4.8 ms with 12, 5.2 with 14).
+//
+// Steps before a merge goes on in the long form: 16 (8 and 32: 256^3 white noise
+// 148 and 144, of 16 values 169 and 183 us); in a batch, where the call alone
+// costs registers, 32 (2572 us with 16, 2570 with 32 and 64, 2560 without).
+constexpr uint32_t kShortField = 16, kShortBatch = 32;  // steps before the long form
+
+static __device__ __noinline__ bool merge_long(uint64_t *W, const Field f, uint32_t S, float fS, uint32_t u, uint32_t v)
+{
+    return merge_steps<true>(W, f, S, fS, u, v);
+}
+
 template <int LX, int LY, int LZ, class Loc>
-__global__ void __launch_bounds__(128, std::is_same<Loc, OneField>::value ? 12 : 16) k_cross(Loc loc, uint32_t *status)
+__global__ void __launch_bounds__(128, std::is_same<Loc, OneField>::value ? 12 : 16)
+    k_cross(Loc loc, uint32_t stride, uint32_t *status)
 {
     if (block_skips(status)) return;
     using TS = Tile<LX, LY, LZ>;
@@ -655,7 +669,8 @@ __global__ void __launch_bounds__(128, std::is_same<Loc, OneField>::value ? 12 :
     __shared__ uint16_t list[HS];
     __shared__ uint32_t s_n;
     uint32_t tile;
-    const FieldDesc fd = loc.tile(blockIdx.x, tile);
+    constexpr bool ONE = std::is_same<Loc, OneField>::value;
+    const FieldDesc fd = loc.tile(ONE ? (uint32_t)((uint64_t)blockIdx.x * stride % gridDim.x) : blockIdx.x, tile);
     const Field f{fd.f, fd.sg};
     constexpr uint32_t kWords = TS::template kTileWords<false>;
     const uint32_t *rec = fd.faces + (size_t)tile * kWords;
@@ -671,7 +686,7 @@ __global__ void __launch_bounds__(128, std::is_same<Loc, OneField>::value ? 12 :
         off[g] = incl - c0 - c1, off[g + 1] = incl - c1;
         if (threadIdx.x == 31) off[64] = incl, s_n = 0;
     }
-    constexpr bool DEDUP = std::is_same<Loc, OneField>::value;  // see above
+    constexpr bool DEDUP = ONE;  // see above
     if (DEDUP)
         for (uint32_t i = threadIdx.x; i < HS; i += NT) hkey[i] = EMPTY, hlev[i] = EMPTY;
     __syncthreads();
@@ -683,10 +698,11 @@ __global__ void __launch_bounds__(128, std::is_same<Loc, OneField>::value ? 12 :
             if (off[g + w] <= i) g += w;
         const uint32_t p = 16 * g + i - off[g];
         const uint32_t nb = g < GX ? 1u : g < GX + GY ? fd.ntx : fd.ntx * fd.nty;  // the neighbour tile
-        const uint32_t ta = rec[TS::kFaceHead + p], S = rec[TS::kFaceHead + 2 * TS::kFaceSide + p];
-        const uint32_t tb = rec[(size_t)nb * kWords + TS::kFaceHead + TS::kFaceSide + p];
+        uint32_t ta = rec[TS::kFaceHead + p], S = rec[TS::kFaceHead + 2 * TS::kFaceSide + p];
+        uint32_t tb = rec[(size_t)nb * kWords + TS::kFaceHead + TS::kFaceSide + p];
         if (!DEDUP) {
-            ok &= merge(fd.W, f, S, f[S], ta, tb);
+            float fS = f[S];
+            if (!merge_steps<false, kShortBatch>(fd.W, f, S, fS, ta, tb)) ok &= merge_long(fd.W, f, S, fS, ta, tb);
             continue;
         }
         const unsigned long long key = (unsigned long long)ta << 32 | tb,
@@ -702,12 +718,34 @@ __global__ void __launch_bounds__(128, std::is_same<Loc, OneField>::value ? 12 :
             h = (h + 1) & (HS - 1);
         }
     }
-    if (DEDUP) __syncthreads();
-    for (uint32_t j = threadIdx.x; DEDUP && j < s_n; j += NT) {
-        const uint32_t h = list[j], kS = (uint32_t)(hlev[h] >> 32);
-        // the value with order key kS
-        const float fS = __uint_as_float((kS & 0x80000000u) ? kS ^ 0x80000000u : ~kS);
-        ok &= merge(fd.W, f, (uint32_t)hlev[h], fS, (uint32_t)(hkey[h] >> 32), (uint32_t)hkey[h]);
+    if constexpr (DEDUP) {
+        __syncthreads();
+        // the merge in slot h: tops, level
+        auto slot = [&](uint32_t h, uint32_t &S, float &fS, uint32_t &u, uint32_t &v) {
+            const uint32_t kS = (uint32_t)(hlev[h] >> 32);
+            fS = __uint_as_float((kS & 0x80000000u) ? kS ^ 0x80000000u : ~kS);  // the value with that order key
+            S = (uint32_t)hlev[h], u = (uint32_t)(hkey[h] >> 32), v = (uint32_t)hkey[h];
+        };
+        // merges that are not done soon go on in the long form after the others
+        // (in a loop of its own, so that its registers stay out of this one)
+        uint32_t todo = 0;  // a bit for each of the thread's turns
+        static_assert(HS / NT <= 32, "a bit per turn");
+        for (uint32_t j = threadIdx.x, k = 0; j < s_n; j += NT, k++) {
+            const uint32_t h = list[j];
+            uint32_t S, u, v;
+            float fS;
+            slot(h, S, fS, u, v);
+            if (!merge_steps<false, kShortField>(fd.W, f, S, fS, u, v)) {
+                hkey[h] = (unsigned long long)u << 32 | v, hlev[h] = (unsigned long long)order_key(fS) << 32 | S;
+                todo |= 1u << k;
+            }
+        }
+        for (; todo; todo &= todo - 1) {
+            uint32_t S, u, v;
+            float fS;
+            slot(list[threadIdx.x + NT * (__ffs(todo) - 1)], S, fS, u, v);
+            ok &= merge_steps<true>(fd.W, f, S, fS, u, v);
+        }
     }
     if (!ok) raise_status(status, ST_TIMEOUT);
 }
@@ -1372,7 +1410,8 @@ static cudaError_t run_build(const Loc &loc, uint32_t ntiles, uint32_t *queue, i
     }
     {
         PhaseScope ps(kMerge, st);
-        k_cross<VV::LX, VV::LY, VV::LZ, Loc><<<ntiles, 128, 0, st>>>(loc, status);
+        const uint32_t stride = std::is_same<Loc, OneField>::value ? scatter_stride(ntiles) : 1u;
+        k_cross<VV::LX, VV::LY, VV::LZ, Loc><<<ntiles, 128, 0, st>>>(loc, stride, status);
         count_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -17,6 +17,25 @@ constexpr uint32_t kNoLocal = 0xFFFFu;  // no vertex of the tile
 // (o + T may wrap where n is within T of 2^32.)
 MT_HD uint32_t tile_side(uint32_t o, uint32_t T, uint32_t n) { return n - o < T ? n - o : T; }
 
+// The order in which CTAs take the n tiles of a field to merge the edges between
+// them: CTA i takes tile i * scatter_stride(n) mod n. Merged at the same time,
+// neighbours are linked each to the next, a chain that later merges and the
+// repair have to climb; a stride coprime to n, near n over the golden ratio,
+// keeps the tiles that are merged together apart, which leaves chains as short
+// as a random order would.
+inline uint32_t scatter_stride(uint32_t n)
+{
+    if (n < 64) return 1;
+    for (uint32_t k = (uint32_t)(0.6180339887 * n);; k++) {
+        uint32_t a = n, b = k;
+        while (b) {
+            const uint32_t t = a % b;
+            a = b, b = t;
+        }
+        if (a == 1) return k;
+    }
+}
+
 // Local id, in a tile of (1 << LX, 1 << LY, 1 << LZ) vertices of which the
 // first (wx, wy, wz) lie in the grid, of the vertex whose id is `rel` above
 // that of the tile's first vertex (an Id that has wrapped for an earlier one);

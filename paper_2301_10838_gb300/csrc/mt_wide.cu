@@ -35,6 +35,7 @@
 
 #include "../../include/mt.h"
 #include "mt_device.cuh"
+#include "mt_index.h"
 #include "mt_internal.h"
 
 namespace mt {
@@ -138,7 +139,11 @@ __device__ __forceinline__ bool wload(const uint64_t *W, uint64_t u, uint64_t &l
 // read with the step before it. A word read ahead may be torn; it is read
 // again, until its halves carry one tag, when the climb moves to it. Returns
 // false if a read stayed torn or the step budget ran out.
-// 512^3 lognormal: k_w_cross 0.97 ms, 1.31 ms with one climb after the other.
+// 512^3 lognormal: k_w_cross 0.99 ms, 1.31 ms with one climb after the other.
+// A merge that is not done soon goes on in the long form, which shortens the
+// chains it climbs (merge_steps in mt_device.cuh); the call costs the short form
+// 0.03 ms there, and a 65536 x 3 x 3 field of 16 values takes 0.22 ms instead of
+// 2.6.
 struct WideMerge {
     uint64_t *W;
     FieldW f;
@@ -153,14 +158,37 @@ struct WideMerge {
         return (a.lo >> kIdBits) == (a.hi >> kIdBits) || wload(W, a.x, a.lo, a.hi);
     }
 
-    __device__ bool merge(uint64_t S, float fS, uint64_t a, uint64_t b) const
+    // where a climb has come from, in the LONG form of a merge: the vertex, its
+    // word (lo is the saddle) and its saddle's value
+    struct Trail {
+        uint64_t x, lo, hi;
+        float fs;
+    };
+    static constexpr uint64_t NONE = ~0ull;
+
+    // x -> y at the trail's saddle, y = a.x -> z at the saddle sa: if sa comes
+    // first x is linked to z (see merge_steps in mt_device.cuh)
+    __device__ __forceinline__ void shorten(Trail &p, const Node &a, uint64_t sa, float fsa, uint64_t z) const
+    {
+        if (p.x != NONE && before_w(fsa, sa, p.fs, p.lo & kIdMask)) {
+            const uint64_t tag = (uint64_t)(((p.lo >> kIdBits) + 1) & kTagMask) << kIdBits;
+            uint64_t olo, ohi;
+            cas128(W + 2 * p.x, p.lo, p.hi, (p.lo & kIdMask) | tag, z | tag, olo, ohi);
+        }
+        p = Trail{a.x, a.lo, a.hi, fsa};
+    }
+
+    // 1: done, 0: out of steps, -1: a read stayed torn
+    template <bool LONG, uint32_t LIMIT = kMergeStepLimit>
+    __device__ __forceinline__ int run(uint64_t &S, float &fS, uint64_t &a, uint64_t &b) const
     {
         Node u{a, 0, 0, f[a]}, v{b, 0, 0, f[b]};
+        Trail pu{NONE, 0, 0, 0.0f}, pv = pu;
         ld_word(W, a, u.lo, u.hi);
         ld_word(W, b, v.lo, v.hi);
-        for (uint32_t steps = 0; steps < kMergeStepLimit; steps++) {
-            if (u.x == v.x) return true;
-            if (!settle(u) || !settle(v)) return false;
+        for (uint32_t steps = 0; steps < LIMIT; steps++) {
+            if (u.x == v.x) return 1;
+            if (!settle(u) || !settle(v)) return -1;
             const uint64_t su = u.lo & kIdMask, sv = v.lo & kIdMask;
             Node nu{u.hi & kIdMask, 0, 0, 0.0f}, nv{v.hi & kIdMask, 0, 0, 0.0f};  // behind the links
             const bool ru = su == u.x && nu.x == u.x, rv = sv == v.x && nv.x == v.x;
@@ -170,6 +198,8 @@ struct WideMerge {
             ld_word(W, nv.x, nv.lo, nv.hi);
             const bool mu = !ru && (su == S || before_w(fsu, su, fS, S)),
                        mv = !rv && (sv == S || before_w(fsv, sv, fS, S));
+            if (LONG && mu) shorten(pu, u, su, fsu, nu.x);
+            if (LONG && mv) shorten(pv, v, sv, fsv, nv.x);
             if (mu) u = nu;
             if (mv) v = nv;
             if (mu || mv) continue;
@@ -179,18 +209,30 @@ struct WideMerge {
             uint64_t olo, ohi;
             cas128(W + 2 * hi.x, hi.lo, hi.hi, S | tag, (sw ? v.x : u.x) | tag, olo, ohi);
             if (olo == hi.lo && ohi == hi.hi) {
-                if (sw ? ru : rv) return true;  // displaced a root: it carries no link
+                if (sw ? ru : rv) return 1;  // displaced a root: it carries no link
                 S = sw ? su : sv, fS = sw ? fsu : fsv;  // re-insert the displaced link
-                if (sw) u = nu;
-                else v = nv;
+                if (sw) u = nu, pu.x = NONE;
+                else v = nv, pv.x = NONE;
             } else if (sw) {
                 u.lo = olo, u.hi = ohi;
             } else {
                 v.lo = olo, v.hi = ohi;
             }
         }
-        return false;
+        a = u.x, b = v.x;
+        return 0;
     }
+
+    __device__ bool merge(uint64_t S, float fS, uint64_t a, uint64_t b) const
+    {
+        const int r = run<false, kShort>(S, fS, a, b);
+        return r ? r > 0 : merge_long(S, fS, a, b);
+    }
+    __device__ __noinline__ bool merge_long(uint64_t S, float fS, uint64_t a, uint64_t b) const
+    {
+        return run<true>(S, fS, a, b) > 0;
+    }
+    static constexpr uint32_t kShort = 32;  // steps before the long form (16: no faster, 96: 65536 x 3 x 3 slower)
 };
 
 // One CTA per 16x16x16 tile: the edges from the tile to its +x, +y and +z
@@ -201,8 +243,8 @@ struct WideMerge {
 // of the edge's ends), so only the local minima of the level over each face
 // are merged: about 132 of the 768 edges on a lognormal field. They are
 // listed first, so that all lanes have one to merge.
-__global__ void __launch_bounds__(256) k_w_cross(FieldW f, Geo g, uint32_t ntx, uint32_t nty, uint64_t *W,
-                                                 uint32_t *status)
+__global__ void __launch_bounds__(256, 4) k_w_cross(FieldW f, Geo g, uint32_t ntx, uint32_t nty, uint64_t *W,
+                                                 uint32_t stride, uint32_t *status)
 {
     if (block_skips(status)) return;
     constexpr uint32_t F = kSide * kSide;
@@ -211,7 +253,7 @@ __global__ void __launch_bounds__(256) k_w_cross(FieldW f, Geo g, uint32_t ntx, 
     __shared__ uint16_t list[3 * F];
     __shared__ uint32_t s_n;
     const WideMerge M{W, f};
-    const uint32_t tile = blockIdx.x;
+    const uint32_t tile = stride == 1 ? blockIdx.x : (uint32_t)((uint64_t)blockIdx.x * stride % gridDim.x);
     const uint32_t tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
     const uint64_t x0 = (uint64_t)tx * kSide, y0 = (uint64_t)ty * kSide, z0 = (uint64_t)tz * kSide;
     const uint32_t wx = (uint32_t)min((uint64_t)kSide, g.nx - x0), wy = (uint32_t)min((uint64_t)kSide, g.ny - y0),
@@ -448,7 +490,13 @@ mt_status mt_build_triplets_wide(const float *d_f, mt_grid g, uint64_t *d_W, voi
                    ntz = (uint32_t)((geo.nz + kSide - 1) / kSide);
     {
         PhaseScope ps(kMerge, s);
-        k_w_cross<<<ntx * nty * ntz, 256, 0, s>>>(f, geo, ntx, nty, d_W, ws.status);
+        // Grids a few tiles thick are merged in scattered order (scatter_stride):
+        // a line of 2^18 constant vertices 0.10 ms instead of 0.20. With 16-byte
+        // words others lose more to L2 than shorter chains give back: 512^3
+        // lognormal 1.00 ms, in order 0.96.
+        const uint32_t tiles = ntx * nty * ntz, most = ntx > nty ? (ntx > ntz ? ntx : ntz) : (nty > ntz ? nty : ntz);
+        const uint32_t stride = tiles / most < 32 ? scatter_stride(tiles) : 1u;
+        k_w_cross<<<tiles, 256, 0, s>>>(f, geo, ntx, nty, d_W, stride, ws.status);
         count_launch();
     }
     {

@@ -1,4 +1,4 @@
-"""The repair pass's local ids and tile sides against exact arithmetic, on the CPU.
+"""Local ids, tile sides and the order of the tiles against exact arithmetic, on the CPU.
 
 csrc/mt_index.h finds a vertex's place in its tile by reciprocals; here it is
 compiled for the host and compared with 64-bit division, with 32-bit and 64-bit
@@ -78,6 +78,13 @@ int main()
             if (tile_side((uint32_t)o, 16, (uint32_t)n) != want && bad++ < 5)
                 printf("axis of %llu: not %llu vertices in the tile at %llu\n", n, want, o);
         }
+    // the scattered order of the tiles takes each tile once
+    for (u64 i = 0; i < 20000; i++) {
+        const u64 n = i < 10000 ? i + 1 : rnd() % 0x7FFFFFFFull + 1, k = scatter_stride((uint32_t)n);
+        u64 a = n, b = k;
+        while (b) { const u64 t = a % b; a = b, b = t; }
+        if ((a != 1 || k == 0) && bad++ < 5) printf("%llu tiles: a stride of %llu\n", n, k);
+    }
     const u64 side[] = {1, 2, 3, 15, 16, 17, 33, 509, 1024, 65535, 65536, (1u << 28) - 1, (1u << 28) + 1,
                         (1u << 29) + 16, 1431655764, 2147483648u, 3000000019u, 4294967295u};
     for (u64 a : side)
