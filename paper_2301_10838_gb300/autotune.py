@@ -6,9 +6,10 @@ file (``MT_AUTOTUNE_CACHE``, default ``~/.cache/mt_gb300_autotune.json``)
 keyed by the GPU name and a shape class, so that later runs on the same kind
 of input skip the timing. Every configuration gives the same results.
 
-Configurations are the MT_CFG_* bits of include/mt.h: tile shape (batches:
-16x16x8 or 16x16x16; single fields: 16x16x16 or 32x16x16), level buckets per
-tile (the merge/repair rounds) and the repair CTA size.
+Configurations are the MT_CFG_* bits of include/mt.h, of which the tile shape
+chooses among kernels (batches: 16x16x8 or 16x16x16; single fields: 16x16x16 or
+32x16x16); the other bits are accepted and choose nothing. An entry is used only
+by the kernels it was timed with (KERNELS).
 """
 
 from __future__ import annotations
@@ -23,6 +24,10 @@ import torch
 from . import binding as B
 
 _LOCK = threading.Lock()
+
+# Revision of the kernels that the configurations choose among, kept with every
+# entry: raised when a change to them may change which one is fastest.
+KERNELS = 2
 
 
 def cache_path() -> str:
@@ -50,14 +55,18 @@ def _key(device, cls: str) -> str:
 
 
 def lookup(device, cls: str):
-    """The cached entry {"cfg": .., "ms": ..} or None."""
+    """The cached entry {"cfg": .., "ms": ..} or None (no entry, or one timed
+    with other kernels)."""
     with _LOCK:
         try:
             with open(cache_path()) as fh:
                 cache = json.load(fh)
         except (OSError, ValueError):
             return None
-    return cache.get(_key(device, cls))
+    hit = cache.get(_key(device, cls))
+    if hit is None or hit.get("kernels") != KERNELS:
+        return None
+    return {"cfg": hit["cfg"], "ms": hit["ms"]}
 
 
 def store(device, cls: str, cfg: int, ms) -> None:
@@ -68,7 +77,7 @@ def store(device, cls: str, cfg: int, ms) -> None:
                 cache = json.load(fh)
         except (OSError, ValueError):
             cache = {}
-        cache[_key(device, cls)] = {"cfg": int(cfg), "ms": ms}
+        cache[_key(device, cls)] = {"cfg": int(cfg), "ms": ms, "kernels": KERNELS}
         os.makedirs(os.path.dirname(path) or ".", exist_ok=True)
         tmp = path + f".{os.getpid()}"
         with open(tmp, "w") as fh:
