@@ -107,11 +107,12 @@ mt_status mt_build_triplets_ex(const float *d_f, mt_grid g, uint64_t *d_W, void 
 mt_status mt_build_triplets_cfg(const float *d_f, mt_grid g, uint64_t *d_W, void *d_ws, size_t ws_bytes, uint32_t flags,
                                 uint32_t cfg, void *stream);
 
-/* Autotuner for single fields: builds the tree of d_f once per
- * configuration (cfg 0, 2, 4, 6, 8, 10, 12, 14: the single-field knobs) to
- * warm up and three times timed (CUDA events on `stream`), writes the best
- * times to ms[0..7] (in that order; ms holds 8 floats) and the fastest
- * configuration to *best. d_W receives the triplets. Synchronises. */
+/* Autotuner for single fields: builds the tree of d_f once per tile shape
+ * (cfg 0 and MT_CFG_LARGE_TILES) to warm up and three times timed (CUDA events
+ * on `stream`), writes the best times to ms[0..7] (of cfg 0, 2, 4, 6, 8, 10,
+ * 12, 14, the single-field knobs, in that order: each gets its tile shape's
+ * time; ms holds 8 floats) and the fastest configuration to *best. d_W receives
+ * the triplets. Synchronises. */
 mt_status mt_build_autotune(const float *d_f, mt_grid g, uint64_t *d_W, void *d_ws, size_t ws_bytes, uint32_t flags,
                             void *stream, float *ms, uint32_t *best);
 
@@ -295,9 +296,9 @@ mt_status mt_batch_launch(const mt_batch_plan *plan, int cfg, uint64_t *d_npairs
 mt_status mt_batch_build(const float *d_arena, const mt_grid *h_grids, uint32_t nfields, uint64_t *d_W_arena,
                          uint32_t *d_pairs_arena, uint64_t *d_npairs, void *d_ws, size_t ws_bytes, void *stream);
 
-/* Autotuner: runs every launch configuration (cfg 0 to MT_CFG_COUNT - 1) of
- * the batch once to warm up and three times timed (CUDA events on
- * `stream`), writes the best time of each to ms[0..MT_CFG_COUNT-1] and the
+/* Autotuner: runs the batch once per tile shape (cfg 0 and MT_CFG_SMALL_TILES) to
+ * warm up and three times timed (CUDA events on `stream`), writes the best time
+ * to ms[0..MT_CFG_COUNT-1] (each configuration gets its tile shape's) and the
  * fastest configuration to *best. Synchronises. */
 mt_status mt_batch_autotune(const mt_batch_plan *plan, uint64_t *d_npairs, void *d_ws, size_t ws_bytes, void *stream,
                             float *ms, int *best);

@@ -1,9 +1,8 @@
 """Batched merge trees over many uneven fields (host-side orchestration).
 
 ``Batch`` packs fields into device arenas, prepares the field table in libmt,
-picks the launch configuration (tile shape, level buckets, repair CTA size)
-with libmt's autotuner (cached per GPU and batch shape class, ``autotune``),
-and optionally captures the batched launch in a CUDA graph so that a
+picks the launch configuration (the tile shape) with libmt's autotuner (cached
+per GPU and batch shape class, ``autotune``), and optionally captures the batched launch in a CUDA graph so that a
 repeated batch costs one graph launch. All merge-tree work runs in libmt's
 kernels.
 """
@@ -56,8 +55,8 @@ class Batch:
 
     def tune(self, use_cache: bool = True) -> int:
         """Pick the launch configuration: cached for this GPU and shape class,
-        else libmt's autotuner over all MT_CFG_COUNT configurations (which
-        needs the fields loaded). Returns it."""
+        else libmt's autotuner over both tile shapes (which needs the fields
+        loaded). Returns it."""
         cls = autotune.batch_class(self.shapes)
         if use_cache:
             hit = autotune.lookup(self.device, cls)

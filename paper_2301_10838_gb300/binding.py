@@ -284,9 +284,9 @@ def mt_build_triplets_ex(f: torch.Tensor, W: torch.Tensor, ws: torch.Tensor, fla
 
 def mt_build_triplets_cfg(f: torch.Tensor, W: torch.Tensor, ws: torch.Tensor, flags: int, cfg: int,
                           stream=None) -> None:
-    """mt_build_triplets_ex with a launch configuration (MT_CFG_FOUR_ROUNDS,
-    MT_CFG_REPAIR_256, MT_CFG_LARGE_TILES bits); the triplets do not depend
-    on it."""
+    """mt_build_triplets_ex with a launch configuration (MT_CFG_LARGE_TILES
+    chooses 32x16x16 tiles; MT_CFG_FOUR_ROUNDS and MT_CFG_REPAIR_256 are accepted
+    and choose nothing); the triplets do not depend on it."""
     g = grid_of(f)
     n = f.numel()
     _check(load().mt_build_triplets_cfg(_dev(f, "f", (torch.float32,)), g, _dev(W, "W", _I64, n),
@@ -295,8 +295,8 @@ def mt_build_triplets_cfg(f: torch.Tensor, W: torch.Tensor, ws: torch.Tensor, fl
 
 
 def mt_build_autotune(f: torch.Tensor, W: torch.Tensor, ws: torch.Tensor, flags: int = 0, stream=None):
-    """Times the single-field configurations (cfg 0, 2, .., 14); returns
-    ({cfg: best ms}, best cfg). W receives the triplets."""
+    """Times the tile shapes of the single-field configurations (cfg 0, 2, ..,
+    14); returns ({cfg: best ms}, best cfg). W receives the triplets."""
     g = grid_of(f)
     n = f.numel()
     ms = (ctypes.c_float * 8)()
@@ -569,8 +569,7 @@ def mt_batch_build(arena: torch.Tensor, grids, W_arena: torch.Tensor, pairs_aren
 
 
 def mt_batch_autotune(plan: BatchPlan, npairs: torch.Tensor, ws: torch.Tensor, stream=None):
-    """Times every launch configuration of the batch; returns ([ms per cfg],
-    best cfg)."""
+    """Times both tile shapes on the batch; returns ([ms per cfg], best cfg)."""
     ms = (ctypes.c_float * MT_CFG_COUNT)()
     best = ctypes.c_int(0)
     _check(load().mt_batch_autotune(ctypes.byref(plan), _dev(npairs, "npairs", _I64, plan.nfields),

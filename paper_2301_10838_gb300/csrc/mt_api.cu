@@ -270,7 +270,11 @@ mt_status mt_build_autotune(const float *d_f, mt_grid g, uint64_t *d_W, void *d_
     constexpr int kCfgs = 8;  // the even configurations 0 .. 14
     mt_status st = MT_OK;
     for (int i = 0; i < kCfgs && st == MT_OK; i++) {
-        const uint32_t cfg = 2u * (uint32_t)i;
+        const uint32_t cfg = 2u * (uint32_t)i, same = cfg & MT_CFG_LARGE_TILES;  // the other knobs choose nothing
+        if (same != cfg) {
+            ms[i] = ms[same / 2];
+            continue;
+        }
         st = mt_build_triplets_cfg(d_f, g, d_W, d_ws, ws_bytes, flags, cfg, stream);  // warm-up
         float best_ms = 1e30f;
         for (int rep = 0; rep < 3 && st == MT_OK; rep++) {

@@ -185,6 +185,11 @@ mt_status mt_batch_autotune(const mt_batch_plan *plan, uint64_t *d_npairs, void 
     }
     mt_status st = MT_OK;
     for (int c = 0; c < MT_CFG_COUNT && st == MT_OK; c++) {
+        const int same = c & (int)MT_CFG_SMALL_TILES;  // the other knobs choose nothing
+        if (same != c) {
+            ms[c] = ms[same];
+            continue;
+        }
         st = mt_batch_launch(plan, c, d_npairs, d_ws, ws_bytes, stream);  // warm-up
         if (st != MT_OK) break;
         float best_ms = 1e30f;
