@@ -284,16 +284,20 @@ static cudaError_t run_pairs(const Loc &loc, uint32_t nfields, uint64_t nchunks,
                              uint64_t *out = nullptr, uint64_t marked = 0)
 {
     PhaseScope ps(kPairs, st);
-    const bool simp = eps > 0.0f;
     const unsigned grid = (unsigned)nchunks;
-    if (marked)  // the number of vertices
-        k_mask_count<<<(unsigned)((nchunks + kCompactWarps - 1) / kCompactWarps), kCompactThreads, 0, st>>>(
-            mask, marked, nchunks, counts, status);
-    else if (simp) k_pairs_count<Loc, true><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
-    else k_pairs_count<Loc, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
+    constexpr bool ONE = std::is_same<Loc, OneField>::value;  // a batch has no eps, bits or mapped counters
+    bool simp = false;
+    if constexpr (ONE) {
+        simp = eps > 0.0f;
+        if (marked)  // the number of vertices
+            k_mask_count<<<(unsigned)((nchunks + kCompactWarps - 1) / kCompactWarps), kCompactThreads, 0, st>>>(
+                mask, marked, nchunks, counts, status);
+        else if (simp) k_pairs_count<Loc, true><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
+    }
+    if (!marked && !simp) k_pairs_count<Loc, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if constexpr (std::is_same<Loc, OneField>::value) {
+    if constexpr (ONE) {
         if (mask && nchunks <= kSumChunks) {
             k_pairs_write<Loc, false, true, true><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
             count_launch(2);
@@ -302,9 +306,11 @@ static cudaError_t run_pairs(const Loc &loc, uint32_t nfields, uint64_t nchunks,
     }
     k_scan_counts<Loc><<<nfields, 1024, 0, st>>>(loc, counts, npairs, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (mask) k_pairs_write<Loc, false, true, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
-    else if (simp) k_pairs_write<Loc, true, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
-    else k_pairs_write<Loc, false, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
+    if constexpr (ONE) {
+        if (mask) k_pairs_write<Loc, false, true, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
+        else if (simp) k_pairs_write<Loc, true, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
+    }
+    if (!mask && !simp) k_pairs_write<Loc, false, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
     count_launch(3);
     return cudaGetLastError();
 }
