@@ -99,10 +99,9 @@ struct Tile {
     static constexpr int kFaceHead = (G + 15) / 16 * 4, kFaceSide = 16 * G;
     static constexpr int kFaceWords = kFaceHead + 3 * kFaceSide;
     // after the face record, for the repair pass: the minima of every column
-    // (16 bits each), the tile's highest key; the wide path has only these
-    static constexpr int kNoteWords = NT / 2 + 4;
-    template <bool WIDE> static constexpr int kNote = WIDE ? 0 : kFaceWords;
-    template <bool WIDE> static constexpr int kTileWords = kNote<WIDE> + kNoteWords;
+    // (16 bits each), the tile's highest key (the wide path has only these, see
+    // wide_note_words)
+    static constexpr int kNoteWords = NT / 2 + 4, kTileWords = kFaceWords + kNoteWords;
     static_assert(TY * TZ <= NT && TX * TZ <= NT, "one edge of a face per thread");
     static constexpr int FX = TY * TZ, FY = TX * TZ, FZ = TX * TY, FH = FX + FY + FZ;  // edges of the + faces
     static_assert(2 * FH * 8 <= TV * 4, "the faces' levels fit the key array");
@@ -484,9 +483,17 @@ __device__ __forceinline__ void tile_body(const FieldDesc &fd, uint32_t tile, ui
     // 7. for k_repair: the words of the inner vertices say which tile minimum
     //    they descend to (they get their triplets once all merges are done);
     //    the tile's minima and highest key
-    uint32_t *rec = fd.faces + (size_t)tile * TS::template kTileWords<WIDE>;
-    reinterpret_cast<uint16_t *>(rec + TS::template kNote<WIDE>)[col] = (uint16_t)minima;
-    if (threadIdx.x == 0) rec[TS::template kNote<WIDE> + NT / 2] = s_kmax - 1;
+    uint32_t *rec = fd.faces;
+    if constexpr (WIDE) {
+        const uint32_t mx = min(nx, TX), words = wide_note_words(nx, ny);
+        rec += (size_t)tile * words;
+        if (cx < mx && cy < min(ny, TY)) reinterpret_cast<uint16_t *>(rec)[cx + cy * mx] = (uint16_t)minima;
+        if (threadIdx.x == 0) rec[words - 1] = s_kmax - 1;
+    } else {
+        rec += (size_t)tile * TS::kTileWords;
+        reinterpret_cast<uint16_t *>(rec + TS::kFaceWords)[col] = (uint16_t)minima;
+        if (threadIdx.x == 0) rec[TS::kFaceWords + NT / 2] = s_kmax - 1;
+    }
     if (inx) {
         const Id u0 = gid(col);
 #pragma unroll
@@ -672,7 +679,7 @@ __global__ void __launch_bounds__(128, std::is_same<Loc, OneField>::value ? 12 :
     constexpr bool ONE = std::is_same<Loc, OneField>::value;
     const FieldDesc fd = loc.tile(ONE ? (uint32_t)((uint64_t)blockIdx.x * stride % gridDim.x) : blockIdx.x, tile);
     const Field f{fd.f, fd.sg};
-    constexpr uint32_t kWords = TS::template kTileWords<false>;
+    constexpr uint32_t kWords = TS::kTileWords;
     const uint32_t *rec = fd.faces + (size_t)tile * kWords;
     if (threadIdx.x < 32) {
         static_assert(G <= 64, "two groups per lane");
@@ -989,8 +996,17 @@ __global__ void __launch_bounds__(1 << (LX + LY), RepairShape<LX, LY, LZ, LAB, W
 
     // 1. number the tile's minima (the bits the tile kernel left per column)
     using TS = Tile<LX, LY, LZ>;
-    const uint32_t *note = fd.faces + (size_t)tile * TS::template kTileWords<WIDE> + TS::template kNote<WIDE>;
-    const uint32_t minima = reinterpret_cast<const uint16_t *>(note)[col], kmax = note[NT / 2];
+    const uint32_t *note = fd.faces;
+    uint32_t minima = 0, kmax;
+    if constexpr (WIDE) {
+        const uint32_t mx = min(nx, TX), words = wide_note_words(nx, ny);
+        note += (size_t)tile * words;
+        if (cx < mx && cy < min(ny, TY)) minima = reinterpret_cast<const uint16_t *>(note)[cx + cy * mx];
+        kmax = note[words - 1];
+    } else {
+        note += (size_t)tile * TS::kTileWords + TS::kFaceWords;
+        minima = reinterpret_cast<const uint16_t *>(note)[col], kmax = note[NT / 2];
+    }
     {
         const uint32_t cnt = __popc(minima);
         uint32_t incl = cnt;
@@ -1337,8 +1353,8 @@ void tile_shape(int variant, uint32_t &tx, uint32_t &ty, uint32_t &tz)
 // than its record takes.
 uint32_t face_words(int variant)
 {
-    static_assert(TileOf<0>::kTileWords<false> <= 2 * TileOf<0>::FH && TileOf<1>::kTileWords<false> <= 2 * TileOf<1>::FH &&
-                      TileOf<2>::kTileWords<false> <= 2 * TileOf<2>::FH,
+    static_assert(TileOf<0>::kTileWords <= 2 * TileOf<0>::FH && TileOf<1>::kTileWords <= 2 * TileOf<1>::FH &&
+                      TileOf<2>::kTileWords <= 2 * TileOf<2>::FH,
                   "the tile records fit the workspace");
     return 2 * (variant == 1 ? TileOf<1>::FH : variant == 2 ? TileOf<2>::FH : TileOf<0>::FH);
 }
@@ -1428,7 +1444,7 @@ uint32_t *build_mask(uint32_t *faces, uint32_t nx, uint32_t ny, uint32_t nz, uin
     uint32_t tx, ty, tz;
     tile_shape(v, tx, ty, tz);
     if (nx % tx != 0) return nullptr;
-    constexpr int w0 = TileOf<0>::kTileWords<false>, w2 = TileOf<2>::kTileWords<false>;
+    constexpr int w0 = TileOf<0>::kTileWords, w2 = TileOf<2>::kTileWords;
     static_assert(2 * TileOf<0>::FH - w0 >= TileOf<0>::TV / 32 && 2 * TileOf<2>::FH - w2 >= TileOf<2>::TV / 32,
                   "a bit per vertex fits behind the records");
     static_assert(w0 % 4 == 0 && w2 % 4 == 0, "16-byte aligned");
@@ -1464,8 +1480,8 @@ cudaError_t launch_build(const float *f, uint64_t *W, uint32_t nx, uint32_t ny, 
 }
 
 // The tile kernel and the repair pass with 64-bit ids and 128-bit words (the
-// wide path), on 16x16x16 tiles; notes: wide_note_words() u32 per tile.
-uint32_t wide_note_words() { return TileOf<0>::kTileWords<true>; }
+// wide path), on 16x16x16 tiles.
+static_assert(TileOf<0>::TX == 16 && TileOf<0>::TY == 16 && TileOf<0>::TZ == 16, "as wide_note_words has it");
 
 static bool wide_field(const float *f, uint64_t *W2, uint32_t *notes, uint32_t nx, uint32_t ny, uint32_t nz, float sg,
                        OneField &loc, uint64_t &ntiles)

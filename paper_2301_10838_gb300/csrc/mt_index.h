@@ -17,6 +17,12 @@ constexpr uint32_t kNoLocal = 0xFFFFu;  // no vertex of the tile
 // (o + T may wrap where n is within T of 2^32.)
 MT_HD uint32_t tile_side(uint32_t o, uint32_t T, uint32_t n) { return n - o < T ? n - o : T; }
 
+// Notes that the wide path's tile kernel leaves per 16x16x16 tile for the repair
+// pass, in u32 words: the minima of every column (16 bits each), then the tile's
+// highest key. A grid less than 16 wide has the columns of its own sides only, so
+// that the notes of a line take 3 bytes per vertex (0.13 in a solid grid).
+MT_HD uint32_t wide_note_words(uint32_t nx, uint32_t ny) { return ((nx < 16 ? nx : 16) * (ny < 16 ? ny : 16) + 1) / 2 + 1; }
+
 // The order in which CTAs take the n tiles of a field to merge the edges between
 // them: CTA i takes tile i * scatter_stride(n) mod n. Merged at the same time,
 // neighbours are linked each to the next, a chain that later merges and the

@@ -124,15 +124,15 @@ cudaError_t launch_pairs(const uint64_t *W, uint64_t n, uint32_t *pairs, uint64_
                          cudaStream_t st, const float *f = nullptr, float sg = 1.0f, float eps = 0.0f,
                          uint64_t *out = nullptr, bool clear = true, bool marked = false);
 
-// Batched build and pairs over a packed descriptor table already in device
-// memory; cfg holds the MT_CFG_* knobs (mt_build.cu, mt_query.cu).
 // The tile kernel and the repair pass for the wide-id path, on 16x16x16 tiles
-// and 128-bit words of two 64-bit ids (mt_build.cu).
-uint32_t wide_note_words();  // u32 per tile that the two share (notes)
+// and 128-bit words of two 64-bit ids (mt_build.cu); notes: wide_note_words (mt_index.h)
+// u32 per tile, which the two share.
 cudaError_t launch_tile_wide(const float *f, uint64_t *W2, uint32_t *notes, uint32_t nx, uint32_t ny, uint32_t nz,
                              float sg, uint32_t *status, cudaStream_t st);
 cudaError_t launch_repair_wide(const float *f, uint64_t *W2, uint32_t *notes, uint32_t nx, uint32_t ny, uint32_t nz,
                                float sg, uint32_t *status, cudaStream_t st);
+// Batched build and pairs over a packed descriptor table already in device
+// memory; cfg holds the MT_CFG_* knobs (mt_build.cu, mt_query.cu).
 cudaError_t launch_batch_build(const FieldDesc *d_descs, uint32_t nfields, uint32_t ntiles, uint32_t cfg,
                                uint32_t *status, uint32_t *queue, cudaStream_t st);
 cudaError_t launch_batch_pairs(const FieldDesc *d_descs, uint32_t nfields, uint64_t nchunks, uint32_t *counts,

@@ -50,7 +50,7 @@ constexpr int kWThreads = 256;
 
 // Workspace: [0, 256) status word, [256, 512) meta (npairs, roots, root),
 // then per-chunk pair counts (u32) and offsets (u64), then the notes that the
-// tile kernel leaves for the repair pass.
+// tile kernel leaves for the repair pass, or the pair compaction's bits.
 struct WideWs {
     uint32_t *status;
     uint64_t *meta;
@@ -72,7 +72,8 @@ size_t wide_ws_bytes(const Geo &g)
 {
     const uint64_t nchunks = (g.n + kWChunk - 1) / kWChunk, t = kSide;
     const uint64_t tiles = ((g.nx + t - 1) / t) * ((g.ny + t - 1) / t) * ((g.nz + t - 1) / t);
-    return 512 + al256(nchunks * 4) + al256(nchunks * 8) + al256(tiles * wide_note_words() * 4);
+    const size_t notes = tiles * wide_note_words((uint32_t)g.nx, (uint32_t)g.ny) * 4, bits = nchunks * (kWChunk / 8);
+    return 512 + al256(nchunks * 4) + al256(nchunks * 8) + al256(notes > bits ? notes : bits);
 }
 
 bool carve(void *base, size_t bytes, const Geo &g, WideWs &ws)
