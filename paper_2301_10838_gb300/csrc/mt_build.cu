@@ -640,10 +640,10 @@ __global__ void __launch_bounds__(Tile<LX, LY, LZ>::NT, Tile<LX, LY, LZ>::kCTAs)
 // 93 of the 132 edges per tile on a lognormal field.
 //
 // The kernel is bound by the latency of its chains of dependent reads (a
-// quarter of the issue slots used, HBM 12 % busy): 4.3 ms on the 1024^3
-// lognormal field, 4.6 with the tiles in order instead of scattered (256^3
-// white noise 143 and 155 us, of 16 values 165 and 240, a line of 2^18 constant
-// vertices 55 and 390); 6.3 ms with a merge that read a vertex's value and a
+// quarter of the issue slots used, HBM 12 % busy): 4.7 ms on the 1024^3
+// lognormal field, 4.8 with the tiles in order instead of scattered (512^3 0.55
+// and 0.63, 256^3 white noise 143 and 155 us, a line of 2^18 constant vertices
+// 55 and 390); 6.3 ms with a merge that read a vertex's value and a
 // re-inserted link's level only when it needed them, in order and without the
 // hash; 5.6 ms with the new merge alone. The fields of a batch are small enough
 // for L2, where the hash costs more than the merges it saves (512 uneven
@@ -785,10 +785,10 @@ __global__ void __launch_bounds__(128, std::is_same<Loc, OneField>::value ? 12 :
 // Tables that are full (more than kMin minima, a crowded hash) leave a link
 // without a node; whoever needs it goes on along the global chain.
 //
-// What it costs, on the 1024^3 lognormal field: 8.4 ms, 10.9 ms with labels
+// What it costs, on the 1024^3 lognormal field: 8.5 ms, 10.8 ms with labels
 // (11.7 and 14.2 ms with copies of each target's first 8 links found through
 // a hash per vertex, from triplets that the tile kernel had repaired itself
-// at 3.8 ms more), 11.4 ms with labels and the pairs marked, which saves 1.2 ms
+// at 3.8 ms more), 11.1 ms with labels and the pairs marked, which saves 1.2 ms
 // of the pair compaction. With 6 CTAs per SM: numbering 1.0, links 3.2 (chains
 // of dependent reads), targets and labels 0.7 to 1.2, inner vertices 4.9 to
 // 5.4 (16 to 24 bytes each way per vertex, 130 thread instructions). Issue
@@ -868,9 +868,9 @@ struct RepairShape {
                                     (LAB ? (size_t)kMin * 2 + TV / 8 : 0);
     static_assert((kMin + kHash) % 2 == 0, "the bits after the 16-bit arrays are 4-byte aligned");
     static constexpr int kFit = (int)(227 * 1024 / (kSmem + 1024));
-    // CTAs per SM the registers are limited for: 7 of 256 threads (36
-    // registers) take 8.4 ms without labels on the 1024^3 field, 6 take 9.7;
-    // with labels 6 (40 registers) take 10.8 ms and 7 take 11.0
+    // CTAs per SM the registers are limited for: 7 of 256 threads (32
+    // registers, 20 bytes spilt) take 8.5 ms without labels on the 1024^3 field,
+    // 6 take 9.7; with labels 6 (40 registers) take 10.8 ms and 7 take 11.0
     static constexpr int kWant = (LAB || WIDE ? 1536 : 1792) / NT, kCTAs = kFit < kWant ? kFit : kWant;
 };
 
@@ -1426,7 +1426,9 @@ static cudaError_t run_build(const Loc &loc, uint32_t ntiles, uint32_t *queue, i
     }
     {
         PhaseScope ps(kMerge, st);
-        const uint32_t stride = std::is_same<Loc, OneField>::value ? scatter_stride(ntiles) : 1u;
+        uint32_t stride = 1;  // the scattered order costs the large tiles more in L2 than it saves (1024^3: 5.0 -> 6.8 ms)
+        if constexpr (std::is_same<Loc, OneField>::value)
+            if (V == 0 || thin_tiles(loc.d.ntx, loc.d.nty, ntiles / (loc.d.ntx * loc.d.nty))) stride = scatter_stride(ntiles);
         k_cross<VV::LX, VV::LY, VV::LZ, Loc><<<ntiles, 128, 0, st>>>(loc, stride, status);
         count_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -42,6 +42,15 @@ inline uint32_t scatter_stride(uint32_t n)
     }
 }
 
+// Whether a grid of tiles is only a few tiles thick: then neighbours in the order
+// of their numbers make up whole chains, and nothing is gained from their
+// sharing lines in L2.
+inline bool thin_tiles(uint32_t ntx, uint32_t nty, uint32_t ntz)
+{
+    const uint32_t m = ntx > nty ? ntx : nty, most = m > ntz ? m : ntz;
+    return (uint64_t)ntx * nty * ntz / most < 32;
+}
+
 // Local id, in a tile of (1 << LX, 1 << LY, 1 << LZ) vertices of which the
 // first (wx, wy, wz) lie in the grid, of the vertex whose id is `rel` above
 // that of the tile's first vertex (an Id that has wrapped for an earlier one);

@@ -491,12 +491,10 @@ mt_status mt_build_triplets_wide(const float *d_f, mt_grid g, uint64_t *d_W, voi
                    ntz = (uint32_t)((geo.nz + kSide - 1) / kSide);
     {
         PhaseScope ps(kMerge, s);
-        // Grids a few tiles thick are merged in scattered order (scatter_stride):
-        // a line of 2^18 constant vertices 0.10 ms instead of 0.20. With 16-byte
-        // words others lose more to L2 than shorter chains give back: 512^3
-        // lognormal 1.00 ms, in order 0.96.
-        const uint32_t tiles = ntx * nty * ntz, most = ntx > nty ? (ntx > ntz ? ntx : ntz) : (nty > ntz ? nty : ntz);
-        const uint32_t stride = tiles / most < 32 ? scatter_stride(tiles) : 1u;
+        // Thin grids are merged in scattered order: a line of 2^18 constant
+        // vertices 0.10 ms instead of 0.20. With 16-byte words others lose more to
+        // L2 than shorter chains give back: 512^3 lognormal 1.00 ms, in order 0.96.
+        const uint32_t tiles = ntx * nty * ntz, stride = thin_tiles(ntx, nty, ntz) ? scatter_stride(tiles) : 1u;
         k_w_cross<<<tiles, 256, 0, s>>>(f, geo, ntx, nty, d_W, stride, ws.status);
         count_launch();
     }
