@@ -14,7 +14,7 @@ namespace mt {
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Workspace layout (all offsets 256-byte aligned):
-//   [0, 256)     status word, round flag
+//   [0, 256)     status word
 //   [256, 512)   meta: npairs, number of roots, root
 //   [512, ...)   per-chunk counts of the ordered compaction
 //   then, for a build, face_words(v) u32 per tile of the tile shape v in use

@@ -19,14 +19,14 @@ enum : uint32_t {
 };
 
 // Table sizes of the shared-memory hashes and lists. Each table has a path
-// for when it is full (merge in place, repair from an overflow bitmap, chase
-// the global chain); the defaults keep those paths rare. A library built with
-// MT_STRESS_TABLES shrinks the tables so that the tests reach every such
-// path; its results are the same.
+// for when it is full (merge an edge in place, climb the global chain); the
+// defaults keep those paths rare. A library built with MT_STRESS_TABLES shrinks
+// the tables so that the tests reach every such path, and takes wide labels
+// through bricks for small fields, too; its results are the same.
 #ifdef MT_STRESS_TABLES
-constexpr int kTileListShrink = 64;       // k_tile: edge list 64x smaller
-constexpr uint32_t kRepairShrink = 64;    // k_repair: hash, copies and minima list 64x smaller
-constexpr uint32_t kLabelShrink = 64;     // k_labels: hash of chain starts 64x smaller
+constexpr int kTileListShrink = 64;       // k_tile: edge list
+constexpr uint32_t kRepairShrink = 64;    // k_repair: nodes of the tile's minima and of foreign ones
+constexpr uint32_t kLabelShrink = 64;     // k_labels: hash of chain starts
 #else
 constexpr int kTileListShrink = 1;
 constexpr uint32_t kRepairShrink = 1;
