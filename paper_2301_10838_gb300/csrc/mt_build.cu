@@ -639,8 +639,8 @@ __global__ void __launch_bounds__(Tile<LX, LY, LZ>::NT, Tile<LX, LY, LZ>::kCTAs)
 // of each pair is merged (a shared-memory hash with 64-bit atomicMin): about
 // 93 of the 132 edges per tile on a lognormal field.
 //
-// The kernel is bound by the latency of its chains of dependent reads (a
-// quarter of the issue slots used, HBM 12 % busy): 4.7 ms on the 1024^3
+// The kernel is bound by the latency of its chains of dependent reads (38 % of
+// the issue slots used, HBM 39 % busy at 512^3): 4.7 ms on the 1024^3
 // lognormal field, 4.8 with the tiles in order instead of scattered (512^3 0.55
 // and 0.63, 256^3 white noise 143 and 155 us, a line of 2^18 constant vertices
 // 55 and 390); 6.3 ms with a merge that read a vertex's value and a
