@@ -14,6 +14,7 @@ import torch
 
 import oracle
 import paper_2301_10838_gb300 as mt
+from paper_2301_10838_gb300 import fields
 
 pytestmark = pytest.mark.gpu
 
@@ -64,3 +65,29 @@ def test_step_counts_past_the_end_of_the_list():
     part = torch.full((k // 2 + 9, 2), -1, dtype=torch.int32, device="cuda")
     assert mt.mt_build_step(f, W, 0.5, labels, part[:k // 2], ws, allow_partial=True) == (k, root)
     assert torch.equal(part[:k // 2], full[:k // 2]) and bool((part[k // 2:] == -1).all())
+
+
+@pytest.mark.slow
+def test_step_equals_the_calls_1024():
+    """The benchmark's step on its field: the one-call form, whose pairs are
+    marked in the repair pass, against the three calls (whose results the
+    full-size test compares with the oracle)."""
+    f = fields.named_field("lognorm1024", seed=1, device="cuda").contiguous()
+    n, g = f.numel(), mt.grid_of(f)
+    t = float(f.reshape(-1)[::4099].median())
+    ws = mt.workspace(g)
+    W, W2 = (torch.empty(n, dtype=torch.int64, device="cuda") for _ in range(2))
+    la, lb = (torch.empty(n, dtype=torch.int32, device="cuda") for _ in range(2))
+    a, b = (torch.full((n // 8, 2), -1, dtype=torch.int32, device="cuda") for _ in range(2))
+    mt.mt_build_triplets(f, W, ws)
+    mt.mt_components_at(f, W, t, la, ws)
+    for eps in (0.0, 0.5):
+        a.fill_(-1)
+        b.fill_(-1)
+        k, root = mt.mt_simplified_pairs(f, W, eps, 0, a, ws)
+        assert mt.mt_build_step(f, W2, t, lb, b, ws, eps=eps) == (k, root)
+        assert torch.equal(W, W2) and torch.equal(a, b)
+        if eps > 0:
+            mt.mt_simplified_components_at(f, W, t, eps, 0, la, ws)
+            mt.mt_sync_status(ws)
+        assert torch.equal(la, lb)
