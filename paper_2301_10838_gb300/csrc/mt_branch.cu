@@ -23,8 +23,10 @@
 //      sorted by value: a stable radix sort of (32-bit key, id), 8 bits per
 //      pass, passes whose digit is the same in every key skipped;
 //   4. the other large branches are compacted and sorted by value the same
-//      way, then stably by branch. On small grids the root's branch goes this
-//      way, too, since launches are what counts there.
+//      way, then stably by branch if there is more than one. On small grids the
+//      root's branch goes this way, too, since launches are what counts there
+//      (a constant field of 200^3, where it is the only one: 199 us, 317 with
+//      the sort by branch).
 // A radix pass is a digit histogram per block, an exclusive scan of the
 // histograms (digit major, block minor), and a scatter that ranks each block's
 // keys stably: a warp owns a contiguous run of the block's keys, finds the

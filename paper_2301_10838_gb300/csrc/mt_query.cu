@@ -307,10 +307,13 @@ static cudaError_t run_pairs(const Loc &loc, uint32_t nfields, uint64_t nchunks,
     k_scan_counts<Loc><<<nfields, 1024, 0, st>>>(loc, counts, npairs, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if constexpr (ONE) {
-        if (mask) k_pairs_write<Loc, false, true, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
-        else if (simp) k_pairs_write<Loc, true, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
+        if (mask)
+            k_pairs_write<Loc, false, true, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
+        else if (simp)
+            k_pairs_write<Loc, true, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
     }
-    if (!mask && !simp) k_pairs_write<Loc, false, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
+    if (!mask && !simp)
+        k_pairs_write<Loc, false, false, false><<<grid, kCompactThreads, 0, st>>>(loc, counts, mask, eps, status, out);
     count_launch(3);
     return cudaGetLastError();
 }
